@@ -244,7 +244,7 @@ def streaming_rows(kt, steps, n, m, A_out, hbm):
     return rows
 
 
-KERNEL_NAMES = ("tri_enum", "tri_hubs", "tri_reverse_list", "tri_eo_fresh_reserve", "tri_eo_list_reserve",
+KERNEL_NAMES = ("tri_enum", "tri_hubs", "tri_rest", "tri_alive", "tri_reverse_list", "tri_eo_fresh_reserve", "tri_eo_list_reserve",
                 "tri_eo_list_accept", "tri_eo_accept", "tri_eo_list_reset", "tri_classify", "compact_orient",
                 "compact_trmask", "row_maps")
 
@@ -362,14 +362,18 @@ def run_ours(args, rank, world):
     kt = {name: ctx.kernel_time(name) for name in KERNEL_NAMES}
 
     hbm, peak_src = peaks()
-    # one enumeration pass = the hub launch (vertices with long out-lists, when
-    # there are any) + the main launch; the pass is the roofline's unit
-    enum_ms = kt["tri_enum"][0] + kt["tri_hubs"][0]
+    # one enumeration = the hub launch (vertices with long out-lists, when there
+    # are any) + the main launch, and for a union kernel the compaction of the
+    # live arcs and the launches over them; it is the roofline's unit
+    enum_ms = kt["tri_enum"][0] + kt["tri_hubs"][0] + kt["tri_rest"][0] + kt["tri_alive"][0]
     passes = max(kt["tri_enum"][1], 1)
-    # the passes stream the shorter list of each arc (W probes in all); W+ is
-    # scaled by the share of W they streamed (later edge-once passes skip
-    # considered arcs)
-    fwd_total = work["forward_probes"] * pst["probes"] / max(work["probes"], 1)
+    # an enumeration answers for the W+ probes of the plain forward algorithm;
+    # of the W that streaming every arc's shorter list takes, a union kernel
+    # streams what its live edges need, and later edge-once passes skip
+    # considered arcs: those are charged W+ scaled by the share of W
+    fwd_total = work["forward_probes"] * passes
+    if args.kernel.startswith("tr_eo"):
+        fwd_total = work["forward_probes"] * pst["probes"] / max(work["probes"], 1)
     enum_bytes = enum_pass_bytes(n, m, fwd_total / passes)
     pass_s = enum_ms / passes / 1e3
     enum_achieved = enum_bytes / pass_s / 1e9 if pass_s > 0 else None
@@ -478,14 +482,14 @@ def run_ours(args, rank, world):
                    "max_out_degree": work["max_out_degree"], "kept_arcs": int(A_out),
                    "l2": "inputs larger than L2 (CSR %.0f MB > 129 MB)" % ((8 * (n + 1) + 8 * m) / 1e6),
                    "parallelism": "replicas" if world > 1 else "single GPU"},
-        "roofline": {"bound": "hbm", "kernel": "tri_enum pass (hub launch + main launch)",
+        "roofline": {"bound": "hbm", "kernel": "triangle enumeration (hub and main launches of its passes)",
                      "achieved": enum_achieved, "peak": hbm, "unit": "GB/s",
                      "frac": (enum_achieved / hbm) if enum_achieved else None,
                      "traffic": measured_traffic(args.workload, args.kernel),
                      "peak_source": peak_src, "algorithmic_bytes_per_launch": enum_bytes,
                      "launch_ms": enum_ms / passes, "launches": passes / psteps,
                      "byte_model": "8(n+1) + 4m + 4 W+ per enumeration pass",
-                     "launch_split_ms": {"tri_hubs": kt["tri_hubs"][0] / passes, "tri_enum": kt["tri_enum"][0] / passes},
+                     "launch_split_ms": {k: kt[k][0] / passes for k in ("tri_hubs", "tri_enum", "tri_alive", "tri_rest")},
                      "streamed": {"algorithmic_bytes_per_launch": streamed_bytes,
                                   "achieved": streamed_bytes / pass_s / 1e9 if pass_s > 0 else None,
                                   "frac": streamed_bytes / pass_s / 1e9 / hbm if pass_s > 0 else None,

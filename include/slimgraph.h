@@ -117,8 +117,9 @@ typedef struct sg_div_result {
 /* Launch accounting of a context (for benchmarks and profiles). */
 typedef struct sg_stats {
     uint64_t kernel_launches; /* kernels this library launched on the context */
-    uint64_t probes;          /* wedge-closing probes done by triangle kernels */
-    uint64_t triangles;       /* triangles found by triangle kernels */
+    uint64_t probes;          /* list elements streamed through tables by triangle kernels */
+    uint64_t triangles;       /* triangles found by triangle kernels (by union kernels: those
+                                 decided, since one whose edges are all deleted needs no decision) */
     uint64_t eo_rounds;       /* Edge-Once reservation rounds run */
     uint64_t eo_listed;       /* triangles written to Edge-Once lists (16 bytes each) */
     uint64_t eo_passes;       /* Edge-Once enumeration passes (each bids for its round) */

@@ -126,16 +126,26 @@ static sg_status compress_tr(Ctx *c, const Graph *g, sg_kernel k, double p, uint
     const bool maxw = (k == SG_TR_MAXW || k == SG_TR_EO_MAXW);
     RowMaps rm;
     Oriented o;
-    uint8_t *del = nullptr;
+    uint32_t *del = nullptr;
     sg_status st = build_row_maps(c, g, &rm);
     if (st == SG_OK) st = orient(c, g, rm, maxw, &o);
-    if (st == SG_OK) st = dalloc(c, (void **)&del, (size_t)std::max<int64_t>(o.m, 1));
+    if (st == SG_OK) st = dalloc(c, (void **)&del, sizeof(uint32_t) * del_words(o.m));
     if (st == SG_OK) {
-        cudaError_t e = cudaMemsetAsync(del, 0, (size_t)std::max<int64_t>(o.m, 1), c->stream);
+        cudaError_t e = cudaMemsetAsync(del, 0, sizeof(uint32_t) * del_words(o.m), c->stream);
         if (e != cudaSuccess) st = cuda_fail(e, "cudaMemsetAsync(del)");
     }
-    if (st == SG_OK) st = tr_mark(c, g, o, k, p, seed, del);
-    if (st == SG_OK) st = resolve_mask(c, g, rm, o, del, out);
+    // the union kernels' second pass works in the output's arrays; an edge-once
+    // kernel sizes its list by the memory free before they are allocated
+    const bool eo = k == SG_TR_EO || k == SG_TR_EO_MAXW || k == SG_TR_EO_MINCOUNT;
+    Graph *h = nullptr;
+    if (st == SG_OK && !eo) st = new_graph(c, g->n, g->nnz, g->w != nullptr, &h);
+    if (st == SG_OK) st = tr_mark(c, g, o, k, p, seed, del, h);
+    if (st == SG_OK) {
+        st = resolve_mask(c, g, rm, o, del, &h);
+        if (st == SG_OK) *out = h;
+    } else {
+        delete_graph(c, h);
+    }
     dfree(c, del);
     free_oriented(c, &o);
     free_row_maps(c, &rm);

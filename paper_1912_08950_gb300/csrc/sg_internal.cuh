@@ -209,9 +209,28 @@ struct Oriented {
 };
 sg_status orient(Ctx *c, const Graph *g, const RowMaps &rm, bool weights, Oriented *o);
 void free_oriented(Ctx *c, Oriented *o);
-// H = G minus the edges whose oriented arc has del[] != 0
-sg_status resolve_mask(Ctx *c, const Graph *g, const RowMaps &rm, const Oriented &o, const uint8_t *del,
+// H = G minus the edges whose oriented arc has its deletion flag set
+// (into *out, allocated here unless the caller did; freed on failure)
+sg_status resolve_mask(Ctx *c, const Graph *g, const RowMaps &rm, const Oriented &o, const uint32_t *del,
                        Graph **out);
+// a library-owned graph of n vertices with room for nnz_cap arcs
+sg_status new_graph(Ctx *c, int64_t n, int64_t nnz_cap, bool weighted, Graph **out);
+void delete_graph(Ctx *c, Graph *h);
+// words of the deletion flags of m oriented arcs, one bit each
+inline size_t del_words(int64_t m) { return (size_t)((m > 0 ? m : 1) + 31) / 32; }
+// The live arcs of E+ (deletion flag clear), in order: vertex x's are
+// list[off[x], off[x + 1]), each (head, arc index).  off and list borrow the
+// output graph's arrays, which are written only after the enumeration: off its
+// n + 1 offsets, list its columns (4 nnz bytes = 8 per edge).
+struct AliveArcs {
+    int64_t *off = nullptr;
+    uint2 *list = nullptr;
+    CompactScratch cs;
+};
+sg_status alive_alloc(Ctx *c, const Oriented &o, const Graph *out, AliveArcs *a);
+// rec[v] = (off+, d+, first live arc, live arcs) of every vertex
+sg_status alive_build(Ctx *c, const Oriented &o, const uint32_t *del, const AliveArcs &a, uint4 *rec);
+void alive_free(Ctx *c, AliveArcs *a);
 
 // batched variants over a disjoint union (sg_compact.cu)
 struct BatchDev {
@@ -221,8 +240,8 @@ struct BatchDev {
 sg_status batch_orient(Ctx *c, const Graph *u, const RowMaps &rm, const BatchDev &b, bool weights, Oriented *o,
                        unsigned long long *scan, int grid_per_sm);
 sg_status batch_final(Ctx *c, const Graph *u, const RowMaps &rm, const Oriented &o, const BatchDev &b,
-                      const uint8_t *del, uint32_t *delbits, int64_t *off_out, uint32_t *col_out, float *w_in,
-                      float *w_out, const CompactScratch &cs, int grid_per_sm);
+                      const uint32_t *del, int64_t *off_out, uint32_t *col_out, float *w_in, float *w_out,
+                      const CompactScratch &cs, int grid_per_sm);
 // the reverse list of o (see Oriented::inl) into inl; in a batch only the
 // graphs with a triangle kernel are listed
 sg_status reverse_list(Ctx *c, const Graph *g, const RowMaps &rm, const Oriented &o, uint2 *inl,
@@ -232,8 +251,10 @@ sg_status reverse_list(Ctx *c, const Graph *g, const RowMaps &rm, const Oriented
 sg_status low_degree(Ctx *c, const Graph *g, uint32_t *new_to_old, Graph **out);
 
 // triangles (sg_triangles.cu)
-sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double p, uint64_t seed,
-                  uint8_t *del);
+// sets the deletion flags of one TR kernel; h: the output graph, allocated but
+// not written yet (union kernels borrow its arrays), or NULL (edge-once)
+sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double p, uint64_t seed, uint32_t *del,
+                  const Graph *h);
 sg_status tr_count(Ctx *c, const Graph *g, const Oriented &o, int64_t *count, int64_t *probes, int64_t *maxdeg,
                    int64_t *in_arcs, int64_t *fwd_probes);
 // batched union TR, with no host synchronisation (capturable in a CUDA graph)
@@ -241,8 +262,8 @@ struct BatchTri {
     uint32_t *heavy = nullptr;
     unsigned long long *buckets = nullptr;  // counts, fills, total
     uint32_t *din = nullptr;                // in-arcs streamed from the head's side
+    uint2 *vrec = nullptr;                  // off+ and d+ of every vertex
     uint2 *inl = nullptr;
-    int log_slots = 3;
     size_t smem = 0;
     int max_deg = 1;      // largest out-degree (sizes the heavy vertex arrays)
     int light_max = 64;
@@ -250,7 +271,7 @@ struct BatchTri {
 };
 sg_status batch_tr_prepare(Ctx *c, const Graph *u, const Oriented &o, BatchTri *bt);
 sg_status batch_tr_mark(Ctx *c, const Graph *u, const Oriented &o, const BatchDev &b, const BatchTri &bt,
-                        uint8_t *del);
+                        uint32_t *del);
 void batch_tr_free(Ctx *c, BatchTri *bt);
 
 sg_status tr_vertex_counts(Ctx *c, const Graph *g, const Oriented &o, unsigned long long *vcnt);

@@ -24,8 +24,9 @@
 // Philox4x32-10 on the sorted original ids (a, b, c) selects the triangle
 // (r0 < floor(p 2^32)) and picks the edge to delete (r1, the heaviest edge, or
 // the edge in the fewest triangles of G, counted by an earlier EdgeCount pass);
-// the p-2 kernel deletes the two edges r1 does not pick.  Union kernels store
-// del[arc] = 1 (a plain, idempotent byte store).  The
+// the p-2 kernel deletes the two edges r1 does not pick.  Union kernels set the
+// arc's deletion flag (a bit, idempotent) and stop looking for triangles whose
+// edges are all deleted (tri_union_kernel).  The
 // Edge-Once kernel instead reserves each edge of every live selected triangle
 // with a 64-bit atomicMin of (r2 << 32 | third vertex); an edge pass then
 // accepts every triangle that holds all three of its reservations.  Accepted
@@ -50,16 +51,30 @@ constexpr int kHeavyCap = 1024;  // largest phase-1 table (entries; 26 KB of sha
 constexpr int kHubTW = 32;        // warps per CTA of the hub launch (one CTA per SM)
 constexpr int kHubCap = 4096;     // largest hub table (entries; 104 KB of shared memory)
 constexpr int kQ = 128;           // per-warp hit ring (<= 31 left over + 2 slabs of hits fit)
+constexpr int kWindow = 32;       // list elements a union pass streams before it looks at an arc again
+constexpr int kWhole = 1 << 29;        // blocks of the window of a list streamed whole
+constexpr int kFilterLog = 4;          // log2 of the filter bits per table slot (four slots per entry)
+constexpr int kFilterBits = 4 << kFilterLog;  // per entry
+constexpr int kUnionLightMax = 128;    // union passes: largest out-degree processed by one warp
+constexpr int kUnionLightItems = 512;  // ... with at most this many lists to stream
+// lists up to this long are always streamed whole (see tri_union_kernel): 256 on
+// graphs with a hub launch, where the second pass costs more (R-MAT s26 at p =
+// 0.5: both passes 528 ms against 551 at 128; s23 equal), 128 on the others
+// (s22: 19.2 ms against 22.3 at 256; 64 leaves a third more arc ends to pass 2)
+constexpr int kShortList = 128, kShortListHubs = 256;
 constexpr int kEoBuckets = 6;     // edge-once list buckets (rounds 0..5 of the prefix schedule)
 // context workspaces of the edge-once rounds: the list and the two active lists
 constexpr int kWsList = 0, kWsActive0 = 1, kWsActive1 = 2;
 
-// Count: totals only.  EdgeCount / VertexCount: add every triangle to the
+// Count: totals only (tri_enum_kernel; Union* and BatchUnion run in tri_union_kernel).  EdgeCount / VertexCount: add every triangle to the
 // counters of its three edges / vertices.  Union*: the union-semantics TR kernels.  EoReserve: one
 // edge-once bidding pass.  EoEmit: lists the live selected triangles for the
 // edge-once list rounds.  BatchUnion: union kernels over a batch of graphs.
 enum class Mode { Count, EdgeCount, VertexCount, UnionRandom, UnionMaxw, UnionP2, UnionMinCount, EoReserve, EoEmit,
                   BatchUnion };
+template <Mode M>
+constexpr bool kUnion = M == Mode::UnionRandom || M == Mode::UnionMaxw || M == Mode::UnionP2 ||
+                        M == Mode::UnionMinCount || M == Mode::BatchUnion;
 // the edge-once passes skip arcs that are already considered
 template <Mode M>
 constexpr bool kEdgeOnce = M == Mode::EoReserve || M == Mode::EoEmit;
@@ -71,6 +86,15 @@ __device__ __forceinline__ bool considered_bit(const uint32_t *c, int64_t e) {
 }
 __device__ __forceinline__ void set_considered(uint32_t *c, int64_t e) { atomicOr(c + (e >> 5), 1u << (e & 31)); }
 
+// Deletion flags: one bit per oriented arc.  They only ever change from 0 to 1
+// during a pass, so a stale read is a flag not seen yet.
+__device__ __forceinline__ void delete_arc(uint32_t *del, uint32_t e) { atomicOr(del + (e >> 5), 1u << (e & 31)); }
+__device__ __forceinline__ bool arc_deleted(const uint32_t *del, uint32_t e) {
+    uint32_t w;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(del + (e >> 5)) : "memory");
+    return (w >> (e & 31)) & 1u;
+}
+
 struct TriArgs {
     const int64_t *offp;
     const uint32_t *colp;
@@ -81,7 +105,8 @@ struct TriArgs {
     int64_t n;
     uint32_t k0, k1;
     unsigned long long tp;
-    uint8_t *del;
+    uint32_t *del;                // deletion flags, one bit per oriented arc
+    uint32_t dead_flag;           // union passes: a bit no arc index uses (kArcDead), or 0
     const uint32_t *considered;  // edge-once flag bits (see considered_bit)
     unsigned long long *resv;
     uint32_t *tcnt;               // triangles of G through each arc of E+ (EdgeCount adds, min-count reads)
@@ -90,9 +115,13 @@ struct TriArgs {
     unsigned long long *ctr;
     const uint32_t *heavy;
     int64_t n_heavy;
-    int heavy_log_slots;
     int heavy_cap;               // entries of the phase-1 table; larger N+(u) go in chunks
     int light_max;               // out-degrees up to this go to the warp-per-vertex phase
+    int short_max;               // union passes: lists up to this long are always streamed whole
+    const uint2 *vrec;           // off+ and d+ of vertex v at entry v * vstep
+    int vstep;                   // 1, or 2: the first halves of the records arec
+    const uint4 *arec;           // off+, d+, first live arc, live arcs (second union pass: alive_build)
+    const uint2 *alive;
     int light_items;             // ... when they also have at most this many arcs to stream
     int *err;                    // device error word (a cuckoo stash overflow)
     unsigned long long *work;    // [0] next heavy vertex, [1] next light vertex block
@@ -204,12 +233,6 @@ __device__ __forceinline__ uint32_t slot_of(uint32_t key, int log_slots) {
 }
 
 __device__ __forceinline__ int ceil_log2(int x) { return x <= 1 ? 0 : 32 - __clz(x - 1); }
-static int ceil_log2_host(int x) {
-    int l = 0;
-    while ((1 << l) < x) ++l;
-    return l;
-}
-
 template <typename T>
 __device__ __forceinline__ void swap2(T &a, T &b) {
     const T t = a;
@@ -230,111 +253,63 @@ __device__ __forceinline__ I mincount_arc(const uint32_t *tcnt, I e01, I e02, I 
     return best;
 }
 
-// One triangle (u, v, w) with its three oriented arcs: selection and action.
-// Warp-collective (the edge-once list writer uses ballots); lanes without a
-// triangle pass valid = false.
+// sort the vertices of a triangle, keeping e_ij = the arc joining x_i and x_j
+__device__ __forceinline__ void sort_triangle(uint32_t &x0, uint32_t &x1, uint32_t &x2, uint32_t &e01, uint32_t &e02,
+                                              uint32_t &e12) {
+    if (x0 > x1) { swap2(x0, x1); swap2(e02, e12); }
+    if (x1 > x2) { swap2(x1, x2); swap2(e01, e02); }
+    if (x0 > x1) { swap2(x0, x1); swap2(e02, e12); }
+}
+
+// the heaviest of a sorted triangle's edges under (weight, lo, hi)
+__device__ __forceinline__ uint32_t maxw_arc(const float *wp, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t e01,
+                                             uint32_t e02, uint32_t e12) {
+    const float w01 = __ldg(wp + e01), w02 = __ldg(wp + e02), w12 = __ldg(wp + e12);
+    uint32_t best = e01;
+    float bw = w01;
+    uint32_t bl = x0, bh = x1;
+    if (w02 > bw || (w02 == bw && (x0 > bl || (x0 == bl && x2 > bh)))) { best = e02; bw = w02; bl = x0; bh = x2; }
+    if (w12 > bw || (w12 == bw && (x1 > bl || (x1 == bl && x2 > bh)))) { best = e12; }
+    return best;
+}
+
+// One triangle (u, v, w) with its three oriented arcs under an edge-once pass:
+// selection and bid or listing.  Warp-collective (the list writer uses
+// ballots); lanes without a triangle pass valid = false.
 template <Mode M>
 __device__ __forceinline__ void decide(const TriArgs &a, bool valid, uint32_t u, uint32_t v, uint32_t w,
                                        uint32_t iuv, uint32_t iuw, uint32_t ivw, unsigned &live, Emitter &em,
                                        uint32_t head_uv = 0) {
-    if constexpr (M == Mode::Count || M == Mode::EdgeCount || M == Mode::VertexCount) {
+    if constexpr (!kEdgeOnce<M>) {
         return;
     } else {
         bool emit = false;
         uint4 rec = make_uint4(0u, 0u, 0u, 0u);
         uint32_t rec_r2 = 0;
-        if constexpr (M == Mode::BatchUnion) {
-            if (valid) {
-                // the triangle's graph: its own seed, p and kernel, local ids as keys
-                const BatchParam &P = a.bparams[__ldg(a.vgid + u)];
-                const uint32_t base = (uint32_t)P.vbase;
-                uint32_t x0 = u - base, x1 = v - base, x2 = w - base;
-                uint32_t e01 = iuv, e02 = iuw, e12 = ivw;
-                if (x0 > x1) { swap2(x0, x1); swap2(e02, e12); }
-                if (x1 > x2) { swap2(x1, x2); swap2(e01, e02); }
-                if (x0 > x1) { swap2(x0, x1); swap2(e02, e12); }
-                const uint4 r = philox4x32_10(make_uint4(x0, x1, x2, kTagTri), P.k0, P.k1);
-                if ((unsigned long long)r.x < P.tp) {
-                    uint32_t best;
-                    if (P.kernel == (int)SG_TR_MAXW) {
-                        const float w01 = __ldg(a.wp + e01), w02 = __ldg(a.wp + e02), w12 = __ldg(a.wp + e12);
-                        best = e01;
-                        float bw = w01;
-                        uint32_t bl = x0, bh = x1;
-                        if (w02 > bw || (w02 == bw && (x0 > bl || (x0 == bl && x2 > bh)))) { best = e02; bw = w02; bl = x0; bh = x2; }
-                        if (w12 > bw || (w12 == bw && (x1 > bl || (x1 == bl && x2 > bh)))) { best = e12; }
-                    } else {
-                        const int k = (int)(((unsigned long long)r.y * 3ull) >> 32);
-                        best = k == 0 ? e01 : (k == 1 ? e02 : e12);
-                        if (P.kernel == (int)SG_TR_P2) {  // the drawn edge is the one kept
-                            if (k != 0) a.del[e01] = 1;
-                            if (k != 1) a.del[e02] = 1;
-                            if (k != 2) a.del[e12] = 1;
-                            return;
-                        }
-                    }
-                    a.del[best] = 1;
-                }
-            }
-            return;
-        }
         if (valid) {
-            // sort the vertices, keeping e_ij = the arc joining x_i and x_j
             uint32_t x0 = u, x1 = v, x2 = w;
             uint32_t e01 = iuv, e02 = iuw, e12 = ivw;
-            if (x0 > x1) { swap2(x0, x1); swap2(e02, e12); }
-            if (x1 > x2) { swap2(x1, x2); swap2(e01, e02); }
-            if (x0 > x1) { swap2(x0, x1); swap2(e02, e12); }
+            sort_triangle(x0, x1, x2, e01, e02, e12);
             const uint4 r = philox4x32_10(make_uint4(x0, x1, x2, kTagTri), a.k0, a.k1);
-            if ((unsigned long long)r.x < a.tp) {  // the triangle is selected
-                if constexpr (M == Mode::UnionRandom) {
-                    const int k = (int)(((unsigned long long)r.y * 3ull) >> 32);
-                    a.del[k == 0 ? e01 : (k == 1 ? e02 : e12)] = 1;
-                } else if constexpr (M == Mode::UnionP2) {
-                    // x = 2: the drawn edge stays, the other two go
-                    const int k = (int)(((unsigned long long)r.y * 3ull) >> 32);
-                    if (k != 0) a.del[e01] = 1;
-                    if (k != 1) a.del[e02] = 1;
-                    if (k != 2) a.del[e12] = 1;
-                } else if constexpr (M == Mode::UnionMinCount) {
-                    a.del[mincount_arc(a.tcnt, e01, e02, e12)] = 1;
-                } else if constexpr (M == Mode::UnionMaxw) {
-                    // heaviest edge under (weight, lo, hi)
-                    const float w01 = __ldg(a.wp + e01), w02 = __ldg(a.wp + e02), w12 = __ldg(a.wp + e12);
-                    uint32_t best = e01;
-                    float bw = w01;
-                    uint32_t bl = x0, bh = x1;
-                    if (w02 > bw || (w02 == bw && (x0 > bl || (x0 == bl && x2 > bh)))) { best = e02; bw = w02; bl = x0; bh = x2; }
-                    if (w12 > bw || (w12 == bw && (x1 > bl || (x1 == bl && x2 > bh)))) { best = e12; }
-                    a.del[best] = 1;
-                } else if constexpr (M == Mode::EoReserve) {
-                    if (a.considered == nullptr || !(considered_bit(a.considered, e01) | considered_bit(a.considered, e02) |
-                                                     considered_bit(a.considered, e12))) {
-                        // the round's prefix of the (r2, a, b, c) order bids for its edges
-                        if ((unsigned long long)r.z < a.eo_theta) {
-                            const unsigned long long hi = (unsigned long long)r.z << 32;
-                            atomicMin(a.resv + e01, hi | x2);
-                            atomicMin(a.resv + e02, hi | x1);
-                            atomicMin(a.resv + e12, hi | x0);
-                        }
-                        ++live;
-                    }
-                } else {  // EoEmit: list the live selected triangle (and bid, in case the list overflows)
-                    if (a.considered == nullptr || !(considered_bit(a.considered, e01) | considered_bit(a.considered, e02) |
-                                                     considered_bit(a.considered, e12))) {
-                        if ((unsigned long long)r.z < a.eo_theta) {
-                            const unsigned long long hi = (unsigned long long)r.z << 32;
-                            atomicMin(a.resv + e01, hi | x2);
-                            atomicMin(a.resv + e02, hi | x1);
-                            atomicMin(a.resv + e12, hi | x0);
-                        }
-                        ++live;
-                        emit = true;
-                        rec_r2 = r.z;
-                        // w is last in the degree order; of u and v the head of iuv is the later one
-                        const bool u_first = head_uv == v;
-                        rec = make_uint4(u_first ? u : v, iuv, u_first ? iuw : ivw, u_first ? ivw : iuw);
-                    }
+            // the triangle is selected, and none of its edges is considered
+            if ((unsigned long long)r.x < a.tp &&
+                (a.considered == nullptr || !(considered_bit(a.considered, e01) | considered_bit(a.considered, e02) |
+                                              considered_bit(a.considered, e12)))) {
+                // the round's prefix of the (r2, a, b, c) order bids for its edges
+                // (the listing pass too, in case the list overflows)
+                if ((unsigned long long)r.z < a.eo_theta) {
+                    const unsigned long long hi = (unsigned long long)r.z << 32;
+                    atomicMin(a.resv + e01, hi | x2);
+                    atomicMin(a.resv + e02, hi | x1);
+                    atomicMin(a.resv + e12, hi | x0);
+                }
+                ++live;
+                if constexpr (M == Mode::EoEmit) {  // list the live selected triangle
+                    emit = true;
+                    rec_r2 = r.z;
+                    // w is last in the degree order; of u and v the head of iuv is the later one
+                    const bool u_first = head_uv == v;
+                    rec = make_uint4(u_first ? u : v, iuv, u_first ? iuw : ivw, u_first ? ivw : iuw);
                 }
             }
         }
@@ -344,7 +319,7 @@ __device__ __forceinline__ void decide(const TriArgs &a, bool valid, uint32_t u,
 
 // Decide the 32 oldest queued triangles with all lanes.
 template <Mode M>
-__device__ __forceinline__ void drain32_body(const TriArgs &a, const HitQueue &q, int head, uint32_t u,
+__device__ __forceinline__ void drain32(const TriArgs &a, const HitQueue &q, int head, uint32_t u,
                                              unsigned &live, Emitter &em) {
     const int k = (head + (threadIdx.x & 31)) & (kQ - 1);
     const uint32_t iuw = q.iuw[k];
@@ -354,25 +329,11 @@ __device__ __forceinline__ void drain32_body(const TriArgs &a, const HitQueue &q
     decide<M>(a, true, u, q.v[k], __ldg(a.colp + iuw), iuv, iuw, q.ivw[k], live, em, huv);
     __syncwarp();
 }
-template <Mode M>
-__device__ __noinline__ void drain32_call(const TriArgs &a, const HitQueue &q, int head, uint32_t u, unsigned &live,
-                                          Emitter &em) {
-    drain32_body<M>(a, q, head, u, live, em);
-}
-// Out of line, so that the probe loop's register budget stays small -- except
-// for the listing pass, whose 64-register budget holds it inline without the
-// spills a call costs there (R-MAT s22: 80 -> 72 ms).
-template <Mode M>
-__device__ __forceinline__ void drain32(const TriArgs &a, const HitQueue &q, int head, uint32_t u, unsigned &live,
-                                        Emitter &em) {
-    drain32_body<M>(a, q, head, u, live, em);
-}
-
 // Decide everything queued for the table vertex u (the last group with idle lanes).
 template <Mode M>
 __device__ __forceinline__ void flush_hits(const TriArgs &a, const HitQueue &q, QState &qs, uint32_t u,
                                            unsigned &live, Emitter &em) {
-    if constexpr (M != Mode::Count && M != Mode::EdgeCount && M != Mode::VertexCount) {
+    if constexpr (kEdgeOnce<M>) {
         const int lane = threadIdx.x & 31;
         while (qs.n >= 32) {
             drain32<M>(a, q, qs.head, u, live, em);
@@ -426,6 +387,8 @@ struct Table {
     uint32_t *slot;
     unsigned long long *stash;
     int *stash_n;
+    uint32_t *dead = nullptr;    // union passes: deletion flags of the table's arcs, by position,
+    uint32_t *filter = nullptr;  // and one bit per hash of kFilterBits per entry
 };
 
 __device__ __forceinline__ void table_insert(const Table &t, int log_slots, uint32_t w, int i, int *err) {
@@ -643,7 +606,7 @@ __device__ __forceinline__ void finish(const TriArgs &a, unsigned live, unsigned
 // CTA of 32 warps per SM shares a table of up to kHubCap entries, so those
 // lists are streamed once instead of once per table chunk.
 template <Mode M>
-constexpr int kEnumCtasPerSm = (M == Mode::Count || M == Mode::EdgeCount || M == Mode::VertexCount) ? 5 : 4;
+constexpr int kEnumCtasPerSm = kEdgeOnce<M> ? 4 : 5;
 
 template <Mode M, int TW>
 __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tri_enum_kernel(TriArgs a) {
@@ -838,6 +801,540 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tr
     finish<M>(a, live, probes, tris, em);
 }
 
+// ------------------------------------------------------------ union passes
+// The union kernels delete, for every selected triangle, the edge (or edges)
+// its draw names, and deletions accumulate.  So a triangle whose three edges
+// are already deleted need not be decided, and an arc whose edge is already
+// deleted need not be streamed for triangles whose other two edges are deleted
+// too.  Most edges die early: on R-MAT s22 at p = 0.5 an edge lies in 99
+// triangles on average and each deletes it with probability 1/6.  Two passes
+// use that and give the same flags as deciding every triangle:
+//
+//   first pass (kAlive = false)   every arc u->v streams the shorter list
+//     through the table of the longer one as the counting passes do, but only
+//     until its own edge is deleted: windows of 1, 2, 4, ... blocks of kWindow
+//     elements, from a start spread over the list, between which the edge's
+//     flag is looked at.  A list of at most short_max elements (kShortList) is
+//     always streamed whole.  At the end a live arc has been streamed whole; a
+//     long list not streamed whole belongs to a deleted arc.
+//   second pass (kAlive = true)   for the deleted arcs u->v with two lists
+//     longer than short_max, the triangles {u, v, w} that still matter have
+//     u->w or v->w live after the first pass: the live arcs of v (compacted by
+//     alive_build) stream through the table of N+(u) and the live arcs of u
+//     through that of N+(v); where those together are no shorter than the
+//     shorter list, that list streams whole instead.
+//
+// Bound by instruction issue (69% of the slots at s23, the integer pipe at
+// 47%, DRAM at 19%): about half of the instructions are the list elements
+// (mapping, filter, queue), a fifth the claims and windows, a fifth the
+// decisions.  R-MAT at p = 0.5, elements streamed and triangles decided against
+// all of them, and the enumeration's time before (one pass that decides every
+// triangle) and now: s22 0.35 and 0.14, 41.8 -> 19.2 ms; s26 0.32 and 0.09,
+// 1094 -> 528 ms.  Max-weight on a Chung-Lu graph of 2^21 vertices at p = 1,
+// where light edges never die: 0.69 and 0.35, 11.5 -> 8.3 ms.
+template <Mode M>
+__device__ __forceinline__ void kill_arc(const TriArgs &a, const Table &tb, uint32_t tbase, uint32_t cn, uint32_t e) {
+    delete_arc(a.del, e);
+    const uint32_t r = e - tbase;  // an arc of the table: its flag in shared memory too
+    if (r < cn) atomicOr(tb.dead + (r >> 5), 1u << (r & 31));
+}
+
+// One triangle (u, v, w) with its three oriented arcs: selection and deletion.
+template <Mode M>
+__device__ __forceinline__ void decide_union(const TriArgs &a, const Table &tb, uint32_t tbase, uint32_t cn,
+                                             uint32_t u, uint32_t v, uint32_t w, uint32_t iuv, uint32_t iuw,
+                                             uint32_t ivw) {
+    uint32_t x0 = u, x1 = v, x2 = w, e01 = iuv, e02 = iuw, e12 = ivw;
+    uint32_t k0 = a.k0, k1 = a.k1;
+    unsigned long long tp = a.tp;
+    bool maxw = M == Mode::UnionMaxw, p2 = M == Mode::UnionP2;
+    if constexpr (M == Mode::BatchUnion) {
+        // the triangle's graph: its own seed, p and kernel, local ids as keys
+        const BatchParam &P = a.bparams[__ldg(a.vgid + u)];
+        const uint32_t base = (uint32_t)P.vbase;
+        x0 -= base;
+        x1 -= base;
+        x2 -= base;
+        k0 = P.k0;
+        k1 = P.k1;
+        tp = P.tp;
+        maxw = P.kernel == (int)SG_TR_MAXW;
+        p2 = P.kernel == (int)SG_TR_P2;
+    }
+    sort_triangle(x0, x1, x2, e01, e02, e12);
+    const uint4 r = philox4x32_10(make_uint4(x0, x1, x2, kTagTri), k0, k1);
+    if ((unsigned long long)r.x >= tp) return;  // not selected
+    uint32_t best;
+    if constexpr (M == Mode::UnionMinCount) {
+        best = mincount_arc(a.tcnt, e01, e02, e12);
+    } else if (maxw) {
+        best = maxw_arc(a.wp, x0, x1, x2, e01, e02, e12);
+    } else {
+        const int k = (int)(((unsigned long long)r.y * 3ull) >> 32);
+        if (p2) {  // x = 2: the drawn edge stays, the other two go
+            if (k != 0) kill_arc<M>(a, tb, tbase, cn, e01);
+            if (k != 1) kill_arc<M>(a, tb, tbase, cn, e02);
+            if (k != 2) kill_arc<M>(a, tb, tbase, cn, e12);
+            return;
+        }
+        best = k == 0 ? e01 : (k == 1 ? e02 : e12);
+    }
+    kill_arc<M>(a, tb, tbase, cn, best);
+}
+
+// The table vertex a warp works on.
+struct TabCtx {
+    Table tb;
+    int sh;                 // 32 - log2(slots)
+    int fsh;                // 32 - log2(filter bits)
+    int stash_n;
+    uint32_t u, tbase, cn;  // vertex, arc of table position 0, entries
+    int d;                  // d+(u)
+};
+
+// A warp's scratch: the ring of list elements that may close a triangle --
+// (v, arc u-v, w, arc v->w), one 16-byte store and load each -- the arcs whose
+// lists it is streaming, (v, arc u-v, list start minus the elements before it,
+// flags), and the arcs waiting for a free lane, (v, arc u-v, list start, length
+// and flags).
+constexpr int kPool = 64;
+struct UnionScratch {
+    uint4 ring[kQ];
+    uint4 arc[32];
+    uint4 pool[kPool];
+};
+// flags, beside the length in the pool: the arc's list is the live arcs of v;
+// the arc was deleted before its list streamed (kept in the ring entry's arc
+// v->w, when arc indices leave the bit free: TriArgs::dead_flag)
+constexpr uint32_t kArcLive = 1u << 30, kArcDead = 1u << 31;
+constexpr int kLenMask = (1 << 30) - 1;
+
+// The table's filter: 2^L * kFilterBits / 4 bits, w's at the high bits of w *
+// kH1.  Most list elements are in no triangle (R-MAT: 85-90%), and one
+// shared-memory word and a bit test drop nearly all of them where the two
+// cuckoo lookups take twice the instructions; what passes (the hits and about
+// 1 / kFilterBits of the others) is looked up 32 at a time when it is decided.
+__device__ __forceinline__ uint32_t filter_bit(const TabCtx &t, uint32_t w) { return (w * kH1) >> t.fsh; }
+__device__ __forceinline__ bool filter_pass(const TabCtx &t, uint32_t w) {
+    const uint32_t f = filter_bit(t, w);
+    return (t.tb.filter[f >> 5] >> (f & 31)) & 1u;
+}
+
+// Look the oldest `cnt` (<= 32) queued elements up and decide the triangles
+// they close that still have a live edge.
+template <Mode M>
+__device__ __forceinline__ void drain_union(const TriArgs &a, const TabCtx &t, const UnionScratch &q, int head, int cnt,
+                                            unsigned long long &tris) {
+    const int lane = threadIdx.x & 31;
+    bool hit = false;
+    if (lane < cnt) {
+        const uint4 h = q.ring[(head + lane) & (kQ - 1)];  // v, arc u-v, w, arc v->w
+        uint32_t k = 0;
+        hit = table_find(t.tb, t.sh, h.z, k);
+        if (t.stash_n != 0 && !hit) {  // rare
+            const unsigned long long c = stash_find(t.tb.stash, t.stash_n, h.z);
+            hit = c != kStashNone;
+            k = (uint32_t)c;
+        }
+        // on an arc that was deleted before its list streamed, a triangle
+        // matters while one of its other edges lives
+        const uint32_t vw = h.w & ~a.dead_flag;
+        if (hit && (h.w & a.dead_flag) && ((t.tb.dead[k >> 5] >> (k & 31)) & 1u)) hit = !arc_deleted(a.del, vw);
+        if (hit) decide_union<M>(a, t.tb, t.tbase, t.cn, t.u, h.x, h.z, h.y, t.tbase + k, vw);
+    }
+    const unsigned m = __ballot_sync(kFull, hit);
+    if (lane == 0) tris += (unsigned)__popc(m);
+}
+
+template <Mode M>
+__device__ __forceinline__ void flush_union(const TriArgs &a, const TabCtx &t, const UnionScratch &q, QState &qs,
+                                            unsigned long long &tris) {
+    while (qs.n > 0) {
+        drain_union<M>(a, t, q, qs.head, min(qs.n, 32), tris);
+        qs.head = (qs.head + 32) & (kQ - 1);
+        qs.n -= 32;
+    }
+    qs.head = 0;
+    qs.n = 0;
+}
+
+// A list element: w (kEmpty: none), the arc v->w and the entry of v's arc in
+// the scratch.
+struct Elem {
+    uint32_t w, arc;
+    int k;
+};
+
+// Filter two list elements per lane, queue what passes, and decide what a full
+// group has gathered.
+template <Mode M>
+__device__ __forceinline__ void probe_union(const TriArgs &a, const TabCtx &t, const Elem &x, const Elem &y,
+                                            UnionScratch &q, QState &qs, unsigned long long &tris) {
+    const bool hx = x.w != kEmpty && filter_pass(t, x.w);
+    const bool hy = y.w != kEmpty && filter_pass(t, y.w);
+    const unsigned mx = __ballot_sync(kFull, hx), my = __ballot_sync(kFull, hy);
+    if (mx | my) {
+        const uint32_t lt = lanemask_lt();
+        const int px = __popc(mx);
+        const int tail = qs.head + qs.n;
+        if (hx) {
+            const uint4 e = q.arc[x.k];
+            q.ring[(tail + __popc(mx & lt)) & (kQ - 1)] = make_uint4(e.x, e.y, x.w, x.arc | (e.w & a.dead_flag));
+        }
+        if (hy) {
+            const uint4 e = q.arc[y.k];
+            q.ring[(tail + px + __popc(my & lt)) & (kQ - 1)] = make_uint4(e.x, e.y, y.w, y.arc | (e.w & a.dead_flag));
+        }
+        qs.n += px + __popc(my);
+        __syncwarp();
+        while (qs.n >= 32) {
+            drain_union<M>(a, t, q, qs.head, 32, tris);
+            qs.head = (qs.head + 32) & (kQ - 1);
+            qs.n -= 32;
+        }
+    }
+}
+
+// Stream the wanted lists of the lanes' arcs (lane: sl elements from sp; none
+// if 0) as one sequence of elements, 64 at a time: the lists are short (a
+// window of 32, about ten live arcs), and a list at a time would leave most
+// lanes idle.  A lane finds its element's arc from the arcs that start inside
+// its slab of 32 (an OR over the lanes).
+template <Mode M, bool kAlive>
+__device__ __forceinline__ void stream_lists(const TriArgs &a, const TabCtx &t, uint32_t sv, uint32_t se, uint32_t sp,
+                                             int sl, uint32_t flags, UnionScratch &q, QState &qs,
+                                             unsigned long long &probes, unsigned long long &tris, bool count) {
+    const int lane = threadIdx.x & 31;
+    // number the elements consecutively
+    int inc = sl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += x;
+    }
+    const int total = __shfl_sync(kFull, inc, 31);
+    const int start = sl > 0 ? inc - sl : INT_MIN;
+    const unsigned wanted = __ballot_sync(kFull, sl > 0);
+    if (sl > 0) q.arc[__popc(wanted & lanemask_lt())] = make_uint4(sv, se, sp - (uint32_t)start, flags);
+    __syncwarp();
+    const uint32_t le = lanemask_lt() | (1u << lane);
+    int before = -1;  // arcs that start before the slab, minus one
+    auto element = [&](int s) {
+        Elem x{kEmpty, 0u, 0};
+        const unsigned rel = (unsigned)start - (unsigned)s;
+        const unsigned starts = __reduce_or_sync(kFull, rel < 32u ? 1u << rel : 0u);
+        x.k = before + __popc(starts & le);
+        before += __popc(starts);
+        if (s + lane < total) {
+            const uint4 r = q.arc[x.k];
+            x.arc = r.z + (uint32_t)(s + lane);
+            if (kAlive && (r.w & kArcLive)) {
+                const uint2 l = __ldg(a.alive + x.arc);
+                x.w = l.x;
+                x.arc = l.y;
+            } else {
+                x.w = __ldg(a.colp + x.arc);
+            }
+        }
+        return x;
+    };
+    if (count) probes += (unsigned)sl;
+    Elem nx = element(0), ny = element(32);
+    for (int s = 64;; s += 64) {
+        const Elem x = nx, y = ny;
+        if (s < total) {
+            nx = element(s);
+            ny = element(s + 32);
+        }
+        probe_union<M>(a, t, x, y, q, qs, tris);
+        if (s >= total) break;
+    }
+    __syncwarp();  // the scratch's arcs are read before they are written again
+}
+
+// Stream the lists of the table vertex's arcs: item i < nin is entry ib + i of
+// the in-lists, item nin + i the out-arc ou + i.  The warp claims 32 items at
+// a time (from the CTA's counter `next`, or its own); the lanes load their
+// records, flags and list bounds, and the arcs that this pass wants from this
+// end (fewer than half of them) wait in the pool until a lane is free.  A lane
+// holds one arc: in the first pass a live arc with a long list streams windows
+// of 1, 2, 4, ... blocks of kWindow until its edge is deleted (a kill takes
+// about 40 elements on R-MAT graphs) and its lane takes the next arc.  The
+// records of one claim load while the windows stream, the ids of the next with
+// them.
+template <Mode M, bool kAlive>
+__device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, int *next, uint32_t ou, int64_t ib, int nin,
+                                            int ax, UnionScratch &q, QState &qs, unsigned long long &probes,
+                                            unsigned long long &tris, bool count) {
+    const int lane = threadIdx.x & 31;
+    const int items = nin + t.d;
+    auto claim = [&]() {
+        int i = 0;
+        if (lane == 0) i = atomicAdd(next, 32);
+        return __shfl_sync(kFull, i, 0);
+    };
+    auto load_ids = [&](int c, uint32_t &v, uint32_t &e) {
+        const int i = c + lane;
+        if (i < nin) {
+            const uint2 it = __ldg(a.inl + ib + i);
+            v = it.x;
+            e = it.y;
+        } else if (i < items) {
+            e = ou + (uint32_t)(i - nin);
+            v = __ldg(a.colp + e);
+        }
+    };
+    int c = claim();  // the claim whose ids are loaded
+    uint32_t rv = 0, re = 0;
+    load_ids(c, rv, re);
+    int phead = 0, pn = 0;            // the pool
+    uint32_t sv = 0, se = 0, lst = 0; // the lane's arc: other end, arc, list start,
+    int len = 0, b = 0, left = 0;     // list length, next block, blocks not streamed yet
+    int w = 0;                        // blocks of the next window
+    for (;;) {
+        // records of the claimed items, ids of the next claim
+        const int gc = pn <= kPool - 32 ? c : items;  // the pool has room for a whole claim
+        const bool got = gc + lane < items;
+        bool dead = false;
+        uint4 rec = make_uint4(0u, 0u, 0u, 0u);  // off+, d+, first live arc, live arcs
+        const uint32_t gv = rv, ge = re;
+        if (got) {
+            dead = arc_deleted(a.del, ge);
+            if constexpr (kAlive) {
+                rec = __ldg(a.arec + gv);
+            } else {
+                const uint2 r = __ldg(a.vrec + (size_t)gv * a.vstep);
+                rec.x = r.x;
+                rec.y = r.y;
+            }
+        }
+        if (gc < items) {
+            c = claim();
+            load_ids(c, rv, re);
+        }
+        // the windows of the lanes' arcs
+        if (__any_sync(kFull, left > 0)) {
+            const int n = len & kLenMask;
+            const int nb = (n + kWindow - 1) / kWindow;
+            const int k = min(min(w, left), nb - b);  // up to the list's end, where it wraps
+            const int sl = left > 0 ? min(k * kWindow, n - b * kWindow) : 0;
+            stream_lists<M, kAlive>(a, t, sv, se, lst + (uint32_t)(b * kWindow), sl, (uint32_t)len, q, qs,
+                                    probes, tris, count);
+            if (left > 0) {
+                left -= k;
+                b = b + k == nb ? 0 : b + k;
+                w *= 2;
+            }
+            if constexpr (!kAlive) {
+                if (__any_sync(kFull, left > 0)) {
+                    if (c >= items && pn == 0) flush_union<M>(a, t, q, qs, tris);  // nothing else to stream meanwhile
+                    if (left > 0 && arc_deleted(a.del, se)) left = 0;
+                }
+            }
+        }
+        // the claimed arcs to stream from this end: the longer list's
+        if (gc < items) {
+            uint32_t sp = rec.x;
+            int sl = 0;
+            if (got) {
+                const int dv = (int)rec.y;
+                const bool own = gc + lane >= nin ? dv <= t.d : dv < t.d;
+                if constexpr (!kAlive) {
+                    if (own && (!dead || dv <= a.short_max)) sl = dead && dv > 0 ? (int)((uint32_t)dv | kArcDead) : dv;
+                } else if (dead && min(dv, t.d) > a.short_max) {
+                    if ((int)rec.w + ax >= min(dv, t.d)) {
+                        if (own) sl = (int)((uint32_t)dv | kArcDead);
+                    } else if (rec.w != 0) {
+                        sp = rec.z;
+                        sl = (int)(rec.w | kArcLive | kArcDead);
+                    }
+                }
+            }
+            const unsigned m = __ballot_sync(kFull, sl != 0);
+            if (sl != 0) q.pool[(phead + pn + __popc(m & lanemask_lt())) & (kPool - 1)] = make_uint4(gv, ge, sp, (uint32_t)sl);
+            pn += __popc(m);
+        }
+        __syncwarp();
+        // free lanes take waiting arcs
+        const unsigned idle = __ballot_sync(kFull, left == 0);
+        const int take = min(pn, __popc(idle));
+        const int rank = __popc(idle & lanemask_lt());
+        if (left == 0 && rank < take) {
+            const uint4 r = q.pool[(phead + rank) & (kPool - 1)];
+            sv = r.x;
+            se = r.y;
+            lst = r.z;
+            len = (int)r.w;
+            const int n1 = len & kLenMask;
+            left = (n1 + kWindow - 1) / kWindow;
+            b = 0;
+            w = kWhole;
+            if (!kAlive && n1 > a.short_max) {
+                b = (int)__umulhi(se * 0x9E3779B1u, (uint32_t)left);  // a start spread over the list
+                w = 1;
+            }
+        }
+        phead = (phead + take) & (kPool - 1);
+        pn -= take;
+        __syncwarp();
+        if (take == 0 && idle == kFull && c >= items) break;
+    }
+}
+
+// One launch of a union pass: the heavy vertices a CTA each (largest work bound
+// first; the warps claim groups of 32 arcs), then the light ones a warp each.
+// Bound by instruction issue on the integer pipe, like the counting passes:
+// four CTAs of 8 warps per SM at 64 registers (the drain is inlined).
+template <Mode M, int TW, bool kAlive>
+__global__ void __launch_bounds__(TW * 32, TW == kTW ? 4 : 1) tri_union_kernel(TriArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int s_next;
+    __shared__ long long s_h;
+    __shared__ int s_stash_n[TW + 1];
+    __shared__ unsigned long long s_stash[TW + 1][kStash];
+    __shared__ uint32_t s_dead[TW][kUnionLightMax / 32];
+    __shared__ int s_lnext[TW];
+    __shared__ int s_bad;
+    unsigned char *tbl = smem + sizeof(UnionScratch) * TW;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    UnionScratch &q = reinterpret_cast<UnionScratch *>(smem)[warp];
+    QState qst;
+    unsigned long long probes = 0, tris = 0;
+    const int64_t n_heavy = a.n_heavy_dev ? (int64_t)*a.n_heavy_dev : a.n_heavy;
+    if constexpr (kAlive) {  // live lists of a scan that gave up are not followed
+        if (threadIdx.x == 0) s_bad = *(volatile int *)a.err;
+        __syncthreads();
+        if (s_bad != 0) return;
+    }
+
+    // ---- heavy vertices
+    {
+        const int cap = a.heavy_cap;  // table capacity: larger N+(u) is processed in chunks
+        TabCtx t;
+        t.tb = Table{reinterpret_cast<uint32_t *>(tbl), s_stash[TW], &s_stash_n[TW],
+                     reinterpret_cast<uint32_t *>(tbl) + 4 * cap,
+                     reinterpret_cast<uint32_t *>(tbl) + 4 * cap + (cap + 31) / 32};
+        for (;;) {
+            if (threadIdx.x == 0) s_h = (long long)atomicAdd(a.work, 1ull);
+            __syncthreads();
+            const int64_t h = s_h;
+            if (h >= n_heavy) break;
+            t.u = __ldg(a.heavy + h);
+            const int64_t ou = __ldg(a.offp + t.u);
+            t.d = (int)(__ldg(a.offp + t.u + 1) - ou);
+            const int nin = (int)__ldg(a.din + t.u);
+            const int64_t ib = __ldg(a.offs + t.u) - ou;             // start of u's in-arcs in inl
+            int ax = 0;
+            if constexpr (kAlive) {
+                if (t.d <= a.short_max) {
+                    __syncthreads();  // s_h is read before it is written again
+                    continue;
+                }
+                ax = (int)__ldg(a.arec + t.u).w;
+            }
+            for (int c0 = 0; c0 < t.d; c0 += cap) {
+                const int cn = min(cap, t.d - c0);
+                const int log_slots = ceil_log2(4 * cn) < 3 ? 3 : ceil_log2(4 * cn);
+                t.sh = 32 - log_slots;
+                t.fsh = t.sh - kFilterLog;
+                t.tbase = (uint32_t)(ou + c0);
+                t.cn = (uint32_t)cn;
+                for (int s2 = threadIdx.x; s2 < (1 << log_slots); s2 += blockDim.x) t.tb.slot[s2] = kSlotEmpty;
+                for (int s2 = threadIdx.x; s2 < (1 << (log_slots + kFilterLog - 5)); s2 += blockDim.x) t.tb.filter[s2] = 0;
+                if (threadIdx.x == 0) {
+                    s_next = 0;
+                    *t.tb.stash_n = 0;
+                }
+                __syncthreads();
+                for (int k0 = warp * 32; k0 < cn; k0 += TW * 32) {
+                    const int k = k0 + lane;
+                    bool dead = false;
+                    if (k < cn) {
+                        const uint32_t w = __ldg(a.colp + t.tbase + k), f = filter_bit(t, w);
+                        atomicOr(t.tb.filter + (f >> 5), 1u << (f & 31));
+                        table_insert(t.tb, log_slots, w, k, a.err);
+                        dead = arc_deleted(a.del, t.tbase + (uint32_t)k);
+                    }
+                    const unsigned dm = __ballot_sync(kFull, dead);
+                    if (lane == 0) t.tb.dead[k0 >> 5] = dm;
+                }
+                __syncthreads();
+                t.stash_n = min(*t.tb.stash_n, kStash);
+                stream_arcs<M, kAlive>(a, t, &s_next, (uint32_t)ou, ib, nin, ax, q, qst, probes, tris, c0 == 0);
+                flush_union<M>(a, t, q, qst, tris);
+                __syncthreads();  // the table is rebuilt for the next chunk or vertex
+            }
+        }
+    }
+
+    // ---- light vertices
+    if constexpr (TW == kTW && !kAlive) {
+        TabCtx t;
+        constexpr int kWords = 4 * kUnionLightMax + 4 * kUnionLightMax * kFilterBits / 4 / 32;  // slots, filter
+        uint32_t *own = reinterpret_cast<uint32_t *>(tbl) + warp * kWords;
+        t.tb = Table{own, s_stash[warp], &s_stash_n[warp], s_dead[warp], own + 4 * kUnionLightMax};
+        for (;;) {
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(a.work + 1, 32ull);
+            base = __shfl_sync(kFull, base, 0);
+            if ((int64_t)base >= a.n) break;
+            const int64_t ul = (int64_t)base + lane;
+            uint32_t oul = 0;
+            int dl = 0, nl = 0;
+            if (ul < a.n) {
+                const int64_t o0 = __ldg(a.offp + ul);
+                oul = (uint32_t)o0;
+                dl = (int)(__ldg(a.offp + ul + 1) - o0);
+                nl = (int)__ldg(a.din + ul);
+            }
+            // d+(u) < 2 closes no triangle at u (and then u has no in-arcs to stream)
+            unsigned lm = __ballot_sync(kFull, dl >= 2 && dl <= a.light_max && dl + nl <= a.light_items);
+            while (lm) {
+                const int src = __ffs(lm) - 1;
+                lm &= lm - 1;
+                t.u = (uint32_t)(base + src);
+                t.tbase = __shfl_sync(kFull, oul, src);
+                t.d = __shfl_sync(kFull, dl, src);
+                t.cn = (uint32_t)t.d;
+                const int nin = __shfl_sync(kFull, nl, src);
+                const int log_slots = max(3, ceil_log2(4 * t.d));
+                t.sh = 32 - log_slots;
+                t.fsh = t.sh - kFilterLog;
+                for (int s2 = lane; s2 < (1 << log_slots); s2 += 32) t.tb.slot[s2] = kSlotEmpty;
+                for (int s2 = lane; s2 < (1 << (log_slots + kFilterLog - 5)); s2 += 32) t.tb.filter[s2] = 0;
+                if (lane == 0) {
+                    *t.tb.stash_n = 0;
+                    s_lnext[warp] = 0;
+                }
+                __syncwarp();
+                for (int k0 = 0; k0 < t.d; k0 += 32) {
+                    const int k = k0 + lane;
+                    bool dead = false;
+                    if (k < t.d) {
+                        const uint32_t w = __ldg(a.colp + t.tbase + k), f = filter_bit(t, w);
+                        atomicOr(t.tb.filter + (f >> 5), 1u << (f & 31));
+                        table_insert(t.tb, log_slots, w, k, a.err);
+                        dead = arc_deleted(a.del, t.tbase + (uint32_t)k);
+                    }
+                    const unsigned dm = __ballot_sync(kFull, dead);
+                    if (lane == 0) t.tb.dead[k0 >> 5] = dm;
+                }
+                __syncwarp();
+                t.stash_n = min(*t.tb.stash_n, kStash);
+                stream_arcs<M, false>(a, t, &s_lnext[warp], t.tbase, nin > 0 ? __ldg(a.offs + t.u) - (int64_t)t.tbase : 0,
+                                      nin, 0, q, qst, probes, tris, true);
+                flush_union<M>(a, t, q, qst, tris);
+                __syncwarp();
+            }
+        }
+    }
+    const unsigned long long P = warp_sum(probes), T = warp_sum(tris);
+    if (lane == 0) {
+        atomicAdd(a.ctr + kCtrProbes, P);
+        atomicAdd(a.ctr + kCtrTriangles, T);
+    }
+}
+
 // Heavy vertices in decreasing out-degree order, by log2 buckets: pass 1
 // counts the vertices of each bucket (and the maximum out-degree), pass 2
 // scatters them so that larger buckets come first.
@@ -861,10 +1358,11 @@ __device__ __forceinline__ int heavy_key(int64_t d, int64_t nin, int64_t hub_min
 }
 
 // Also writes every vertex's in-degree d(u) - d+(u): the length of its
-// in-list in the reverse list (see Oriented::inl).
+// in-list in the reverse list (see Oriented::inl), and its off+ and d+ as one
+// 8-byte record.
 __global__ void classify_count_kernel(const int64_t *__restrict__ offp, const int64_t *__restrict__ offs,
-                                      uint32_t *din, int64_t n, int light_max, int light_items, int64_t hub_min,
-                                      unsigned long long *bucket_cnt, unsigned long long *ctr) {
+                                      uint32_t *din, uint2 *vrec, int vstep, int64_t n, int light_max, int light_items,
+                                      int64_t hub_min, unsigned long long *bucket_cnt, unsigned long long *ctr) {
     __shared__ unsigned int s_cnt[kKeys];
     if (threadIdx.x < kKeys) s_cnt[threadIdx.x] = 0;
     __syncthreads();
@@ -876,6 +1374,7 @@ __global__ void classify_count_kernel(const int64_t *__restrict__ offp, const in
         int64_t nin = (offs[u + 1] - offs[u]) - d;
         nin = nin < 0 ? 0 : nin;
         din[u] = (uint32_t)nin;
+        if (vrec) vrec[u * vstep] = make_uint2((uint32_t)offp[u], (uint32_t)d);
         if (is_heavy(d, nin, light_max, light_items)) atomicAdd(&s_cnt[heavy_key(d, nin, hub_min)], 1u);
     }
 #pragma unroll
@@ -960,18 +1459,13 @@ __global__ void eo_accept_kernel(TriArgs a, const int64_t *__restrict__ off, uin
             if constexpr (CH == kChoiceMinCount) {
                 chosen = mincount_arc(a.tcnt, e01, e02, e12);
             } else if constexpr (CH == kChoiceMaxw) {
-                const float w01 = __ldg(a.wp + e01), w02 = __ldg(a.wp + e02), w12 = __ldg(a.wp + e12);
-                chosen = e01;
-                float bw = w01;
-                uint32_t bl = x0, bh = x1;
-                if (w02 > bw || (w02 == bw && (x0 > bl || (x0 == bl && x2 > bh)))) { chosen = e02; bw = w02; bl = x0; bh = x2; }
-                if (w12 > bw || (w12 == bw && (x1 > bl || (x1 == bl && x2 > bh)))) { chosen = e12; }
+                chosen = maxw_arc(a.wp, x0, x1, x2, (uint32_t)e01, (uint32_t)e02, (uint32_t)e12);
             } else {
                 const uint4 rr = philox4x32_10(make_uint4(x0, x1, x2, kTagTri), a.k0, a.k1);
                 const int k = (int)(((unsigned long long)rr.y * 3ull) >> 32);
                 chosen = k == 0 ? e01 : (k == 1 ? e02 : e12);
             }
-            if (chosen == e) a.del[e] = 1;
+            if (chosen == e) delete_arc(a.del, (uint32_t)e);
         }
     }
 }
@@ -982,7 +1476,7 @@ __global__ void eo_accept_kernel(TriArgs a, const int64_t *__restrict__ off, uin
 template <int CH>
 __global__ void eo_list_accept_kernel(const TriRec *__restrict__ L, int64_t len,
                                       const unsigned long long *__restrict__ resv, uint32_t *considered,
-                                      uint8_t *del, const float *__restrict__ wp, const uint32_t *__restrict__ tcnt) {
+                                      uint32_t *del, const float *__restrict__ wp, const uint32_t *__restrict__ tcnt) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += stride) {
         const TriRec r = L[i];
@@ -996,17 +1490,12 @@ __global__ void eo_list_accept_kernel(const TriRec *__restrict__ L, int64_t len,
         if constexpr (CH == kChoiceMinCount) {
             chosen = mincount_arc(tcnt, r.e01, r.e02, r.e12);
         } else if constexpr (CH == kChoiceMaxw) {
-            const float w01 = __ldg(wp + r.e01), w02 = __ldg(wp + r.e02), w12 = __ldg(wp + r.e12);
-            chosen = r.e01;
-            float bw = w01;
-            uint32_t bl = r.x0, bh = r.x1;
-            if (w02 > bw || (w02 == bw && (r.x0 > bl || (r.x0 == bl && r.x2 > bh)))) { chosen = r.e02; bw = w02; bl = r.x0; bh = r.x2; }
-            if (w12 > bw || (w12 == bw && (r.x1 > bl || (r.x1 == bl && r.x2 > bh)))) { chosen = r.e12; }
+            chosen = maxw_arc(wp, r.x0, r.x1, r.x2, r.e01, r.e02, r.e12);
         } else {
             const int k = (int)(((unsigned long long)r.r1 * 3ull) >> 32);
             chosen = k == 0 ? r.e01 : (k == 1 ? r.e02 : r.e12);
         }
-        del[chosen] = 1;
+        delete_arc(del, chosen);
     }
 }
 
@@ -1149,6 +1638,11 @@ struct Plan {
     uint32_t *heavy = nullptr;
     unsigned long long *buckets = nullptr;  // counts [kKeys], fills [kKeys]
     uint32_t *din = nullptr;                // in-arcs streamed from the head's side, per vertex
+    bool records = false;                   // union passes: off+ and d+ of vertex v at vrec[v * vstep]
+    uint2 *vrec = nullptr;
+    int vstep = 1;
+    void *rec_own = nullptr;                // the records' allocation, if they have one
+    uint4 *arec = nullptr;                  // the same as 16-byte records (vstep 2), if there is room for them
     uint2 *inl = nullptr;                   // their (tail, arc), at offs(v) - offp(v) per vertex
     const int64_t *offs = nullptr;          // symmetric offsets of the graph
     int64_t n_heavy = 0, max_deg = 0;
@@ -1158,9 +1652,9 @@ struct Plan {
     size_t hub_smem = 0;
     int light_max = kLightMax;
     int light_items = kLightItems;
-    int log_slots = 3;
     size_t smem = 0;
     int heavy_cap = 8;  // phase-1 table entries
+    size_t usmem = 0, uhub_smem = 0;  // shared memory of the union passes' launches
 };
 
 static sg_status read_ctr(Ctx *c, int first, int count, unsigned long long *out) {
@@ -1175,12 +1669,21 @@ static void free_plan(Ctx *c, Plan *pl) {
     dfree(c, pl->heavy);
     dfree(c, pl->buckets);
     dfree(c, pl->din);
+    dfree(c, pl->rec_own);
+    pl->rec_own = nullptr;
+    pl->vrec = nullptr;
+    pl->arec = nullptr;
     pl->heavy = nullptr;
     pl->buckets = nullptr;
     pl->din = nullptr;
     pl->inl = nullptr;
 }
 
+
+// a union table of `cap` entries: four slots each, one deletion flag bit, the filter
+static size_t union_table_bytes(int cap) {
+    return (size_t)cap * 4 * sizeof(uint32_t) + (size_t)(cap + 31) / 32 * 4 + (size_t)cap * kFilterBits / 8;
+}
 
 // inl_cap: room for in-arc records; nnz - m when E+ holds all m arcs, nnz
 // when it may hold fewer (batches orient only their triangle-kernel graphs).
@@ -1193,6 +1696,22 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
     sg_status st = dalloc(c, (void **)&pl->heavy, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
     if (st == SG_OK) st = dalloc(c, (void **)&pl->buckets, sizeof(unsigned long long) * 2 * kKeys);
     if (st == SG_OK) st = dalloc(c, (void **)&pl->din, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
+    if (st == SG_OK && pl->records) {
+        // 16-byte records in the unused half of E+'s column array (room for nnz
+        // = 2m entries), or else 8-byte ones and no second pass
+        const uintptr_t b = ((uintptr_t)(o.col + o.m) + 15) & ~(uintptr_t)15, e = (uintptr_t)(o.col + 2 * o.m);
+        if (o.m > 0 && b + sizeof(uint4) * (size_t)o.n <= e) {
+            pl->arec = reinterpret_cast<uint4 *>(b);
+            pl->vstep = 2;
+        } else if (dalloc(c, &pl->rec_own, sizeof(uint4) * (size_t)std::max<int64_t>(o.n, 1)) == SG_OK) {
+            pl->arec = static_cast<uint4 *>(pl->rec_own);
+            pl->vstep = 2;
+        } else {
+            set_error("");
+            st = dalloc(c, &pl->rec_own, sizeof(uint2) * (size_t)std::max<int64_t>(o.n, 1));
+        }
+        pl->vrec = pl->arec ? reinterpret_cast<uint2 *>(pl->arec) : static_cast<uint2 *>(pl->rec_own);
+    }
     if (st != SG_OK) return st;
     pl->inl = o.inl;  // the orientation's reverse list (not owned by the plan)
     SG_CUDA(cudaMemsetAsync(pl->buckets, 0, sizeof(unsigned long long) * 2 * kKeys, c->stream));
@@ -1200,7 +1719,8 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((o.n + 255) / 256, (int64_t)c->num_sms * 8));
     if (o.n > 0) {
         SG_LAUNCH(c, "tri_classify");
-        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, offs, pl->din, o.n, pl->light_max,
+        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, offs, pl->din, pl->vrec, pl->vstep,
+                                                                       o.n, pl->light_max,
                                                                        pl->light_items, (int64_t)kHeavyCap,
                                                                        pl->buckets, c->d_ctr);
     }
@@ -1238,80 +1758,95 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
     int cap = 8;
     while (cap < pl->max_deg && cap < kHeavyCap) cap *= 2;
     pl->heavy_cap = cap;
-    pl->log_slots = ceil_log2_host(4 * cap);
     const size_t entry_bytes = 4 * sizeof(uint32_t) + 2 * sizeof(uint32_t) + sizeof(unsigned short);
     pl->smem = queue_bytes + std::max(light_bytes, (size_t)cap * entry_bytes);
+    pl->usmem = sizeof(UnionScratch) * kTW +
+                std::max((size_t)kTW * kUnionLightMax * (4 * sizeof(uint32_t) + kFilterBits / 8), union_table_bytes(cap));
     if (pl->n_hubs > 0) {
         int hc = kHeavyCap;
         while (hc < pl->max_deg && hc < kHubCap) hc *= 2;
         pl->hub_cap = hc;
         pl->hub_smem = sizeof(HitQueue) * kHubTW + (size_t)hc * entry_bytes;
+        pl->uhub_smem = sizeof(UnionScratch) * kHubTW + union_table_bytes(hc);
     }
     return SG_OK;
 }
 
-template <Mode M>
-static sg_status launch_enum_raw(Ctx *c, TriArgs a, size_t smem, int grid_per_sm) {
+// One launch of `kernel`: as many CTAs per SM as fit (or grid_per_sm), which
+// claim their vertices through the work counters.
+static sg_status launch_tri(Ctx *c, void (*kernel)(TriArgs), int threads, size_t smem, const TriArgs &a,
+                            const char *name, int grid_per_sm = 0) {
     SG_CUDA(cudaMemsetAsync(a.work, 0, 2 * sizeof(unsigned long long), c->stream));
-    SG_CUDA(cudaFuncSetAttribute(tri_enum_kernel<M, kTW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
-    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tri_enum_kernel<M, kTW>, kTW * 32, smem));
+    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     per_sm = std::max(per_sm, 1);
     if (grid_per_sm > 0) per_sm = std::min(per_sm, grid_per_sm);
-    const int64_t grid = (int64_t)c->num_sms * per_sm;
     {
-        SG_LAUNCH(c, "tri_enum");
-        tri_enum_kernel<M, kTW><<<(unsigned)grid, kTW * 32, smem, c->stream>>>(a);
+        SG_LAUNCH(c, name);
+        kernel<<<(unsigned)(c->num_sms * per_sm), threads, smem, c->stream>>>(a);
     }
     SG_CUDA(cudaGetLastError());
     return SG_OK;
 }
 
-template <Mode M>
-static sg_status launch_enum(Ctx *c, const TriArgs &base, const Plan &pl) {
+// One pass over all vertices: the hubs first, in CTAs that share a large
+// table, then everything else.
+static sg_status launch_pass(Ctx *c, void (*hub)(TriArgs), void (*main)(TriArgs), size_t hub_smem, size_t smem,
+                             const TriArgs &base, const Plan &pl, const char *hub_name, const char *main_name) {
     if (base.n == 0) return SG_OK;
     TriArgs a = base;
     a.heavy = pl.heavy;
     a.n_heavy = pl.n_heavy;
-    a.heavy_log_slots = pl.log_slots;
     a.heavy_cap = pl.heavy_cap;
     a.light_max = pl.light_max;
     a.light_items = pl.light_items;
     a.offs = pl.offs;
     a.din = pl.din;
+    a.vrec = pl.vrec;
+    a.vstep = pl.vstep;
     a.inl = pl.inl;
     a.work = c->d_ctr + kCtrAux;
     if (pl.n_hubs > 0) {
-        // the hubs first, one 32-warp CTA per SM sharing a large table
         TriArgs h = a;
         h.n_heavy = pl.n_hubs;
         h.heavy_cap = pl.hub_cap;
-        SG_CUDA(cudaMemsetAsync(h.work, 0, 2 * sizeof(unsigned long long), c->stream));
-        SG_CUDA(cudaFuncSetAttribute(tri_enum_kernel<M, kHubTW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)pl.hub_smem));
-        int hub_per_sm = 0;
-        SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&hub_per_sm, tri_enum_kernel<M, kHubTW>, kHubTW * 32,
-                                                              pl.hub_smem));
-        const int64_t hgrid = (int64_t)c->num_sms * std::max(hub_per_sm, 1);
-        {
-            SG_LAUNCH(c, "tri_hubs");
-            tri_enum_kernel<M, kHubTW><<<(unsigned)hgrid, kHubTW * 32, pl.hub_smem, c->stream>>>(h);
-        }
-        SG_CUDA(cudaGetLastError());
+        const sg_status st = launch_tri(c, hub, kHubTW * 32, hub_smem, h, hub_name);
+        if (st != SG_OK) return st;
         a.heavy = pl.heavy + pl.n_hubs;
         a.n_heavy = pl.n_heavy - pl.n_hubs;
     }
-    SG_CUDA(cudaMemsetAsync(a.work, 0, 2 * sizeof(unsigned long long), c->stream));
-    SG_CUDA(cudaFuncSetAttribute(tri_enum_kernel<M, kTW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem));
-    int per_sm = 0;
-    SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tri_enum_kernel<M, kTW>, kTW * 32, pl.smem));
-    const int64_t grid = (int64_t)c->num_sms * std::max(per_sm, 1);
-    {
-        SG_LAUNCH(c, "tri_enum");
-        tri_enum_kernel<M, kTW><<<(unsigned)grid, kTW * 32, pl.smem, c->stream>>>(a);
+    return launch_tri(c, main, kTW * 32, smem, a, main_name);
+}
+
+template <Mode M>
+static sg_status launch_enum(Ctx *c, const TriArgs &a, const Plan &pl) {
+    return launch_pass(c, tri_enum_kernel<M, kHubTW>, tri_enum_kernel<M, kTW>, pl.hub_smem, pl.smem, a, pl, "tri_hubs",
+                       "tri_enum");
+}
+
+// The two passes of a union kernel (see tri_union_kernel), h the output graph.
+// Without the second pass's scratch the first streams every list whole.
+template <Mode M>
+static sg_status launch_union(Ctx *c, const Oriented &o, TriArgs a, const Plan &pl, const Graph *h) {
+    AliveArcs al;
+    bool two = pl.max_deg > kShortList && pl.arec != nullptr;
+    if (two && alive_alloc(c, o, h, &al) != SG_OK) {
+        set_error("");
+        two = false;
     }
-    SG_CUDA(cudaGetLastError());
-    return SG_OK;
+    a.short_max = !two ? INT_MAX : (pl.n_hubs > 0 ? kShortListHubs : kShortList);
+    sg_status st = launch_pass(c, tri_union_kernel<M, kHubTW, false>, tri_union_kernel<M, kTW, false>, pl.uhub_smem,
+                               pl.usmem, a, pl, "tri_hubs", "tri_enum");
+    if (two && st == SG_OK) st = alive_build(c, o, a.del, al, pl.arec);
+    if (two && st == SG_OK) {
+        a.arec = pl.arec;
+        a.alive = al.list;
+        st = launch_pass(c, tri_union_kernel<M, kHubTW, true>, tri_union_kernel<M, kTW, true>, pl.uhub_smem, pl.usmem, a,
+                         pl, "tri_rest_hubs", "tri_rest");
+    }
+    if (two) alive_free(c, &al);
+    return st;
 }
 
 static TriArgs base_args(Ctx *c, const Oriented &o) {
@@ -1320,6 +1855,7 @@ static TriArgs base_args(Ctx *c, const Oriented &o) {
     a.colp = o.col;
     a.wp = o.w;
     a.n = o.n;
+    a.dead_flag = o.m <= (int64_t)kArcDead ? kArcDead : 0u;
     a.ctr = c->d_ctr;
     a.err = c->d_err;
     return a;
@@ -1634,8 +2170,18 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
     return st;
 }
 
-sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double p, uint64_t seed, uint8_t *del) {
+sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double p, uint64_t seed, uint32_t *del,
+                  const Graph *h) {
     Plan pl;
+    const bool eo = k == SG_TR_EO || k == SG_TR_EO_MAXW || k == SG_TR_EO_MINCOUNT;
+    if (k == SG_TR_MINCOUNT || eo) {  // the counting and edge-once passes' split
+        pl.light_max = kLightMax;
+        pl.light_items = kLightItems;
+    } else {
+        pl.light_max = kUnionLightMax;
+        pl.light_items = kUnionLightItems;
+        pl.records = true;
+    }
     sg_status st = make_plan(c, o, g->off, &pl);
     TriArgs a = base_args(c, o);
     a.k0 = (uint32_t)(seed & 0xFFFFFFFFu);
@@ -1651,13 +2197,21 @@ sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double
             st = cuda_fail(cudaGetLastError(), "cudaMemsetAsync(tcnt)");
         a.tcnt = tcnt;
         if (st == SG_OK) st = launch_enum<Mode::EdgeCount>(c, a, pl);
+        if (st == SG_OK && !eo) {  // the union passes split the vertices their own way
+            free_plan(c, &pl);
+            pl = Plan{};
+            pl.light_max = kUnionLightMax;
+            pl.light_items = kUnionLightItems;
+            pl.records = true;
+            st = make_plan(c, o, g->off, &pl);
+        }
     }
     if (st == SG_OK) {
         switch (k) {
-        case SG_TR_RANDOM: st = launch_enum<Mode::UnionRandom>(c, a, pl); break;
-        case SG_TR_MAXW: st = launch_enum<Mode::UnionMaxw>(c, a, pl); break;
-        case SG_TR_P2: st = launch_enum<Mode::UnionP2>(c, a, pl); break;
-        case SG_TR_MINCOUNT: st = launch_enum<Mode::UnionMinCount>(c, a, pl); break;
+        case SG_TR_RANDOM: st = launch_union<Mode::UnionRandom>(c, o, a, pl, h); break;
+        case SG_TR_MAXW: st = launch_union<Mode::UnionMaxw>(c, o, a, pl, h); break;
+        case SG_TR_P2: st = launch_union<Mode::UnionP2>(c, o, a, pl, h); break;
+        case SG_TR_MINCOUNT: st = launch_union<Mode::UnionMinCount>(c, o, a, pl, h); break;
         default: st = eo_rounds(c, g, o, k, pl, a); break;
         }
     }
@@ -1705,8 +2259,7 @@ sg_status batch_tr_prepare(Ctx *c, const Graph *u, const Oriented &o, BatchTri *
     pl.light_items = 4 * bt->light_max;
     sg_status st = make_plan(c, o, u->off, &pl);
     if (st == SG_OK) {
-        bt->log_slots = pl.log_slots;
-        bt->smem = pl.smem;
+        bt->smem = pl.usmem;
         bt->max_deg = pl.heavy_cap;
     }
     free_plan(c, &pl);
@@ -1714,6 +2267,7 @@ sg_status batch_tr_prepare(Ctx *c, const Graph *u, const Oriented &o, BatchTri *
     if (!bt->heavy) st = dalloc(c, (void **)&bt->heavy, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
     if (st == SG_OK && !bt->buckets)
         st = dalloc(c, (void **)&bt->buckets, sizeof(unsigned long long) * (2 * kKeys + 1));
+    if (st == SG_OK && !bt->vrec) st = dalloc(c, (void **)&bt->vrec, sizeof(uint2) * (size_t)std::max<int64_t>(o.n, 1));
     if (st == SG_OK && !bt->din) st = dalloc(c, (void **)&bt->din, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
     // Per call only the graphs with a triangle kernel are oriented, so E+ can
     // hold fewer than nnz/2 arcs and the in-list room off(v) - off+(v) then
@@ -1727,6 +2281,8 @@ void batch_tr_free(Ctx *c, BatchTri *bt) {
     dfree(c, bt->heavy);
     dfree(c, bt->buckets);
     dfree(c, bt->din);
+    dfree(c, bt->vrec);
+    bt->vrec = nullptr;
     dfree(c, bt->inl);
     bt->heavy = nullptr;
     bt->buckets = nullptr;
@@ -1736,7 +2292,7 @@ void batch_tr_free(Ctx *c, BatchTri *bt) {
 
 // No host synchronisation: the heavy-vertex count stays on the device.
 sg_status batch_tr_mark(Ctx *c, const Graph *u, const Oriented &o, const BatchDev &b, const BatchTri &bt,
-                        uint8_t *del) {
+                        uint32_t *del) {
     if (o.n == 0) return SG_OK;
     const int light_items = 4 * bt.light_max;
     SG_CUDA(cudaMemsetAsync(bt.buckets, 0, sizeof(unsigned long long) * (2 * kKeys + 1), c->stream));
@@ -1746,7 +2302,7 @@ sg_status batch_tr_mark(Ctx *c, const Graph *u, const Oriented &o, const BatchDe
     {
         SG_LAUNCH(c, "tri_classify");
         // no hub launch in a batch: its graphs are small, and a long N+(u) is chunked
-        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, u->off, bt.din, o.n, bt.light_max,
+        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, u->off, bt.din, bt.vrec, 1, o.n, bt.light_max,
                                                                        light_items, INT64_MAX, bt.buckets, c->d_ctr);
     }
     {
@@ -1762,17 +2318,19 @@ sg_status batch_tr_mark(Ctx *c, const Graph *u, const Oriented &o, const BatchDe
     a.heavy = bt.heavy;
     a.n_heavy = 0;
     a.n_heavy_dev = bt.buckets + 2 * kKeys;
-    a.heavy_log_slots = bt.log_slots;
     a.heavy_cap = bt.max_deg;
+    a.short_max = INT_MAX;  // one pass
     a.light_max = bt.light_max;
     a.light_items = light_items;
     a.offs = u->off;
     a.din = bt.din;
+    a.vrec = bt.vrec;
+    a.vstep = 1;
     a.inl = bt.inl;
     a.work = c->d_ctr + kCtrAux;
     a.bparams = b.params;
     a.vgid = b.vgid;
-    return launch_enum_raw<Mode::BatchUnion>(c, a, bt.smem, bt.grid_per_sm);
+    return launch_tri(c, tri_union_kernel<Mode::BatchUnion, kTW, false>, kTW * 32, bt.smem, a, "tri_enum", bt.grid_per_sm);
 }
 
 }  // namespace sg

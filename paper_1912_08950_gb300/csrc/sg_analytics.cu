@@ -25,187 +25,433 @@ namespace sg {
 constexpr int kPrThreads = 256;
 constexpr int kPrWarps = kPrThreads / 32;
 
-// x'_v = (1-d)/n + d (sum_{u in N(v)} y_u + D/n), y_u = x_u / d_u; emits
-// y' = x'/d and, per block, the FP32 dangling mass of x' (and, on the last
-// iteration, the FP64 partial L1 residual |x' - x|).
+// x'_v = (1-d)/n + d (sum_{u in N(v)} y_u + D/n), y_u = x_u / d_u, D the rank
+// of the degree-0 vertices.
 //
-// Row sums: a warp owns 32 consecutive rows.  Rows longer than 32 arcs are
-// summed by the whole warp, one row at a time (lanes stride the row, then a
-// fixed shuffle tree).  The short rows are summed together: their arcs are
-// numbered consecutively across the 32 rows and streamed in slabs of 32, a
-// lane finds its arc's row among the rows' starts (binary search over the
-// lanes), a segmented shuffle scan sums each row's run inside the slab and the
-// run's last lane adds it to the row's slot in shared memory.  Every order is
-// fixed, so a graph always gives the same vector.
+// An iteration is one gather of y per arc, and the gathers, not the bytes, are
+// the bound: a warp's 32 loads fall into 32 sectors, and the L1 can only have as
+// many misses in flight as it has lines.  So y is kept in order of falling
+// degree -- the arcs' heads are translated to positions once per call (colx)
+// -- and every CTA copies its first kPrHot entries (R-MAT s22: 0.8% of the
+// vertices, the heads of 54% of the arcs) to shared memory when an iteration
+// starts; the L1 keeps the next ones, which share lines.  The heads stream past
+// it (evict-first).  One CTA of 32 warps per SM, eight slabs of 32 arcs in
+// flight per warp.  Per iteration on R-MAT s22 (128 M arcs) 358 us, against 634
+// with y in vertex order and launches of their own for hub rows and D; s20: 92
+// against 172.  Half of the L1 for y is where the line lies: 373 us at 32 K
+// entries before the heads were streamed, 403 at 16 K, 387 at 24 K and 389 at
+// 40 K; 54 K entries (all of the shared memory) leave too few lines: 588.
+//
+// Row sums have a fixed order, so a graph always gives the same vector: rows
+// of up to kShortRow arcs are summed 32 rows at a time -- their arcs are
+// numbered consecutively and streamed in slabs of 32, a lane finds its arc's
+// row among the rows' starts, a segmented shuffle scan sums each row's run
+// inside the slab and the run's last lane adds it to the row's slot; longer
+// rows by a warp (lanes stride the row, then a fixed shuffle tree); hub rows
+// in chunks of kHubChunk arcs (eight interleaved runs per lane, each run's
+// tree, then the eight in order), and the warp that finishes a hub's last chunk
+// adds the chunks in order.
 constexpr int kShortRow = 32;
-constexpr int kHubRow = 1024;    // longer rows are summed in chunks by whole CTAs
-constexpr int kHubChunk = 8192;  // arcs per chunk
+constexpr int kHubRow = 1024;
+constexpr int kHubChunk = 8192;
+constexpr int kPrCta = 1024;              // threads of the iteration kernel
+constexpr int kPrHot = 32 * 1024;         // entries of y in shared memory, at most
+constexpr int kDegBuckets = 256;          // degree buckets: exact below 16, eighths of an octave above
 
-__global__ void __launch_bounds__(kPrThreads) pr_iter_kernel(
-    const int64_t *__restrict__ off, const uint32_t *__restrict__ col, int64_t n, const float *__restrict__ x,
-    const float *__restrict__ y, const float *__restrict__ dangling_in, float base, float damping, float inv_n,
-    float *__restrict__ x_new, float *__restrict__ y_new, float *__restrict__ dangling_part,
-    double *__restrict__ resid_part, const int *__restrict__ hub_slot, const float *__restrict__ hub_part) {
-    __shared__ float s_dang[kPrWarps];
-    __shared__ double s_res[kPrWarps];
-    __shared__ float s_acc[kPrWarps][32];
+__device__ __forceinline__ int degree_bucket(int64_t d) {
+    if (d < 16) return (int)d;
+    const int e = 63 - __clzll((unsigned long long)d);
+    return min(16 + (e - 4) * 8 + (int)((d >> (e - 3)) & 7), kDegBuckets - 1);
+}
+
+struct PrHubs {
+    const uint32_t *row;        // hub rows, in any order
+    const unsigned long long *count;  // [0] hubs, [1] chunks, [2] rows of medium length
+    const int *first;           // first chunk of hub h
+    const uint32_t *chunk_hub;  // hub of chunk c
+    float *part;                // chunk sums
+    unsigned int *done;         // chunks of hub h summed in this iteration (0 between iterations)
+};
+
+struct PrArgs {
+    const int64_t *off;
+    const uint32_t *colx;  // position in y of every arc's head
+    const uint32_t *pos;   // position of every vertex (NULL: its id)
+    int64_t n;
+    int hot;               // the first positions, which a CTA keeps in shared memory (0: none)
+    float base, damping, inv_n;
+    const float *y;
+    float *y_new;
+    float *x_prev;         // the values before the last iteration
+    float *x_out;
+    double *resid_part;    // per CTA
+    PrHubs hubs;
+    const uint32_t *medium;  // rows of more than kShortRow arcs that are no hubs, in any order
+    // the rank of the degree-0 vertices: how many each virtual lane sums, the
+    // warp sums that give D of the last iteration and those of this one
+    const uint32_t *lane_cnt;
+    int vblocks;
+    const float *wsum;
+    float *wsum_new;
+    unsigned int *work, *work_next;  // next unit of this iteration, of the next one
+    int per_claim;         // 32-row groups per claim
+};
+
+// D of the last iteration from its warp sums: every virtual block's eight in
+// order, then a fixed tree over 256 strided sums.  All threads call it.
+__device__ float pr_dangling(const float *wsum, int vblocks, float *s) {
+    if (threadIdx.x < kPrThreads) {
+        float acc = 0.f;
+        for (int i = threadIdx.x; i < vblocks; i += kPrThreads) {
+            float bd = 0.f;
+            for (int w = 0; w < kPrWarps; ++w) bd += __ldg(wsum + (size_t)i * kPrWarps + w);
+            acc += bd;
+        }
+        s[threadIdx.x] = acc;
+    }
+    __syncthreads();
+    for (int h = kPrThreads / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) s[threadIdx.x] += s[threadIdx.x + h];
+        __syncthreads();
+    }
+    return s[0];
+}
+
+// Warp sums of the rank of the degree-0 vertices, each of which holds `val`: a
+// lane of the virtual warps adds its vertices' ranks one by one.
+__device__ __forceinline__ void pr_dangling_sums(const uint32_t *lane_cnt, int vblocks, float val, float *wsum) {
+    const int lane = threadIdx.x & 31;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < (int64_t)vblocks * kPrWarps; w += nw) {
+        float t = 0.f;
+        for (uint32_t k = __ldg(lane_cnt + w * 32 + lane); k > 0; --k) t += val;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+        if (lane == 0) wsum[w] = t;
+    }
+}
+
+// What an iteration stores besides y: nothing, x (the one before the last), or
+// x_out and the FP64 partial L1 residual |x_out - x_prev| (the last).
+enum class PrStore { kNone, kPrev, kLast };
+
+template <bool kHot, PrStore S>
+__global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
+    extern __shared__ float s_y[];
+    __shared__ float s_acc[kPrCta / 32][32];
+    __shared__ float s_red[kPrThreads];
+    __shared__ double s_res[kPrCta / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const float dterm = dangling_in[0] * inv_n;
-    float dang = 0.f;
+    if constexpr (kHot) {
+        const int quads = (a.hot + 3) >> 2;  // (y has room for whole ones)
+        const float4 *src = reinterpret_cast<const float4 *>(a.y);
+        for (int i = threadIdx.x; i < quads; i += kPrCta) reinterpret_cast<float4 *>(s_y)[i] = __ldg(src + i);
+    }
+    const float dterm = pr_dangling(a.wsum, a.vblocks, s_red) * a.inv_n;
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.work_next = 0;
+    if (S != PrStore::kLast) pr_dangling_sums(a.lane_cnt, a.vblocks, a.base + a.damping * (0.f + dterm), a.wsum_new);
+    // one generic load, from shared or global memory as the lane's position
+    // says: two loads behind a branch would each wait for the other's
+    auto rank_of = [&](uint32_t i) {
+        float v;
+        const float *base = kHot && i < (uint32_t)a.hot ? s_y : a.y;
+        asm volatile("ld.f32 %0, [%1];" : "=f"(v) : "l"(base + i));
+        return v;
+    };
     double res = 0.0;
-    const int64_t nwarps = (int64_t)gridDim.x * kPrWarps;
-    for (int64_t r0 = ((int64_t)blockIdx.x * kPrWarps + warp) * 32; r0 < n; r0 += nwarps * 32) {
-        const int64_t v = r0 + lane;
-        int64_t b = 0, e = 0;
-        if (v < n) {
-            b = __ldg(off + v);
-            e = __ldg(off + v + 1);
+    auto finish = [&](int64_t v, int64_t deg, float s) {
+        const float xv = a.base + a.damping * (s + dterm);
+        if (S == PrStore::kPrev) a.x_prev[v] = xv;
+        if (S == PrStore::kLast) {
+            a.x_out[v] = xv;
+            res += fabs((double)xv - (double)__ldg(a.x_prev + v));
+        } else if (deg > 0) {
+            a.y_new[a.pos ? __ldg(a.pos + v) : (uint32_t)v] = xv / (float)deg;
         }
-        const int64_t deg = e - b;
-        const bool longr = deg > kShortRow;
-        // short rows: consecutive numbering of their arcs
-        const int sdeg = longr ? 0 : (int)deg;
-        int vs = sdeg;
+    };
+    // units, the longest first: chunks of hub rows, 32 rows of medium length,
+    // groups of 32 consecutive rows for their short ones
+    const unsigned nchunks = (unsigned)a.hubs.count[1];
+    const unsigned nmed = (unsigned)a.hubs.count[2], med_units = (nmed + 31) / 32;
+    const unsigned groups = (unsigned)((a.n + 31) / 32);
+    const unsigned units = nchunks + med_units + (groups + a.per_claim - 1) / a.per_claim;
+    constexpr int kB = 8;  // slabs in flight
+    for (;;) {
+        unsigned u = 0;
+        if (lane == 0) u = atomicAdd(a.work, 1u);
+        u = __shfl_sync(kFull, u, 0);
+        if (u >= units) break;
+        if (u < nchunks) {  // one chunk of a hub row
+            const uint32_t h = __ldg(a.hubs.chunk_hub + u);
+            const int first = __ldg(a.hubs.first + h);
+            const int64_t v = __ldg(a.hubs.row + h);
+            const int64_t rb = __ldg(a.off + v), re = __ldg(a.off + v + 1);
+            const int64_t cb = rb + (int64_t)((int)u - first) * kHubChunk;
+            const int64_t ce = min(cb + (int64_t)kHubChunk, re);
+            static_assert(kB == kPrWarps, "a step of a chunk is one slab of each run");
+            float t[kB];
+            uint32_t c[kB];
+            auto load = [&](int64_t i) {
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, vs, o);
-            if (lane >= o) vs += t;
-        }
-        const int total = __shfl_sync(kFull, vs, 31);
-        vs -= sdeg;  // exclusive start of this row's arcs
-        s_acc[warp][lane] = 0.f;
-        __syncwarp();
-        for (int s0 = 0; s0 < total; s0 += 32) {
-            const int i = s0 + lane;
-            const bool valid = i < total;
-            int k = 0;  // the last row whose start is <= i
+                for (int w = 0; w < kB; ++w) c[w] = i + w * 32 < ce ? __ldcs(a.colx + i + w * 32) : 0u;
+            };
 #pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const int sk = __shfl_sync(kFull, vs, k + step);
-                if (sk <= i) k += step;
+            for (int w = 0; w < kB; ++w) t[w] = 0.f;
+            load(cb + lane);
+            for (int64_t i = cb + lane; i - lane < ce; i += kPrThreads) {
+                float r[kB];
+#pragma unroll
+                for (int w = 0; w < kB; ++w) r[w] = i + w * 32 < ce ? rank_of(c[w]) : 0.f;
+                load(i + kPrThreads);  // the next step's, while these are on their way
+#pragma unroll
+                for (int w = 0; w < kB; ++w) t[w] += r[w];
             }
-            const int64_t bk = __shfl_sync(kFull, b, k);
-            const int vk = __shfl_sync(kFull, vs, k);
-            float val = valid ? __ldg(y + __ldg(col + bk + (i - vk))) : 0.f;
+            float acc = 0.f;
+#pragma unroll
+            for (int w = 0; w < kB; ++w) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) t[w] += __shfl_xor_sync(kFull, t[w], o);
+                acc += t[w];
+            }
+            if (lane == 0) {
+                const int nch = (int)((re - rb + kHubChunk - 1) / kHubChunk);
+                __stcg(a.hubs.part + u, acc);
+                __threadfence();
+                if (atomicAdd(a.hubs.done + h, 1u) == (unsigned)nch - 1) {  // the row's last chunk
+                    __threadfence();
+                    float s = 0.f;
+                    for (int c2 = 0; c2 < nch; ++c2) s += __ldcg(a.hubs.part + first + c2);
+                    a.hubs.done[h] = 0;
+                    finish(v, re - rb, s);
+                }
+            }
+            continue;
+        }
+        u -= nchunks;
+        if (u < med_units) {
+            // a row per lane; the rows' slabs of 32 arcs as one sequence, kB of them in flight
+            const unsigned mi = u * 32 + lane;
+            int64_t v = -1, b = 0, e = 0;
+            if (mi < nmed) {
+                v = __ldg(a.medium + mi);
+                b = __ldg(a.off + v);
+                e = __ldg(a.off + v + 1);
+            }
+            int vs = (int)((e - b + 31) / 32);  // this row's slabs, then the slabs before it
+            const int mine = vs;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const float t = __shfl_up_sync(kFull, val, o);
-                const int kt = __shfl_up_sync(kFull, k, o);
-                if (lane >= o && kt == k) val += t;
+                const int t = __shfl_up_sync(kFull, vs, o);
+                if (lane >= o) vs += t;
             }
-            const int kn = __shfl_down_sync(kFull, k, 1);
-            if (valid && (lane == 31 || kn != k || i + 1 >= total)) s_acc[warp][k] += val;
+            const int total = __shfl_sync(kFull, vs, 31);
+            vs -= mine;
+            float s = 0.f, t = 0.f;
+            for (int w0 = 0; w0 < total; w0 += 32) {  // 32 slabs: a lane locates one
+                const int sl = w0 + lane;
+                int k = 0;  // the row of slab sl: the last one that starts at or before it
+#pragma unroll
+                for (int step = 16; step >= 1; step >>= 1) {
+                    const int sk = __shfl_sync(kFull, vs, k + step);
+                    if (sk <= sl) k += step;
+                }
+                const int64_t rb = __shfl_sync(kFull, b, k), re = __shfl_sync(kFull, e, k);
+                const int64_t at = rb + (int64_t)(sl - __shfl_sync(kFull, vs, k)) * 32;
+                // arcs of the slab; bit 8: the row's last; its row
+                const int meta = sl < total ? (int)min((int64_t)32, re - at) | (re - at <= 32 ? 256 : 0) | (k << 9) : 0;
+                const int m = min(32, total - w0);
+                uint32_t c[kB];
+                int mn[kB], mc[kB];
+                auto load = [&](int q0) {  // (slabs past the last have no arcs)
+                    int64_t p[kB];
+#pragma unroll
+                    for (int q = 0; q < kB; ++q) {
+                        p[q] = __shfl_sync(kFull, at, (q0 + q) & 31) + lane;
+                        mn[q] = q0 + q < m ? __shfl_sync(kFull, meta, (q0 + q) & 31) : 0;
+                    }
+#pragma unroll
+                    for (int q = 0; q < kB; ++q) c[q] = lane < (mn[q] & 255) ? __ldcs(a.colx + p[q]) : 0u;
+                };
+                load(0);
+                for (int q0 = 0; q0 < m; q0 += kB) {
+                    float r[kB];
+#pragma unroll
+                    for (int q = 0; q < kB; ++q) {
+                        mc[q] = mn[q];
+                        r[q] = 0.f;
+                        if (lane < (mc[q] & 255)) r[q] = rank_of(c[q]);
+                    }
+                    if (q0 + kB < m) load(q0 + kB);  // the next slabs', while these are on their way
+#pragma unroll
+                    for (int q = 0; q < kB; ++q) {
+                        t += r[q];
+                        if (mc[q] & 256) {  // (warp-uniform) the row's fixed tree over the lanes
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+                            if (lane == (mc[q] >> 9)) s = t;
+                            t = 0.f;
+                        }
+                    }
+                }
+            }
+            if (v >= 0) finish(v, e - b, s);
+            continue;
+        }
+        const int64_t g0 = (int64_t)(u - med_units) * a.per_claim;
+        const int64_t g1 = min(g0 + a.per_claim, (int64_t)groups);
+        int64_t nb = 0, ne = 0;
+        auto load_rows = [&](int64_t g) {
+            const int64_t v = g * 32 + lane;
+            nb = ne = 0;
+            if (v < a.n) {
+                nb = __ldg(a.off + v);
+                ne = __ldg(a.off + v + 1);
+            }
+        };
+        load_rows(g0);
+        for (int64_t g = g0; g < g1; ++g) {
+            const int64_t v = g * 32 + lane;
+            const int64_t b = nb, e = ne;
+            if (g + 1 < g1) load_rows(g + 1);
+            const int64_t deg = e - b;
+            const bool shortr = deg <= kShortRow;
+            // consecutive numbering of the short rows' arcs
+            const int sdeg = shortr ? (int)deg : 0;
+            int vs = sdeg;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(kFull, vs, o);
+                if (lane >= o) vs += t;
+            }
+            const int total = __shfl_sync(kFull, vs, 31);
+            vs -= sdeg;  // exclusive start of this row's arcs
+            s_acc[warp][lane] = 0.f;
             __syncwarp();
-        }
-        float s = s_acc[warp][lane];
-        __syncwarp();
-        // hub rows: their chunk sums, in chunk order
-        if (deg > kHubRow) {
-            const int first = __ldg(hub_slot + v);
-            const int nch = (int)((deg + kHubChunk - 1) / kHubChunk);
-            float t = 0.f;
-            for (int c2 = 0; c2 < nch; ++c2) t += __ldg(hub_part + first + c2);
-            s = t;
-        }
-        // long rows: the whole warp, one row at a time, fixed tree order
-        unsigned longm = __ballot_sync(kFull, longr && deg <= kHubRow);
-        while (longm) {
-            const int src = __ffs(longm) - 1;
-            longm &= longm - 1;
-            const int64_t lb = __shfl_sync(kFull, b, src), le = __shfl_sync(kFull, e, src);
-            float t = 0.f;
-            for (int64_t i = lb + lane; i < le; i += 32) t += __ldg(y + __ldg(col + i));
+            constexpr int kS = 4;  // slabs in flight
+            for (int s0 = 0; s0 < total; s0 += 32 * kS) {
+                uint32_t c[kS];
+                int kk[kS];
+                float r[kS];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-            if (lane == src) s = t;
-        }
-        if (v < n) {
-            const float xv = base + damping * (s + dterm);
-            x_new[v] = xv;
-            y_new[v] = deg > 0 ? xv / (float)deg : 0.f;
-            if (deg == 0) dang += xv;
-            if (resid_part) res += fabs((double)xv - (double)__ldg(x + v));
-        }
-    }
-    // fixed-order reductions: lanes, then warps, per block
+                for (int q = 0; q < kS; ++q) {
+                    const int i = s0 + q * 32 + lane;
+                    int k = 0;  // the last row whose start is <= i
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        dang += __shfl_xor_sync(kFull, dang, o);
-        res += __shfl_xor_sync(kFull, res, o);
-    }
-    if (lane == 0) {
-        s_dang[warp] = dang;
-        s_res[warp] = res;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float bd = 0.f;
-        double br = 0.0;
-        for (int i = 0; i < kPrWarps; ++i) {
-            bd += s_dang[i];
-            br += s_res[i];
+                    for (int step = 16; step >= 1; step >>= 1) {
+                        const int sk = __shfl_sync(kFull, vs, k + step);
+                        if (sk <= i) k += step;
+                    }
+                    const int64_t bk = __shfl_sync(kFull, b, k);
+                    const int vk = __shfl_sync(kFull, vs, k);
+                    kk[q] = k;
+                    c[q] = i < total ? __ldcs(a.colx + bk + (i - vk)) : 0u;
+                    if (s0 + (q + 1) * 32 >= total) break;
+                }
+#pragma unroll
+                for (int q = 0; q < kS; ++q) {
+                    if (s0 + q * 32 >= total) break;
+                    r[q] = s0 + q * 32 + lane < total ? rank_of(c[q]) : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < kS; ++q) {
+                    if (s0 + q * 32 >= total) break;
+                    const int i = s0 + q * 32 + lane, k = kk[q];
+                    float val = r[q];
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const float t = __shfl_up_sync(kFull, val, o);
+                        const int kt = __shfl_up_sync(kFull, k, o);
+                        if (lane >= o && kt == k) val += t;
+                    }
+                    const int ka = __shfl_down_sync(kFull, k, 1);
+                    if (i < total && (lane == 31 || ka != k || i + 1 >= total)) s_acc[warp][k] += val;
+                    __syncwarp();
+                }
+            }
+            const float s = s_acc[warp][lane];
+            __syncwarp();
+            if (v < a.n && shortr) finish(v, deg, s);
         }
-        dangling_part[blockIdx.x] = bd;
-        if (resid_part) resid_part[blockIdx.x] = br;
+    }
+    if constexpr (S == PrStore::kLast) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(kFull, res, o);
+        if (lane == 0) s_res[warp] = res;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double br = 0.0;
+            for (int i = 0; i < kPrCta / 32; ++i) br += s_res[i];
+            a.resid_part[blockIdx.x] = br;
+        }
     }
 }
 
-// Hub rows (more than kHubRow arcs) are cut into chunks of kHubChunk arcs;
-// a CTA sums one chunk (threads stride it, then a fixed tree) into its slot.
-__global__ void __launch_bounds__(kPrThreads) pr_hub_kernel(const uint32_t *__restrict__ col,
-                                                            const float *__restrict__ y,
-                                                            const int64_t *__restrict__ chunk_begin,
-                                                            const int64_t *__restrict__ chunk_end,
-                                                            float *__restrict__ hub_part) {
-    __shared__ float s[kPrWarps];
-    const int64_t b = chunk_begin[blockIdx.x], e = chunk_end[blockIdx.x];
-    float t = 0.f;
-    for (int64_t i = b + threadIdx.x; i < e; i += kPrThreads) t += __ldg(y + __ldg(col + i));
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = t;
+// Hub rows and their chunk count, the rows of medium length (in whatever order
+// the atomics give), and the degree histogram.
+__global__ void __launch_bounds__(kPrThreads) pr_degrees_kernel(const int64_t *__restrict__ off, int64_t n, uint32_t *hubs,
+                                                               uint32_t *medium, unsigned long long *counts,
+                                                               unsigned int *hist) {
+    __shared__ unsigned int s_hist[kDegBuckets];
+    for (int i = threadIdx.x; i < kDegBuckets; i += blockDim.x) s_hist[i] = 0;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float acc = 0.f;
-        for (int w = 0; w < kPrWarps; ++w) acc += s[w];
-        hub_part[blockIdx.x] = acc;
-    }
-}
-
-// Hub rows and their chunk count (the list order is whatever the atomics give).
-__global__ void pr_find_hubs_kernel(const int64_t *__restrict__ off, int64_t n, uint32_t *hubs,
-                                    unsigned long long *counts) {
+    const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const int64_t deg = off[v + 1] - off[v];
+    for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x; v0 < n; v0 += stride) {
+        const int64_t v = v0 + threadIdx.x;
+        const int64_t deg = v < n ? off[v + 1] - off[v] : 0;
+        const bool med = deg > kShortRow && deg <= kHubRow;
+        const unsigned m = __ballot_sync(kFull, med);
+        unsigned long long base = 0;
+        if (lane == 0 && m) base = atomicAdd(counts + 2, (unsigned long long)__popc(m));
+        base = __shfl_sync(kFull, base, 0);
+        if (med) medium[base + __popc(m & lanemask_lt())] = (uint32_t)v;
         if (deg > kHubRow) {
             hubs[atomicAdd(counts, 1ull)] = (uint32_t)v;
             atomicAdd(counts + 1, (unsigned long long)((deg + kHubChunk - 1) / kHubChunk));
         }
+        if (v < n) atomicAdd(&s_hist[degree_bucket(deg)], 1u);
     }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kDegBuckets; i += blockDim.x)
+        if (s_hist[i]) atomicAdd(hist + i, s_hist[i]);
 }
 
-// One CTA: each hub's first chunk slot (a running block scan over the hub
-// list, 1024 hubs at a time) and the chunk bounds.
+// One CTA: each hub's first chunk (a running block scan over the hub list, 1024
+// hubs at a time) and the hub of every chunk; and the first position of every
+// degree bucket in y (in place of its count), largest degrees first.
 __global__ void __launch_bounds__(1024) pr_hub_chunks_kernel(const int64_t *__restrict__ off,
-                                                             const uint32_t *__restrict__ hubs, int num_hubs,
-                                                             int *hub_slot, int64_t *chunk_begin,
-                                                             int64_t *chunk_end) {
+                                                             const uint32_t *__restrict__ hubs,
+                                                             const unsigned long long *__restrict__ counts, int *first,
+                                                             uint32_t *chunk_hub, unsigned int *hist) {
     __shared__ int s_warp[32];
     __shared__ int s_run;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int num_hubs = (int)counts[0];
     if (threadIdx.x == 0) s_run = 0;
+    if (warp == 0) {  // the buckets' first positions, largest degrees first
+        constexpr int kPer = kDegBuckets / 32;
+        unsigned int cnt[kPer], sum = 0;
+        for (int i = 0; i < kPer; ++i) sum += cnt[i] = hist[kDegBuckets - 1 - (lane * kPer + i)];
+        unsigned int inc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned int t = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += t;
+        }
+        unsigned int run = inc - sum;
+        for (int i = 0; i < kPer; ++i) {
+            hist[kDegBuckets - 1 - (lane * kPer + i)] = run;
+            run += cnt[i];
+        }
+    }
     __syncthreads();
     for (int h0 = 0; h0 < num_hubs; h0 += 1024) {
         const int h = h0 + threadIdx.x;
-        int64_t b = 0, e = 0;
-        uint32_t v = 0;
         int nch = 0;
         if (h < num_hubs) {
-            v = hubs[h];
-            b = off[v];
-            e = off[v + 1];
-            nch = (int)((e - b + kHubChunk - 1) / kHubChunk);
+            const uint32_t v = hubs[h];
+            nch = (int)((off[v + 1] - off[v] + kHubChunk - 1) / kHubChunk);
         }
         int inc = nch;
 #pragma unroll
@@ -228,44 +474,87 @@ __global__ void __launch_bounds__(1024) pr_hub_chunks_kernel(const int64_t *__re
         __syncthreads();
         int slot = s_run + s_warp[warp] + inc - nch;
         if (h < num_hubs) {
-            hub_slot[v] = slot;
-            for (int64_t c = b; c < e; c += kHubChunk, ++slot) {
-                chunk_begin[slot] = c;
-                chunk_end[slot] = c + kHubChunk < e ? c + kHubChunk : e;
-            }
+            first[h] = slot;
+            for (int c = 0; c < nch; ++c) chunk_hub[slot + c] = (uint32_t)h;
         }
+        slot += nch;
         __syncthreads();
         if (threadIdx.x == 1023) s_run = slot;  // the last thread's next slot is the running total
         __syncthreads();
     }
 }
 
-// x0 = 1/n, y0 = x0/d, per-block dangling mass of x0
-__global__ void __launch_bounds__(kPrThreads) pr_init_kernel(const int64_t *__restrict__ off, int64_t n, float x0,
-                                                             float *__restrict__ x, float *__restrict__ y,
-                                                             float *__restrict__ dangling_part) {
-    __shared__ float s_dang[kPrWarps];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float dang = 0.f;
-    const int64_t nwarps = (int64_t)gridDim.x * kPrWarps;
-    for (int64_t r0 = ((int64_t)blockIdx.x * kPrWarps + warp) * 32; r0 < n; r0 += nwarps * 32) {
-        const int64_t v = r0 + lane;
-        if (v < n) {
-            const int64_t deg = __ldg(off + v + 1) - __ldg(off + v);
-            x[v] = x0;
-            y[v] = deg > 0 ? x0 / (float)deg : 0.f;
-            if (deg == 0) dang += x0;
-        }
-    }
+// Positions in y, by falling degree bucket (in any order inside one: the
+// values move with them, the sums don't change).  A CTA counts a tile of
+// vertices by bucket and takes its places with one atomic per bucket.
+__global__ void __launch_bounds__(kPrThreads) pr_positions_kernel(const int64_t *__restrict__ off, int64_t n,
+                                                                 unsigned int *next, uint32_t *__restrict__ pos) {
+    constexpr int kPer = 8;
+    __shared__ unsigned int s_cnt[kDegBuckets], s_base[kDegBuckets];
+    const int64_t stride = (int64_t)gridDim.x * kPrThreads * kPer;
+    for (int64_t v0 = (int64_t)blockIdx.x * kPrThreads * kPer; v0 < n; v0 += stride) {
+        for (int i = threadIdx.x; i < kDegBuckets; i += kPrThreads) s_cnt[i] = 0;
+        __syncthreads();
+        int bucket[kPer];
+        unsigned int rank[kPer];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dang += __shfl_xor_sync(kFull, dang, o);
-    if (lane == 0) s_dang[warp] = dang;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float bd = 0.f;
-        for (int i = 0; i < kPrWarps; ++i) bd += s_dang[i];
-        dangling_part[blockIdx.x] = bd;
+        for (int j = 0; j < kPer; ++j) {
+            const int64_t v = v0 + j * kPrThreads + threadIdx.x;
+            if (v < n) {
+                bucket[j] = degree_bucket(off[v + 1] - off[v]);
+                rank[j] = atomicAdd(&s_cnt[bucket[j]], 1u);
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kDegBuckets; i += kPrThreads)
+            if (s_cnt[i]) s_base[i] = atomicAdd(next + i, s_cnt[i]);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int64_t v = v0 + j * kPrThreads + threadIdx.x;
+            if (v < n) pos[v] = s_base[bucket[j]] + rank[j];
+        }
+        __syncthreads();
     }
+}
+
+__global__ void __launch_bounds__(kPrThreads) pr_heads_kernel(const uint32_t *__restrict__ col, int64_t nnz,
+                                                             const uint32_t *__restrict__ pos,
+                                                             uint32_t *__restrict__ colx) {
+    constexpr int kPer = 8;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * kPer;
+    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x * kPer + threadIdx.x; i0 < nnz; i0 += stride) {
+        uint32_t c[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) c[j] = i0 + j * kPrThreads < nnz ? __ldg(col + i0 + j * kPrThreads) : 0u;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) c[j] = __ldg(pos + c[j]);
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+            if (i0 + j * kPrThreads < nnz) colx[i0 + j * kPrThreads] = c[j];
+    }
+}
+
+// y0 = x0/d, x0 itself when the first iteration is the last, and the degree-0
+// vertices of every virtual lane: virtual warp w sums the rows w * 32 + lane,
+// then those a whole virtual grid further, and so on.
+__global__ void __launch_bounds__(kPrThreads) pr_init_kernel(PrArgs a, float x0, bool store_x, uint32_t *lane_cnt) {
+    const int64_t stride = (int64_t)a.vblocks * kPrThreads;
+    const int64_t l = (int64_t)blockIdx.x * kPrThreads + threadIdx.x;  // grid: vblocks
+    uint32_t cnt = 0;
+    for (int64_t v = l; v < a.n; v += stride) {
+        const int64_t deg = __ldg(a.off + v + 1) - __ldg(a.off + v);
+        if (deg > 0) a.y_new[a.pos ? __ldg(a.pos + v) : (uint32_t)v] = x0 / (float)deg;
+        else ++cnt;
+        if (store_x) a.x_prev[v] = x0;
+    }
+    lane_cnt[l] = cnt;
+    const int lane = threadIdx.x & 31;
+    float t = 0.f;
+    for (uint32_t k = cnt; k > 0; --k) t += x0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kFull, t, o);
+    if (lane == 0) a.wsum_new[l >> 5] = t;
 }
 
 // one block: sum the per-block partials in a fixed order
@@ -284,106 +573,139 @@ __global__ void __launch_bounds__(kPrThreads) reduce_parts_kernel(const T *__res
     if (threadIdx.x == 0) out[0] = s[0];
 }
 
+// Iterations that pay for the positions and the translated heads: they take
+// 0.66 ms on R-MAT s22 and save about 0.2 ms an iteration.
+constexpr int kPrMinIters = 4;
+
 sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_out, double *resid) {
-    const int64_t n = g->n;
+    const int64_t n = g->n, nnz = g->nnz;
     *resid = 0.0;
     if (n == 0) return SG_OK;
-    const int blocks = (int)std::min<int64_t>((n + kPrThreads - 1) / kPrThreads, (int64_t)c->num_sms * 8);
-    float *buf = nullptr;
-    // x_a, y_a, x_b, y_b, dangling partials, dangling total
+    const int vblocks = (int)std::min<int64_t>((n + kPrThreads - 1) / kPrThreads, (int64_t)c->num_sms * 8);
     const size_t nn = (size_t)n;
-    sg_status st = dalloc(c, (void **)&buf, sizeof(float) * (4 * nn + (size_t)blocks + 4));
-    double *dres = nullptr;
-    if (st == SG_OK) st = dalloc(c, (void **)&dres, sizeof(double) * ((size_t)blocks + 1));
-    if (st != SG_OK) {
+    PrArgs a{};
+    a.off = g->off;
+    a.colx = g->col;
+    a.n = n;
+    a.base = (float)((1.0 - (double)damping) / (double)n);
+    a.damping = damping;
+    a.inv_n = (float)(1.0 / (double)n);
+    a.vblocks = vblocks;
+    a.x_out = x_out;
+    // one allocation: the arrays below, each aligned to 256 bytes
+    const size_t max_hubs = (size_t)(nnz / kHubRow + 1), max_chunks = (size_t)(nnz / kHubChunk) + max_hubs;
+    const int hot_cap = (int)std::min<int64_t>(kPrHot, n);
+    size_t total = 0;
+    auto room = [&](size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t grid_max = (size_t)c->num_sms;
+    const size_t zero_at = room((4 + kDegBuckets / 2 + 1) * sizeof(unsigned long long));  // counts, hist, work
+    const size_t done_at = room(max_hubs * sizeof(unsigned int));
+    const size_t zero_end = total;
+    const size_t y_at[2] = {room(sizeof(float) * (nn + 4)), room(sizeof(float) * (nn + 4))};
+    const size_t x_at = room(sizeof(float) * nn), res_at = room(sizeof(double) * (grid_max + 1));
+    const size_t cnt_at = room(sizeof(uint32_t) * (size_t)vblocks * kPrThreads);
+    const size_t w_at[2] = {room(sizeof(float) * (size_t)vblocks * kPrWarps), room(sizeof(float) * (size_t)vblocks * kPrWarps)};
+    const size_t hubs_at = room(sizeof(uint32_t) * max_hubs), first_at = room(sizeof(int) * max_hubs);
+    const size_t med_at = room(sizeof(uint32_t) * (size_t)(nnz / kShortRow + 1));
+    const size_t chunk_at = room(sizeof(uint32_t) * max_chunks), part_at = room(sizeof(float) * max_chunks);
+    char *buf = nullptr;
+    uint32_t *pos = nullptr, *colx = nullptr;
+    sg_status st = dalloc(c, (void **)&buf, total);
+    if (st != SG_OK) return st;
+    // positions and translated heads: 4 (n + nnz) bytes, without which y stays in vertex order
+    bool hot = iters >= kPrMinIters && nnz > 0;
+    if (hot && (dalloc(c, (void **)&pos, sizeof(uint32_t) * nn) != SG_OK ||
+                dalloc(c, (void **)&colx, sizeof(uint32_t) * (size_t)nnz) != SG_OK)) {
+        set_error("");
+        dfree(c, pos);
+        pos = nullptr;
+        hot = false;
+    }
+    unsigned long long *counts = reinterpret_cast<unsigned long long *>(buf + zero_at);
+    unsigned int *hist = reinterpret_cast<unsigned int *>(counts + 4), *work = hist + kDegBuckets;
+    a.hubs = PrHubs{reinterpret_cast<uint32_t *>(buf + hubs_at), counts, reinterpret_cast<int *>(buf + first_at),
+                    reinterpret_cast<uint32_t *>(buf + chunk_at), reinterpret_cast<float *>(buf + part_at),
+                    reinterpret_cast<unsigned int *>(buf + done_at)};
+    a.medium = reinterpret_cast<uint32_t *>(buf + med_at);
+    a.x_prev = reinterpret_cast<float *>(buf + x_at);
+    a.resid_part = reinterpret_cast<double *>(buf + res_at);
+    a.lane_cnt = reinterpret_cast<uint32_t *>(buf + cnt_at);
+    a.hot = hot ? hot_cap : 0;
+    a.pos = pos;
+    float *y[2] = {reinterpret_cast<float *>(buf + y_at[0]), reinterpret_cast<float *>(buf + y_at[1])};
+    float *w[2] = {reinterpret_cast<float *>(buf + w_at[0]), reinterpret_cast<float *>(buf + w_at[1])};
+    auto release = [&]() {
+        dfree(c, colx);
+        dfree(c, pos);
         dfree(c, buf);
-        return st;
+    };
+    cudaError_t e = cudaMemsetAsync(buf + zero_at, 0, zero_end - zero_at, c->stream);
+    {
+        SG_LAUNCH(c, "pr_setup");
+        pr_degrees_kernel<<<vblocks, kPrThreads, 0, c->stream>>>(g->off, n, const_cast<uint32_t *>(a.hubs.row),
+                                                                const_cast<uint32_t *>(a.medium), counts, hist);
     }
-    float *xa = buf, *ya = buf + nn, *xb = buf + 2 * nn, *yb = buf + 3 * nn;
-    float *dpart = buf + 4 * nn, *dtot = dpart + blocks;
-    const float inv_n = (float)(1.0 / (double)n);
-    const float base = (float)((1.0 - (double)damping) / (double)n);
-    // hub rows: list them once, then their chunks are summed before every iteration
-    uint32_t *hubs = nullptr;
-    unsigned long long *hcnt = nullptr;
-    int *hub_slot = nullptr;
-    int64_t *chunk_b = nullptr, *chunk_e = nullptr;
-    float *hub_part = nullptr;
-    int64_t num_hubs = 0, num_chunks = 0;
-    st = dalloc(c, (void **)&hcnt, 2 * sizeof(unsigned long long));
-    if (st == SG_OK) st = dalloc(c, (void **)&hubs, sizeof(uint32_t) * nn);
-    if (st == SG_OK && cudaMemsetAsync(hcnt, 0, 2 * sizeof(unsigned long long), c->stream) != cudaSuccess)
-        st = cuda_fail(cudaGetLastError(), "cudaMemsetAsync");
-    if (st == SG_OK) {
-        SG_LAUNCH(c, "pr_hubs");
-        pr_find_hubs_kernel<<<blocks, kPrThreads, 0, c->stream>>>(g->off, n, hubs, hcnt);
-        if (cudaMemcpyAsync(c->h_pinned, hcnt, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream) !=
-                cudaSuccess ||
-            cudaStreamSynchronize(c->stream) != cudaSuccess)
-            st = cuda_fail(cudaGetLastError(), "PageRank hub count");
-        num_hubs = c->h_pinned[0];
-        num_chunks = c->h_pinned[1];
+    {
+        SG_LAUNCH(c, "pr_setup");
+        pr_hub_chunks_kernel<<<1, 1024, 0, c->stream>>>(g->off, a.hubs.row, counts, const_cast<int *>(a.hubs.first),
+                                                        const_cast<uint32_t *>(a.hubs.chunk_hub), hist);
     }
-    if (st == SG_OK && num_hubs > 0) {
-        st = dalloc(c, (void **)&hub_slot, sizeof(int) * nn);
-        if (st == SG_OK) st = dalloc(c, (void **)&chunk_b, sizeof(int64_t) * (size_t)num_chunks);
-        if (st == SG_OK) st = dalloc(c, (void **)&chunk_e, sizeof(int64_t) * (size_t)num_chunks);
-        if (st == SG_OK) st = dalloc(c, (void **)&hub_part, sizeof(float) * (size_t)num_chunks);
-        if (st == SG_OK) {
-            SG_LAUNCH(c, "pr_hubs");
-            pr_hub_chunks_kernel<<<1, 1024, 0, c->stream>>>(g->off, hubs, (int)num_hubs, hub_slot, chunk_b, chunk_e);
+    if (hot) {
+        {
+            SG_LAUNCH(c, "pr_setup");
+            pr_positions_kernel<<<vblocks, kPrThreads, 0, c->stream>>>(g->off, n, hist, pos);
         }
+        SG_LAUNCH(c, "pr_setup");
+        const int64_t hb = std::min<int64_t>((nnz + kPrThreads * 8 - 1) / (kPrThreads * 8), (int64_t)c->num_sms * 8);
+        pr_heads_kernel<<<(unsigned)hb, kPrThreads, 0, c->stream>>>(g->col, nnz, pos, colx);
+        a.colx = colx;
     }
-    if (st != SG_OK) {
-        dfree(c, hubs); dfree(c, hcnt); dfree(c, hub_slot); dfree(c, chunk_b); dfree(c, chunk_e); dfree(c, hub_part);
-        dfree(c, buf); dfree(c, dres);
-        return st;
-    }
+    a.y_new = y[0];
+    a.wsum_new = w[0];
     {
         SG_LAUNCH(c, "pr_init");
-        pr_init_kernel<<<blocks, kPrThreads, 0, c->stream>>>(g->off, n, inv_n, xa, ya, dpart);
+        pr_init_kernel<<<vblocks, kPrThreads, 0, c->stream>>>(a, a.inv_n, iters == 1, const_cast<uint32_t *>(a.lane_cnt));
     }
-    {
-        SG_LAUNCH(c, "pr_reduce");
-        reduce_parts_kernel<float><<<1, kPrThreads, 0, c->stream>>>(dpart, blocks, dtot);
+    const int64_t groups = (n + 31) / 32;
+    const int grid = (int)std::min<int64_t>(std::max<int64_t>(groups, nnz / kHubChunk), (int64_t)c->num_sms);
+    a.per_claim = (int)std::max<int64_t>(1, std::min<int64_t>(4, groups / ((int64_t)grid * 32 * 8)));
+    const size_t smem = hot ? sizeof(float) * (((size_t)hot_cap + 3) / 4 * 4) : 0;
+    void (*k[2][3])(PrArgs) = {{pr_iter_kernel<false, PrStore::kNone>, pr_iter_kernel<false, PrStore::kPrev>,
+                                pr_iter_kernel<false, PrStore::kLast>},
+                               {pr_iter_kernel<true, PrStore::kNone>, pr_iter_kernel<true, PrStore::kPrev>,
+                                pr_iter_kernel<true, PrStore::kLast>}};
+    for (int i = 0; i < 3 && hot && e == cudaSuccess; ++i)
+        e = cudaFuncSetAttribute(k[1][i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) {
+        release();
+        return cuda_fail(e, "PageRank setup");
     }
     for (int it = 0; it < iters; ++it) {
-        const bool last = (it == iters - 1);
-        float *xo = last ? x_out : xb;
-        if (num_chunks > 0) {
-            SG_LAUNCH(c, "pr_hub");
-            pr_hub_kernel<<<(unsigned)num_chunks, kPrThreads, 0, c->stream>>>(g->col, ya, chunk_b, chunk_e, hub_part);
-        }
-        {
-            SG_LAUNCH(c, "pr_iter");
-            pr_iter_kernel<<<blocks, kPrThreads, 0, c->stream>>>(g->off, g->col, n, xa, ya, dtot, base, damping, inv_n,
-                                                                 xo, yb, dpart, last ? dres : nullptr, hub_slot,
-                                                                 hub_part);
-        }
-        if (!last) {
-            SG_LAUNCH(c, "pr_reduce");
-            reduce_parts_kernel<float><<<1, kPrThreads, 0, c->stream>>>(dpart, blocks, dtot);
-        }
-        std::swap(xa, xb);
-        std::swap(ya, yb);
+        const int in = it & 1, s = it == iters - 1 ? 2 : (it == iters - 2 ? 1 : 0);
+        a.y = y[in];
+        a.y_new = y[in ^ 1];
+        a.wsum = w[in];
+        a.wsum_new = w[in ^ 1];
+        a.work = work + in;
+        a.work_next = work + (in ^ 1);
+        SG_LAUNCH(c, "pr_iter");
+        k[hot][s]<<<grid, kPrCta, smem, c->stream>>>(a);
     }
     {
         SG_LAUNCH(c, "pr_reduce");
-        reduce_parts_kernel<double><<<1, kPrThreads, 0, c->stream>>>(dres, blocks, dres + blocks);
+        reduce_parts_kernel<double><<<1, kPrThreads, 0, c->stream>>>(a.resid_part, grid, a.resid_part + grid_max);
     }
-    SG_CUDA(cudaGetLastError());
-    SG_CUDA(cudaMemcpyAsync(c->h_pinned, dres + blocks, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    SG_CUDA(cudaStreamSynchronize(c->stream));
-    std::memcpy(resid, c->h_pinned, sizeof(double));
-    dfree(c, hubs);
-    dfree(c, hcnt);
-    dfree(c, hub_slot);
-    dfree(c, chunk_b);
-    dfree(c, chunk_e);
-    dfree(c, hub_part);
-    dfree(c, buf);
-    dfree(c, dres);
-    return SG_OK;
+    e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->h_pinned, a.resid_part + grid_max, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e == cudaSuccess) std::memcpy(resid, c->h_pinned, sizeof(double));
+    release();
+    return e == cudaSuccess ? SG_OK : cuda_fail(e, "PageRank");
 }
 
 // ---------------------------------------------------------------------- KL

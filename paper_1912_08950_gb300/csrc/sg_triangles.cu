@@ -117,6 +117,7 @@ struct TriArgs {
     int64_t n_heavy;
     int heavy_cap;               // entries of the phase-1 table; larger N+(u) go in chunks
     int light_max;               // out-degrees up to this go to the warp-per-vertex phase
+    int light_claim;             // vertices a warp claims at a time in the light phase (at most 32)
     int short_max;               // union passes: lists up to this long are always streamed whole
     const uint2 *vrec;           // off+ and d+ of vertex v at entry v * vstep
     int vstep;                   // 1, or 2: the first halves of the records arec
@@ -721,13 +722,13 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tr
         Table tb{reinterpret_cast<uint32_t *>(tbl) + warp * kLightSlots, s_stash[warp], &s_stash_n[warp]};
         for (;;) {
             unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(a.work + 1, 32ull);
+            if (lane == 0) base = atomicAdd(a.work + 1, (unsigned long long)a.light_claim);
             base = __shfl_sync(kFull, base, 0);
             if ((int64_t)base >= a.n) break;
             const int64_t ul = (int64_t)base + lane;
             uint32_t oul = 0;
             int dl = 0, nl = 0;
-            if (ul < a.n) {
+            if (lane < a.light_claim && ul < a.n) {
                 const int64_t o0 = __ldg(a.offp + ul);
                 oul = (uint32_t)o0;
                 dl = (int)(__ldg(a.offp + ul + 1) - o0);
@@ -1275,13 +1276,13 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? 4 : 1) tri_union_kernel(T
         t.tb = Table{own, s_stash[warp], &s_stash_n[warp], s_dead[warp], own + 4 * kUnionLightMax};
         for (;;) {
             unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(a.work + 1, 32ull);
+            if (lane == 0) base = atomicAdd(a.work + 1, (unsigned long long)a.light_claim);
             base = __shfl_sync(kFull, base, 0);
             if ((int64_t)base >= a.n) break;
             const int64_t ul = (int64_t)base + lane;
             uint32_t oul = 0;
             int dl = 0, nl = 0;
-            if (ul < a.n) {
+            if (lane < a.light_claim && ul < a.n) {
                 const int64_t o0 = __ldg(a.offp + ul);
                 oul = (uint32_t)o0;
                 dl = (int)(__ldg(a.offp + ul + 1) - o0);
@@ -1776,15 +1777,21 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
 // claim their vertices through the work counters.
 static sg_status launch_tri(Ctx *c, void (*kernel)(TriArgs), int threads, size_t smem, const TriArgs &a,
                             const char *name, int grid_per_sm = 0) {
+    TriArgs args = a;
     SG_CUDA(cudaMemsetAsync(a.work, 0, 2 * sizeof(unsigned long long), c->stream));
     SG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     per_sm = std::max(per_sm, 1);
     if (grid_per_sm > 0) per_sm = std::min(per_sm, grid_per_sm);
+    // a light vertex takes some 10 us of one warp: on a small graph claims of 32
+    // would leave most warps idle (n = 1000: 32 warps of 4864 busy, 283 us),
+    // so a warp claims what gives every warp about four turns
+    const int64_t warps = (int64_t)c->num_sms * per_sm * (threads / 32);
+    args.light_claim = (int)std::max<int64_t>(1, std::min<int64_t>(32, a.n / (warps * 4)));
     {
         SG_LAUNCH(c, name);
-        kernel<<<(unsigned)(c->num_sms * per_sm), threads, smem, c->stream>>>(a);
+        kernel<<<(unsigned)(c->num_sms * per_sm), threads, smem, c->stream>>>(args);
     }
     SG_CUDA(cudaGetLastError());
     return SG_OK;

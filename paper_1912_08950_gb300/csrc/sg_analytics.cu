@@ -14,8 +14,10 @@
 // the rows of vertices outside it link their remaining neighbours (an edge
 // leaving the giant component is seen from its other end).
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "sg_internal.cuh"
@@ -36,9 +38,9 @@ constexpr int kPrWarps = kPrThreads / 32;
 // vertices, the heads of 54% of the arcs) to shared memory when an iteration
 // starts; the L1 keeps the next ones, which share lines.  The heads stream past
 // it (evict-first).  One CTA of 32 warps per SM, eight slabs of 32 arcs in
-// flight per warp.  Per iteration on R-MAT s22 (128 M arcs) 358 us, against 634
-// with y in vertex order and launches of their own for hub rows and D; s20: 92
-// against 172.  Half of the L1 for y is where the line lies: 373 us at 32 K
+// flight per warp.  Per iteration on R-MAT s22 (128 M arcs) 339 us, against 634
+// with y in vertex order and launches of their own for hub rows and D; s20: 88
+// against 172; n = 60,000: 20 against 47.  Half of the L1 for y is where the line lies: 373 us at 32 K
 // entries before the heads were streamed, 403 at 16 K, 387 at 24 K and 389 at
 // 40 K; 54 K entries (all of the shared memory) leave too few lines: 588.
 //
@@ -69,8 +71,8 @@ struct PrHubs {
     const unsigned long long *count;  // [0] hubs, [1] chunks, [2] rows of medium length
     const int *first;           // first chunk of hub h
     const uint32_t *chunk_hub;  // hub of chunk c
-    float *part;                // chunk sums
-    unsigned int *done;         // chunks of hub h summed in this iteration (0 between iterations)
+    float *part;                // sums of the chunks, or of their runs
+    unsigned int *done;         // ... of hub h that are there in this iteration (0 between iterations)
 };
 
 struct PrArgs {
@@ -139,6 +141,7 @@ template <bool kHot, PrStore S>
 __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
     extern __shared__ float s_y[];
     __shared__ float s_acc[kPrCta / 32][32];
+    __shared__ longlong2 s_row[kPrCta / 32][32];  // first arc minus its number, and the row, of the short rows
     __shared__ float s_red[kPrThreads];
     __shared__ double s_res[kPrCta / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -170,70 +173,116 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
             a.y_new[a.pos ? __ldg(a.pos + v) : (uint32_t)v] = xv / (float)deg;
         }
     };
-    // units, the longest first: chunks of hub rows, 32 rows of medium length,
-    // groups of 32 consecutive rows for their short ones
+    // units, the longest first: chunks of hub rows, rows of medium length,
+    // groups of 32 consecutive rows for their short ones.  With few chunks (or
+    // medium rows) for the warps there are, a unit is one of a chunk's eight
+    // runs (or fewer than 32 rows): one warp's walk over 8192 arcs takes 30 us,
+    // most of an iteration on a small graph (R-MAT with 60,000 vertices: 54 us
+    // an iteration with whole units, 20 with these; with the runs split up to
+    // four times as many chunks, s20 takes 129 us instead of 92).
+    const unsigned warps = gridDim.x * (kPrCta / 32);
     const unsigned nchunks = (unsigned)a.hubs.count[1];
-    const unsigned nmed = (unsigned)a.hubs.count[2], med_units = (nmed + 31) / 32;
+    const bool split = nchunks < warps / 4;
+    const unsigned hub_units = split ? nchunks * kPrWarps : nchunks;
+    const unsigned nmed = (unsigned)a.hubs.count[2];
+    const unsigned med_rows = max(1u, min(32u, 2 * nmed / warps));
+    const unsigned med_units = (nmed + med_rows - 1) / med_rows;
     const unsigned groups = (unsigned)((a.n + 31) / 32);
-    const unsigned units = nchunks + med_units + (groups + a.per_claim - 1) / a.per_claim;
+    const unsigned units = hub_units + med_units + (groups + a.per_claim - 1) / a.per_claim;
     constexpr int kB = 8;  // slabs in flight
     for (;;) {
         unsigned u = 0;
         if (lane == 0) u = atomicAdd(a.work, 1u);
         u = __shfl_sync(kFull, u, 0);
         if (u >= units) break;
-        if (u < nchunks) {  // one chunk of a hub row
-            const uint32_t h = __ldg(a.hubs.chunk_hub + u);
+        if (u < hub_units) {  // one chunk of a hub row, or one run of it
+            const unsigned chunk = split ? u / kPrWarps : u;
+            const uint32_t h = __ldg(a.hubs.chunk_hub + chunk);
             const int first = __ldg(a.hubs.first + h);
             const int64_t v = __ldg(a.hubs.row + h);
             const int64_t rb = __ldg(a.off + v), re = __ldg(a.off + v + 1);
-            const int64_t cb = rb + (int64_t)((int)u - first) * kHubChunk;
+            const int64_t cb = rb + (int64_t)((int)chunk - first) * kHubChunk;
             const int64_t ce = min(cb + (int64_t)kHubChunk, re);
             static_assert(kB == kPrWarps, "a step of a chunk is one slab of each run");
-            float t[kB];
-            uint32_t c[kB];
-            auto load = [&](int64_t i) {
+            // a step: one slab of each of the eight runs, or eight of the unit's run
+            auto sum_part = [&](int64_t from, auto next_slab, auto next_step, auto add) {
+                uint32_t c[kB];
+                auto load = [&](int64_t i) {
 #pragma unroll
-                for (int w = 0; w < kB; ++w) c[w] = i + w * 32 < ce ? __ldcs(a.colx + i + w * 32) : 0u;
+                    for (int w = 0; w < kB; ++w) c[w] = i + w * next_slab < ce ? __ldcs(a.colx + i + w * next_slab) : 0u;
+                };
+                load(from);
+                for (int64_t i = from; i - lane < ce; i += next_step) {
+                    float r[kB];
+#pragma unroll
+                    for (int w = 0; w < kB; ++w) {
+                        r[w] = 0.f;
+                        if (i + w * next_slab < ce) r[w] = rank_of(c[w]);
+                    }
+                    load(i + next_step);  // the next step's, while these are on their way
+#pragma unroll
+                    for (int w = 0; w < kB; ++w) add(w, r[w]);
+                }
             };
-#pragma unroll
-            for (int w = 0; w < kB; ++w) t[w] = 0.f;
-            load(cb + lane);
-            for (int64_t i = cb + lane; i - lane < ce; i += kPrThreads) {
-                float r[kB];
-#pragma unroll
-                for (int w = 0; w < kB; ++w) r[w] = i + w * 32 < ce ? rank_of(c[w]) : 0.f;
-                load(i + kPrThreads);  // the next step's, while these are on their way
-#pragma unroll
-                for (int w = 0; w < kB; ++w) t[w] += r[w];
-            }
             float acc = 0.f;
+            if (split) {
+                sum_part(cb + lane + (u % kPrWarps) * 32, std::integral_constant<int, kPrThreads>{},
+                         std::integral_constant<int, kPrThreads * kB>{}, [&](int, float r) { acc += r; });
 #pragma unroll
-            for (int w = 0; w < kB; ++w) {
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+            } else {
+                float t[kB];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) t[w] += __shfl_xor_sync(kFull, t[w], o);
-                acc += t[w];
+                for (int w = 0; w < kB; ++w) t[w] = 0.f;
+                sum_part(cb + lane, std::integral_constant<int, 32>{}, std::integral_constant<int, kPrThreads>{},
+                         [&](int w, float r) { t[w] += r; });
+#pragma unroll
+                for (int w = 0; w < kB; ++w) {
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) t[w] += __shfl_xor_sync(kFull, t[w], o);
+                    acc += t[w];
+                }
             }
+            // the warp that sums the row's last part adds the parts in order
+            const int parts = (int)((re - rb + kHubChunk - 1) / kHubChunk) * (split ? kPrWarps : 1);
+            bool last = false;
             if (lane == 0) {
-                const int nch = (int)((re - rb + kHubChunk - 1) / kHubChunk);
                 __stcg(a.hubs.part + u, acc);
                 __threadfence();
-                if (atomicAdd(a.hubs.done + h, 1u) == (unsigned)nch - 1) {  // the row's last chunk
-                    __threadfence();
-                    float s = 0.f;
-                    for (int c2 = 0; c2 < nch; ++c2) s += __ldcg(a.hubs.part + first + c2);
+                last = atomicAdd(a.hubs.done + h, 1u) == (unsigned)parts - 1;
+                __threadfence();
+            }
+            if (__shfl_sync(kFull, (int)last, 0)) {
+                const float *part = a.hubs.part + (size_t)first * (split ? kPrWarps : 1);
+                float s = 0.f, one = 0.f;  // the row's sum, a chunk's
+                for (int p0 = 0; p0 < parts; p0 += 32) {
+                    const float x = p0 + lane < parts ? __ldcg(part + p0 + lane) : 0.f;
+                    for (int j = 0; j < min(32, parts - p0); ++j) {
+                        const float y = __shfl_sync(kFull, x, j);
+                        if (split) {
+                            one += y;
+                            if ((j & (kPrWarps - 1)) == kPrWarps - 1) {
+                                s += one;
+                                one = 0.f;
+                            }
+                        } else {
+                            s += y;
+                        }
+                    }
+                }
+                if (lane == 0) {
                     a.hubs.done[h] = 0;
                     finish(v, re - rb, s);
                 }
             }
             continue;
         }
-        u -= nchunks;
+        u -= hub_units;
         if (u < med_units) {
             // a row per lane; the rows' slabs of 32 arcs as one sequence, kB of them in flight
-            const unsigned mi = u * 32 + lane;
+            const unsigned mi = u * med_rows + lane;
             int64_t v = -1, b = 0, e = 0;
-            if (mi < nmed) {
+            if (lane < med_rows && mi < nmed) {
                 v = __ldg(a.medium + mi);
                 b = __ldg(a.off + v);
                 e = __ldg(a.off + v + 1);
@@ -327,45 +376,48 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
             const int total = __shfl_sync(kFull, vs, 31);
             vs -= sdeg;  // exclusive start of this row's arcs
             s_acc[warp][lane] = 0.f;
+            const unsigned full = __ballot_sync(kFull, sdeg > 0);
+            const int start = sdeg > 0 ? vs : INT_MIN;
+            if (sdeg > 0) s_row[warp][__popc(full & lanemask_lt())] = make_longlong2(b - vs, lane);
             __syncwarp();
             constexpr int kS = 4;  // slabs in flight
+            const unsigned le = lanemask_lt() | (1u << lane);
+            int before = -1;  // rows that start before the slab, minus one
             for (int s0 = 0; s0 < total; s0 += 32 * kS) {
                 uint32_t c[kS];
-                int kk[kS];
+                unsigned starts[kS];  // lanes of the slab where a row starts
+                int row[kS];
                 float r[kS];
 #pragma unroll
                 for (int q = 0; q < kS; ++q) {
                     const int i = s0 + q * 32 + lane;
-                    int k = 0;  // the last row whose start is <= i
-#pragma unroll
-                    for (int step = 16; step >= 1; step >>= 1) {
-                        const int sk = __shfl_sync(kFull, vs, k + step);
-                        if (sk <= i) k += step;
-                    }
-                    const int64_t bk = __shfl_sync(kFull, b, k);
-                    const int vk = __shfl_sync(kFull, vs, k);
-                    kk[q] = k;
-                    c[q] = i < total ? __ldcs(a.colx + bk + (i - vk)) : 0u;
-                    if (s0 + (q + 1) * 32 >= total) break;
+                    const unsigned rel = (unsigned)start - (unsigned)(s0 + q * 32);
+                    starts[q] = __reduce_or_sync(kFull, rel < 32u ? 1u << rel : 0u);
+                    const longlong2 at = s_row[warp][(before + __popc(starts[q] & le)) & 31];
+                    before += __popc(starts[q]);
+                    row[q] = (int)at.y;
+                    c[q] = i < total ? __ldcs(a.colx + at.x + i) : 0u;
                 }
 #pragma unroll
                 for (int q = 0; q < kS; ++q) {
-                    if (s0 + q * 32 >= total) break;
-                    r[q] = s0 + q * 32 + lane < total ? rank_of(c[q]) : 0.f;
+                    r[q] = 0.f;
+                    if (s0 + q * 32 + lane < total) r[q] = rank_of(c[q]);
                 }
 #pragma unroll
                 for (int q = 0; q < kS; ++q) {
-                    if (s0 + q * 32 >= total) break;
-                    const int i = s0 + q * 32 + lane, k = kk[q];
+                    if (s0 + q * 32 >= total) break;  // warp-uniform
+                    // lanes since the row's start in this slab
+                    const unsigned m = starts[q] & le;
+                    const int d = m ? lane - (31 - __clz((int)m)) : lane;
                     float val = r[q];
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
                         const float t = __shfl_up_sync(kFull, val, o);
-                        const int kt = __shfl_up_sync(kFull, k, o);
-                        if (lane >= o && kt == k) val += t;
+                        if (d >= o) val += t;
                     }
-                    const int ka = __shfl_down_sync(kFull, k, 1);
-                    if (i < total && (lane == 31 || ka != k || i + 1 >= total)) s_acc[warp][k] += val;
+                    const int i = s0 + q * 32 + lane;
+                    if (i < total && (lane == 31 || ((starts[q] >> (lane + 1)) & 1u) || i + 1 >= total))
+                        s_acc[warp][row[q]] += val;
                     __syncwarp();
                 }
             }
@@ -611,7 +663,7 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     const size_t w_at[2] = {room(sizeof(float) * (size_t)vblocks * kPrWarps), room(sizeof(float) * (size_t)vblocks * kPrWarps)};
     const size_t hubs_at = room(sizeof(uint32_t) * max_hubs), first_at = room(sizeof(int) * max_hubs);
     const size_t med_at = room(sizeof(uint32_t) * (size_t)(nnz / kShortRow + 1));
-    const size_t chunk_at = room(sizeof(uint32_t) * max_chunks), part_at = room(sizeof(float) * max_chunks);
+    const size_t chunk_at = room(sizeof(uint32_t) * max_chunks), part_at = room(sizeof(float) * max_chunks * kPrWarps);
     char *buf = nullptr;
     uint32_t *pos = nullptr, *colx = nullptr;
     sg_status st = dalloc(c, (void **)&buf, total);

@@ -730,8 +730,10 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
                                 pr_iter_kernel<false, PrStore::kLast>},
                                {pr_iter_kernel<true, PrStore::kNone>, pr_iter_kernel<true, PrStore::kPrev>,
                                 pr_iter_kernel<true, PrStore::kLast>}};
+    // the limit is the function's, shared by all threads and contexts: always the
+    // same value, never this call's
     for (int i = 0; i < 3 && hot && e == cudaSuccess; ++i)
-        e = cudaFuncSetAttribute(k[1][i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(k[1][i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * kPrHot));
     if (e != cudaSuccess) {
         release();
         return cuda_fail(e, "PageRank setup");

@@ -1773,13 +1773,25 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
     return SG_OK;
 }
 
+// Dynamic shared memory of a CTA of `warps` warps with tables of up to `cap`
+// entries: the larger of the counting and edge-once passes' and the union passes'.
+static int max_smem(int warps, int cap) {
+    const size_t enumeration = sizeof(HitQueue) * warps + (size_t)cap * (6 * sizeof(uint32_t) + sizeof(unsigned short));
+    const size_t light = warps == kTW ? (size_t)kTW * kUnionLightMax * (4 * sizeof(uint32_t) + kFilterBits / 8) : 0;
+    const size_t unions = sizeof(UnionScratch) * warps + std::max(light, union_table_bytes(cap));
+    return (int)std::max(enumeration, unions);
+}
+
 // One launch of `kernel`: as many CTAs per SM as fit (or grid_per_sm), which
 // claim their vertices through the work counters.
 static sg_status launch_tri(Ctx *c, void (*kernel)(TriArgs), int threads, size_t smem, const TriArgs &a,
                             const char *name, int grid_per_sm = 0) {
     TriArgs args = a;
     SG_CUDA(cudaMemsetAsync(a.work, 0, 2 * sizeof(unsigned long long), c->stream));
-    SG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // the limit is the function's, shared by all threads and contexts: always the
+    // most any graph asks of it, never this launch's size
+    const int limit = threads == kTW * 32 ? max_smem(kTW, kHeavyCap) : max_smem(kHubTW, kHubCap);
+    SG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
     int per_sm = 0;
     SG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
     per_sm = std::max(per_sm, 1);

@@ -137,6 +137,7 @@ struct TriArgs {
     unsigned long long *list_dem;  // [kEoBuckets] triangles that belong in each bucket, listed or not
     unsigned long long list_base[kEoBuckets], list_cap[kEoBuckets];
     int eo_round;                  // this enumeration's round: earlier buckets fold into it
+    int eo_shift;                  // list claims are halved this often (eo_chunk)
     int eo_hi;                     // buckets from this one on are not listed (counted only)
     int *list_overflow;            // bit b: bucket b ran out of room
 };
@@ -157,8 +158,13 @@ constexpr uint32_t kSentinel = 0xFFFFFFFFu;
 // [2^(26+b), 2^(27+b)) (bucket 0: r2 < 2^27), i.e. those that first bid in
 // edge-once round b of the doubling prefix schedule.
 __device__ __forceinline__ int eo_bucket(uint32_t r2) { return r2 < (1u << 27) ? 0 : (31 - __clz((int)r2)) - 26; }
-// list slots a warp claims at a time, in proportion to the bucket's share
-__host__ __device__ constexpr int eo_chunk(int b) { return b <= 1 ? 64 : (32 << b); }
+// list slots a warp claims at a time, in proportion to the bucket's share: 2048
+// over the buckets, halved `shift` times on graphs that fill less (to 32 each
+// at least, a group's most), as what a warp leaves of a claim is read back as
+// sentinels
+__host__ __device__ constexpr int eo_chunk(int b, int shift) {
+    return (b <= 1 ? 64 : (32 << b)) >> shift > 32 ? (b <= 1 ? 64 : (32 << b)) >> shift : 32;
+}
 
 // Per-warp list writer: per bucket it claims chunks of slots, fills them in
 // order and seals the unused tail of a chunk with sentinels.  The cursors
@@ -199,7 +205,7 @@ __device__ __forceinline__ void emit_push(const TriArgs &a, Emitter &em, bool wa
         const unsigned long long cur = __shfl_sync(kFull, em.cur, b);
         const unsigned long long end = __shfl_sync(kFull, em.cur, 8 + b);
         emit_seal(a, cur, end);
-        const unsigned long long chunk = (unsigned long long)eo_chunk(b);
+        const unsigned long long chunk = (unsigned long long)eo_chunk(b, a.eo_shift);
         unsigned long long base = 0;
         if (lane == 0) base = atomicAdd(a.list_ctr + b, chunk);
         base = __shfl_sync(kFull, base, 0);
@@ -1471,6 +1477,19 @@ __global__ void eo_accept_kernel(TriArgs a, const int64_t *__restrict__ off, uin
     }
 }
 
+// the edge that a listed triangle deletes when it is accepted
+template <int CH>
+__device__ __forceinline__ uint32_t chosen_arc(const TriRec &r, const float *wp, const uint32_t *tcnt) {
+    if constexpr (CH == kChoiceMinCount) {
+        return mincount_arc(tcnt, r.e01, r.e02, r.e12);
+    } else if constexpr (CH == kChoiceMaxw) {
+        return maxw_arc(wp, r.x0, r.x1, r.x2, r.e01, r.e02, r.e12);
+    } else {
+        const int k = (int)(((unsigned long long)r.r1 * 3ull) >> 32);
+        return k == 0 ? r.e01 : (k == 1 ? r.e02 : r.e12);
+    }
+}
+
 // Edge-once rounds over the list of live selected triangles.
 // Accept: a triangle holding the reservations of all three of its edges is
 // accepted; accepted triangles are edge-disjoint, so their stores never race.
@@ -1487,16 +1506,7 @@ __global__ void eo_list_accept_kernel(const TriRec *__restrict__ L, int64_t len,
         set_considered(considered, (int64_t)r.e01);
         set_considered(considered, (int64_t)r.e02);
         set_considered(considered, (int64_t)r.e12);
-        uint32_t chosen;
-        if constexpr (CH == kChoiceMinCount) {
-            chosen = mincount_arc(tcnt, r.e01, r.e02, r.e12);
-        } else if constexpr (CH == kChoiceMaxw) {
-            chosen = maxw_arc(wp, r.x0, r.x1, r.x2, r.e01, r.e02, r.e12);
-        } else {
-            const int k = (int)(((unsigned long long)r.r1 * 3ull) >> 32);
-            chosen = k == 0 ? r.e01 : (k == 1 ? r.e02 : r.e12);
-        }
-        delete_arc(del, chosen);
+        delete_arc(del, chosen_arc<CH>(r, wp, tcnt));
     }
 }
 
@@ -1632,6 +1642,161 @@ __global__ void eo_list_reset_kernel(const TriRec *__restrict__ L, int64_t len, 
         resv[r.e02] = ~0ull;
         resv[r.e12] = ~0ull;
     }
+}
+
+// --------------------------------------------- list rounds in one launch
+// On a small list a round's kernels take a few microseconds each, and the host's
+// part -- three to five launches, a copy and a wait per round -- is most of the
+// time.  This kernel runs all rounds of the list that are left: per round it
+// reserves (last round's survivors and the round's bucket), accepts and resets,
+// with a barrier after each.  The grid is one thread-block cluster: its CTAs are
+// scheduled together and meet at the hardware's cluster barrier, so nothing
+// spins, whatever else runs on the device.  What other CTAs wrote is read past
+// the L1.
+struct EoRun {
+    const uint4 *fresh;     // the bucketed list
+    int64_t base[kEoBuckets], used[kEoBuckets];
+    TriRec *active[2];      // this round's bidders are written to active[1] first
+    int64_t len;            // survivors in active[0]
+    int next_bucket, top, sched;
+    unsigned long long *out_len;  // [2], zero
+    unsigned long long *rounds;   // rounds run
+    unsigned long long *resv;
+    uint32_t *considered, *del;
+    const uint32_t *colp, *tcnt;
+    const float *wp;
+    uint32_t k0, k1;
+};
+constexpr int kEoCta = 1024, kEoCluster = 16;
+// List slots up to which the rounds left run in one launch.  Edge-once TR on
+// R-MAT graphs, per call with launches per round / with this (2^20): 4096
+// vertices at p = 0.5 740 / 640 us, 16,384 at p = 0.2 853 / 779 us, 65,536 at
+// 0.2 1247 / 1153 us.  Sixteen CTAs are slow on more: at 2^21 65,536 vertices take
+// 1370 us, at 2^22 1566 us; eight CTAs instead of sixteen: 3454 against 3386
+// us on s18, whose last rounds run here.
+constexpr int64_t kEoOneLaunch = 1 << 20;
+
+__device__ __forceinline__ bool considered_now(const uint32_t *c, uint32_t e) { return (__ldcg(c + (e >> 5)) >> (e & 31)) & 1u; }
+
+// All threads of the cluster arrive, with what they wrote, before any leaves.
+__device__ __forceinline__ void cluster_barrier() {
+    __threadfence();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Append the CTA's survivors: this thread's slot in the list (all threads call).
+__device__ __forceinline__ unsigned long long append_slot(bool keep, unsigned long long *len) {
+    __shared__ int s_cnt[kEoCta / 32];
+    __shared__ unsigned long long s_base;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned m = __ballot_sync(kFull, keep);
+    if (lane == 0) s_cnt[warp] = __popc(m);
+    __syncthreads();
+    if (warp == 0) {
+        const int c = s_cnt[lane];
+        int inc = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o) inc += t;
+        }
+        s_cnt[lane] = inc - c;
+        if (lane == 31) s_base = inc ? atomicAdd(len, (unsigned long long)inc) : 0ull;
+    }
+    __syncthreads();
+    const unsigned long long slot = s_base + s_cnt[warp] + __popc(m & lanemask_lt());
+    __syncthreads();
+    return slot;
+}
+
+template <int CH>
+__global__ void __cluster_dims__(kEoCluster, 1, 1) __launch_bounds__(kEoCta, 1) eo_rounds_kernel(EoRun g) {
+    const int64_t stride = (int64_t)gridDim.x * kEoCta, t0 = (int64_t)blockIdx.x * kEoCta;
+    int64_t len = g.len;
+    int nb = g.next_bucket, cur = 0;
+    auto bid = [&](const TriRec &r, unsigned long long theta) {
+        if ((unsigned long long)r.r2 < theta) {
+            const unsigned long long hi = (unsigned long long)r.r2 << 32;
+            atomicMin(g.resv + r.e01, hi | r.x2);
+            atomicMin(g.resv + r.e02, hi | r.x1);
+            atomicMin(g.resv + r.e12, hi | r.x0);
+        }
+    };
+    auto load = [](const TriRec *p) {
+        const uint4 a = __ldcg(reinterpret_cast<const uint4 *>(p)), b = __ldcg(reinterpret_cast<const uint4 *>(p) + 1);
+        return TriRec{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    };
+    unsigned long long done = 0;
+    for (int sched = g.sched;; ++sched) {
+        unsigned long long theta = 1ull << (27 + min(sched, kEoBuckets - 1));
+        if (g.top < kEoBuckets) theta = min(theta, 1ull << (26 + g.top));  // the list's window
+        TriRec *in = g.active[cur], *out = g.active[cur ^ 1];
+        unsigned long long *out_len = g.out_len + cur;
+        // reserve: drop the triangles that lost an edge, bid for the others
+        for (int64_t b = t0; b < len; b += stride) {
+            const int64_t i = b + threadIdx.x;
+            TriRec r{kSentinel, 0, 0, 0, 0, 0, 0, 0};
+            if (i < len) r = load(in + i);
+            const bool keep = i < len && !(considered_now(g.considered, r.e01) || considered_now(g.considered, r.e02) ||
+                                           considered_now(g.considered, r.e12));
+            if (keep) bid(r, theta);
+            const unsigned long long slot = append_slot(keep, out_len);
+            if (keep) out[slot] = r;
+        }
+        const int64_t fresh = nb < g.top ? g.used[nb] : 0;
+        for (int64_t b = t0; b < fresh; b += stride) {
+            const int64_t i = b + threadIdx.x;
+            uint4 f = make_uint4(kSentinel, 0u, 0u, 0u);
+            if (i < fresh) f = __ldg(g.fresh + g.base[nb] + i);
+            const bool keep = f.x != kSentinel && !(considered_now(g.considered, f.y) || considered_now(g.considered, f.z) ||
+                                                    considered_now(g.considered, f.w));
+            TriRec r{kSentinel, 0, 0, 0, 0, 0, 0, 0};
+            if (keep) {  // expand: vertices from the arc heads, the draw again
+                r.x0 = f.x;
+                r.x1 = __ldg(g.colp + f.y);
+                r.x2 = __ldg(g.colp + f.z);
+                r.e01 = f.y;
+                r.e02 = f.z;
+                r.e12 = f.w;
+                sort_triangle(r.x0, r.x1, r.x2, r.e01, r.e02, r.e12);
+                const uint4 d = philox4x32_10(make_uint4(r.x0, r.x1, r.x2, kTagTri), g.k0, g.k1);
+                r.r1 = d.y;
+                r.r2 = d.z;
+                bid(r, theta);
+            }
+            const unsigned long long slot = append_slot(keep, out_len);
+            if (keep) out[slot] = r;
+        }
+        if (nb < g.top) ++nb;
+        cluster_barrier();
+        len = (int64_t)__ldcg(out_len);
+        if (len > 0) ++done;
+        // accept: a triangle that holds all three of its reservations
+        for (int64_t i = t0 + threadIdx.x; i < len; i += stride) {
+            const TriRec r = load(out + i);
+            const unsigned long long hi = (unsigned long long)r.r2 << 32;
+            if (__ldcg(g.resv + r.e01) != (hi | r.x2) || __ldcg(g.resv + r.e02) != (hi | r.x1) ||
+                __ldcg(g.resv + r.e12) != (hi | r.x0))
+                continue;
+            set_considered(g.considered, (int64_t)r.e01);
+            set_considered(g.considered, (int64_t)r.e02);
+            set_considered(g.considered, (int64_t)r.e12);
+            delete_arc(g.del, chosen_arc<CH>(r, g.wp, g.tcnt));
+        }
+        if (len == 0 && nb >= g.top) break;
+        cluster_barrier();
+        for (int64_t i = t0 + threadIdx.x; i < len; i += stride) {
+            const TriRec r = load(out + i);
+            g.resv[r.e01] = ~0ull;
+            g.resv[r.e02] = ~0ull;
+            g.resv[r.e12] = ~0ull;
+        }
+        if (t0 == 0 && threadIdx.x == 0) g.out_len[cur ^ 1] = 0;
+        cur ^= 1;
+        cluster_barrier();
+    }
+    if (t0 == 0 && threadIdx.x == 0) *g.rounds = done;
 }
 
 // -------------------------------------------------------------------- host
@@ -1933,6 +2098,11 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
     const int64_t acc_blocks = std::min<int64_t>((o.n + 7) / 8, (int64_t)c->num_sms * 8);
     if (st == SG_OK && cudaMemsetAsync(resv, 0xFF, m * sizeof(unsigned long long), c->stream) != cudaSuccess)
         st = cuda_fail(cudaGetLastError(), "memset");
+    // a warp of the main launch lists about a sixth of its probes' share of p W
+    // (R-MAT graphs); its claims together should be at most half of that
+    const double per_warp = (double)a.tp / 4294967296.0 * (double)pl.work / 6.0 / ((double)c->num_sms * 4 * kTW);
+    a.eo_shift = 0;
+    while (a.eo_shift < 6 && (double)(2048 >> a.eo_shift) > 0.5 * per_warp) ++a.eo_shift;
     auto list_blocks = [&](int64_t len) { return std::min<int64_t>((len + 255) / 256, (int64_t)c->num_sms * 8); };
     cudaMemPool_t pool = nullptr;
     if (cudaDeviceGetMemPool(&pool, c->device) != cudaSuccess) {
@@ -1989,7 +2159,7 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
                     // everything fits: split the room by the shares
                     for (int b = rb; b < kEoBuckets; ++b) {
                         const int64_t cb = (int64_t)((double)cap * w[b] / wsum);
-                        if (cb < 4 * eo_chunk(b)) { hi = b; break; }
+                        if (cb < 4 * eo_chunk(b, a.eo_shift)) { hi = b; break; }
                         give(b, cb);
                     }
                 } else {
@@ -2007,7 +2177,7 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
                     double above = 0.0;
                     for (int b = rb; b < kEoBuckets; ++b) {
                         const double d = have_dem ? (double)(b == rb ? fold : dem[b]) : 0.25 * sel_max * w[b] / wsum;
-                        want[b] = (int64_t)(d * (1.0 + 16.0 / eo_chunk(b))) + emit_warps * eo_chunk(b);
+                        want[b] = (int64_t)(d * (1.0 + 16.0 / eo_chunk(b, a.eo_shift))) + emit_warps * eo_chunk(b, a.eo_shift);
                         if (b > rb) above += (double)want[b];
                     }
                     const int64_t first = std::min<int64_t>(want[rb], cap / 2);
@@ -2015,7 +2185,7 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
                     const double scale = above <= rest ? 1.0 : rest / above;
                     for (int b = rb; b < kEoBuckets; ++b) {
                         const int64_t cb = b == rb ? first : (int64_t)((double)want[b] * scale);
-                        if (cb < 4 * eo_chunk(b)) { hi = b; break; }
+                        if (cb < 4 * eo_chunk(b, a.eo_shift)) { hi = b; break; }
                         give(b, cb);
                     }
                 }
@@ -2104,6 +2274,68 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
                     eo_accept_kernel<kChoiceRandom><<<(unsigned)acc_blocks, 256, 0, c->stream>>>(a, g->off, considered);
                 SG_CUDA(cudaGetLastError());
                 SG_CUDA(cudaMemsetAsync(resv, 0xFF, m * sizeof(unsigned long long), c->stream));
+                continue;
+            }
+        }
+        // ---- a list this short: all rounds left in one launch
+        int64_t rest = lenA;
+        for (int b = next_bucket; b < top; ++b) rest += used[b];
+        if (rest <= kEoOneLaunch) {
+            TriRec *B = nullptr;
+            const int bslot = a_slot == kWsActive0 ? kWsActive1 : kWsActive0;
+            const size_t bytes = (size_t)std::max<int64_t>(rest, 1) * sizeof(TriRec);
+            st = ws_get(c, bslot, bytes, (void **)&B);
+            // (the buffer that holds the survivors has room for them; the first
+            // round reads it, later ones write at most what the round before kept)
+            if (st == SG_OK && (lenA == 0 || c->ws_bytes[a_slot] < bytes)) {
+                TriRec *A2 = nullptr;
+                if (lenA == 0) st = ws_get(c, a_slot, bytes, (void **)&A2);
+                if (lenA == 0) A = A2;
+            }
+            if (st != SG_OK) break;
+            if (c->ws_bytes[a_slot] >= bytes) {
+                SG_CUDA(cudaMemsetAsync(lctr, 0, lctr_bytes, c->stream));
+                EoRun r{};
+                r.fresh = L;
+                for (int b = 0; b < kEoBuckets; ++b) {
+                    r.base[b] = ubase[b];
+                    r.used[b] = used[b];
+                }
+                r.active[0] = A;
+                r.active[1] = B;
+                r.len = lenA;
+                r.next_bucket = next_bucket;
+                r.top = top;
+                r.sched = sched;
+                r.out_len = lctr;
+                r.rounds = lctr + 2;
+                r.resv = resv;
+                r.considered = considered;
+                r.del = a.del;
+                r.colp = a.colp;
+                r.tcnt = a.tcnt;
+                r.wp = a.wp;
+                r.k0 = a.k0;
+                r.k1 = a.k1;
+                auto kernel = choice == kChoiceMaxw ? eo_rounds_kernel<kChoiceMaxw>
+                              : choice == kChoiceMinCount ? eo_rounds_kernel<kChoiceMinCount>
+                                                          : eo_rounds_kernel<kChoiceRandom>;
+                SG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+                {
+                    SG_LAUNCH(c, "tri_eo_rounds");
+                    kernel<<<kEoCluster, kEoCta, 0, c->stream>>>(r);
+                }
+                SG_CUDA(cudaGetLastError());
+                SG_CUDA(cudaMemcpyAsync(c->h_pinned, r.rounds, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+                SG_CUDA(cudaStreamSynchronize(c->stream));
+                c->eo_rounds += (uint64_t)c->h_pinned[0];
+                lenA = 0;
+                next_bucket = top;
+                if (top >= kEoBuckets) break;
+                for (int b = 0; b < top; ++b) dem[b] = 0;
+                L = nullptr;
+                listed = false;
+                sched = top - 1;
                 continue;
             }
         }

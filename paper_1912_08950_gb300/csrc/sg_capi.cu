@@ -1,5 +1,6 @@
 // The extern "C" boundary of the library: contexts, graphs, error reporting,
 // launch accounting and the dispatch of compress / divergence to the kernels.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -37,6 +38,35 @@ sg_status cuda_fail(cudaError_t e, const char *what) {
 }
 
 sg_status dalloc(Ctx *c, void **p, size_t bytes) {
+    const size_t at = (c->arena_used + 255) & ~(size_t)255;
+    if (c->arena && at + bytes <= c->arena_bytes) {
+        *p = c->arena + at;
+        c->arena_used = at + std::max<size_t>(bytes, 16);
+        return SG_OK;
+    }
+    return dalloc_own(c, p, bytes);
+}
+
+Scratch::Scratch(Ctx *c_, size_t bytes) : c(c_) {
+    void *p = nullptr;
+    if (bytes > kScratchMax || c->arena || dalloc_own(c, &p, bytes) != SG_OK) {
+        set_error("");
+        c = nullptr;
+        return;
+    }
+    c->arena = static_cast<char *>(p);
+    c->arena_bytes = bytes;
+    c->arena_used = 0;
+}
+
+Scratch::~Scratch() {
+    if (!c) return;
+    (void)cudaFreeAsync(c->arena, c->stream);
+    c->arena = nullptr;
+    c->arena_bytes = c->arena_used = 0;
+}
+
+sg_status dalloc_own(Ctx *c, void **p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
     cudaError_t e = cudaMallocAsync(p, bytes, c->stream);
@@ -51,6 +81,7 @@ sg_status dalloc(Ctx *c, void **p, size_t bytes) {
 }
 
 void dfree(Ctx *c, void *p) {
+    if (c->arena && p >= c->arena && p < c->arena + c->arena_bytes) return;  // goes with the call's scratch
     if (p) (void)cudaFreeAsync(p, c->stream);
 }
 
@@ -65,10 +96,10 @@ sg_status ws_get(Ctx *c, int slot, size_t bytes, void **p) {
     // a quarter more than asked: list fills vary a little from call to call
     // (the order in which warps claim chunks), and each regrowth maps new memory
     size_t want = bytes + bytes / 4;
-    if (dalloc(c, p, want) != SG_OK) {
+    if (dalloc_own(c, p, want) != SG_OK) {
         want = bytes;
         set_error("");
-        sg_status st = dalloc(c, p, want);
+        sg_status st = dalloc_own(c, p, want);
         if (st != SG_OK) return st;
     }
     c->ws[slot] = *p;
@@ -104,8 +135,15 @@ LaunchScope::~LaunchScope() {
 }
 
 sg_status check_device_error(Ctx *c) {
+    int64_t unused;
+    return read_checked(c, nullptr, &unused);
+}
+
+sg_status read_checked(Ctx *c, const int64_t *dptr, int64_t *out) {
+    if (dptr) SG_CUDA(cudaMemcpyAsync(c->h_pinned + 1, dptr, sizeof(int64_t), cudaMemcpyDeviceToHost, c->stream));
     SG_CUDA(cudaMemcpyAsync(c->h_pinned, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     SG_CUDA(cudaStreamSynchronize(c->stream));
+    *out = c->h_pinned[1];
     int code = 0;
     std::memcpy(&code, c->h_pinned, sizeof(int));
     if (code == kDevOk) return SG_OK;
@@ -124,6 +162,9 @@ sg_status check_device_error(Ctx *c) {
 
 static sg_status compress_tr(Ctx *c, const Graph *g, sg_kernel k, double p, uint64_t seed, Graph **out) {
     const bool maxw = (k == SG_TR_MAXW || k == SG_TR_EO_MAXW);
+    // about what the arrays below and the kernels' own take (5 arrays of nnz
+    // words, 9 of n, the flags); what does not fit is allocated apart
+    const Scratch scratch(c, (size_t)g->n * 48 + (size_t)g->nnz * 24 + (256u << 10));
     RowMaps rm;
     Oriented o;
     uint32_t *del = nullptr;

@@ -965,9 +965,10 @@ sg_status new_graph(Ctx *c, int64_t n, int64_t nnz_cap, bool weighted, Graph **o
     h->device = c->device;
     h->n = n;
     h->owned = true;
-    sg_status st = dalloc(c, (void **)&h->off, sizeof(int64_t) * (size_t)(n + 1));
-    if (st == SG_OK) st = dalloc(c, (void **)&h->col, sizeof(uint32_t) * (size_t)std::max<int64_t>(nnz_cap, 1));
-    if (st == SG_OK && weighted) st = dalloc(c, (void **)&h->w, sizeof(float) * (size_t)std::max<int64_t>(nnz_cap, 1));
+    sg_status st = dalloc_own(c, (void **)&h->off, sizeof(int64_t) * (size_t)(n + 1));
+    if (st == SG_OK) st = dalloc_own(c, (void **)&h->col, sizeof(uint32_t) * (size_t)std::max<int64_t>(nnz_cap, 1));
+    if (st == SG_OK && weighted)
+        st = dalloc_own(c, (void **)&h->w, sizeof(float) * (size_t)std::max<int64_t>(nnz_cap, 1));
     if (st != SG_OK) {
         dfree(c, h->off);
         dfree(c, h->col);
@@ -989,6 +990,7 @@ void delete_graph(Ctx *c, Graph *h) {
 
 sg_status compress_edges(Ctx *c, const Graph *g, sg_kernel k, double p, uint64_t seed, int want_weights,
                          Graph **out) {
+    const Scratch scratch(c, (size_t)g->n * 2 + (size_t)g->nnz / 4 + (64u << 10));
     RowMaps rm;
     CompactScratch cs;
     uint16_t *deg16 = nullptr;
@@ -1019,8 +1021,7 @@ sg_status compress_edges(Ctx *c, const Graph *g, sg_kernel k, double p, uint64_t
             }
         }
     }
-    if (st == SG_OK) st = read_i64(c, h->off + g->n, &h->nnz);
-    if (st == SG_OK) st = check_device_error(c);
+    if (st == SG_OK) st = read_checked(c, h->off + g->n, &h->nnz);
     free_compact_scratch(c, &cs);
     dfree(c, deg16);
     free_row_maps(c, &rm);
@@ -1064,9 +1065,7 @@ sg_status orient(Ctx *c, const Graph *g, const RowMaps &rm, bool weights, Orient
     dfree(c, cs.scan);
     if (st != SG_OK) return st;
     int64_t mp = 0;
-    st = read_i64(c, o->off + g->n, &mp);
-    if (st != SG_OK) return st;
-    st = check_device_error(c);
+    st = read_checked(c, o->off + g->n, &mp);
     if (st != SG_OK) return st;
     if (mp != o->m)
         return fail(SG_ERR_INVALID_GRAPH, "graph is not symmetric: oriented arcs != nnz/2");
@@ -1097,8 +1096,7 @@ sg_status resolve_mask(Ctx *c, const Graph *g, const RowMaps &rm, const Oriented
         MaskPol pol{o.fwd_bits, o.fwd_excl, o.inl, del, std::max<int64_t>(g->nnz - o.m, 1), m1};
         st = run_compact(c, g, rm, pol, g->w, h->off, h->col, h->w, cs, "compact_trmask");
     }
-    if (st == SG_OK) st = read_i64(c, h->off + g->n, &h->nnz);
-    if (st == SG_OK) st = check_device_error(c);
+    if (st == SG_OK) st = read_checked(c, h->off + g->n, &h->nnz);
     free_compact_scratch(c, &cs);
     if (st != SG_OK) {
         delete_graph(c, h);
@@ -1354,8 +1352,7 @@ sg_status low_degree(Ctx *c, const Graph *g, uint32_t *new_to_old, Graph **out) 
         if (cudaMemsetAsync(h->off, 0, sizeof(int64_t), c->stream) != cudaSuccess)
             st = cuda_fail(cudaGetLastError(), "cudaMemsetAsync");
     }
-    if (st == SG_OK) st = read_i64(c, h->off + kept, &h->nnz);
-    if (st == SG_OK) st = check_device_error(c);
+    if (st == SG_OK) st = read_checked(c, h->off + kept, &h->nnz);
     dfree(c, new_id);
     dfree(c, off_c);
     free_compact_scratch(c, &cs);

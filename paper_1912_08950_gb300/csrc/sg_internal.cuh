@@ -53,6 +53,9 @@ struct Ctx {
     // lists), so that repeated calls do not churn the stream-ordered pool
     void *ws[3] = {nullptr, nullptr, nullptr};
     size_t ws_bytes[3] = {0, 0, 0};
+    // scratch of one call on a small graph (Scratch): dalloc hands it out in order
+    char *arena = nullptr;
+    size_t arena_bytes = 0, arena_used = 0;
     std::vector<ProfRec> prof;             // events of launches since reset
     std::vector<cudaEvent_t> event_pool;   // recycled events
 };
@@ -86,6 +89,19 @@ bool ctx_alive(const Ctx *c);
 
 // stream-ordered device allocation on the context stream
 sg_status dalloc(Ctx *c, void **p, size_t bytes);
+// the same, never from a call's scratch: for what outlives the call
+sg_status dalloc_own(Ctx *c, void **p, size_t bytes);
+// One allocation for all scratch of a call on a small graph, where some twenty
+// separate allocations and frees take as long as the kernels (a few us each);
+// freed in stream order when the call ends.  Above kScratchMax bytes (and for
+// what does not fit) dalloc allocates as ever, so that large calls still free
+// each piece as soon as it is done with.
+constexpr size_t kScratchMax = 32u << 20;
+struct Scratch {
+    Ctx *c;
+    Scratch(Ctx *c, size_t bytes);
+    ~Scratch();
+};
 // workspace `slot` of at least `bytes` bytes (contents undefined; owned by the context)
 sg_status ws_get(Ctx *c, int slot, size_t bytes, void **p);
 void dfree(Ctx *c, void *p);
@@ -104,6 +120,8 @@ struct LaunchScope {
 
 // read the device error word and reset it; map it to a status
 sg_status check_device_error(Ctx *c);
+// *dptr and the device error word with one wait
+sg_status read_checked(Ctx *c, const int64_t *dptr, int64_t *out);
 
 // -------------------------------------------------------------- device code
 #ifdef __CUDACC__

@@ -2082,6 +2082,7 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
     int top = kEoBuckets;          // the list holds every live triangle of the buckets below this one
     int sched = 0;                 // step of the prefix schedule: bids come from r2 below the top of bucket sched
     bool listed = false;
+    bool no_small = false;         // the small graph's list size did not fit
     bool try_list = o.m <= (int64_t)0xFFFFFFFFll && c->eo_list_cap >= 0;
     // warps of one enumeration launch, at most: each may leave a chunk per bucket part filled
     const int64_t emit_warps = (int64_t)c->num_sms * (8 * kTW + kHubTW);
@@ -2136,7 +2137,11 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
             if (try_list) {
                 // ---- one enumeration bids for this round and lists the live selected
                 // triangles of as many buckets, from rb on, as the room allows
-                const int64_t cap = list_capacity();
+                // (asking how much memory is free takes longer than a small graph's
+                // rounds: a list that is bounded by 2^24 records is not worth it)
+                const double most = (double)a.tp / 4294967296.0 * (double)pl.work;
+                const bool small = !no_small && !have_dem && c->eo_list_cap == 0 && most <= (double)(1 << 23);
+                const int64_t cap = small ? (int64_t)1 << 24 : list_capacity();
                 hi = kEoBuckets;
                 int64_t run = 0;
                 for (int b = 0; b < kEoBuckets; ++b) a.list_base[b] = a.list_cap[b] = 0;
@@ -2192,7 +2197,16 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
                 if (hi <= rb) hi = 0;  // nothing to list: the pass only bids and counts
                 if (hi > 0) {
                     const size_t lbytes = (size_t)std::max<int64_t>(run, 1) * sizeof(uint4);
-                    if (ws_get(c, kWsList, lbytes, (void **)&L) != SG_OK && pool) {
+                    if (small) {
+                        if (ws_get(c, kWsList, lbytes, (void **)&L) != SG_OK) {  // size it by the free memory then
+                            set_error("");
+                            L = nullptr;
+                            no_small = true;
+                            --round;
+                            --sched;
+                            continue;
+                        }
+                    } else if (ws_get(c, kWsList, lbytes, (void **)&L) != SG_OK && pool) {
                         // the pool's idle memory may be too fragmented: hand it back and retry
                         (void)cudaStreamSynchronize(c->stream);
                         (void)cudaMemPoolTrimTo(pool, 0);

@@ -10,7 +10,7 @@
 // shared-memory hash table of the longer one: every vertex x stages N+(x) in
 // a table once and streams (a) N+(v) for its out-arcs x->v with
 // d+(v) <= d+(x) and (b) N+(u) for its in-arcs u->x with d+(u) < d+(x); the
-// in-arcs of kind (b) are gathered per vertex by one scatter pass.  Each arc
+// in-arcs of kind (b) come from the reverse list.  Each arc
 // is handled once, at the end with the longer list, so the probes number
 // sum over arcs of min(d+(u), d+(v)) -- under half of the plain forward
 // algorithm's sum of d+(v) on power-law graphs.  Vertices with a short N+(x)
@@ -62,6 +62,8 @@ constexpr int kUnionLightItems = 512;  // ... with at most this many lists to st
 // 0.5: both passes 528 ms against 551 at 128; s23 equal), 128 on the others
 // (s22: 19.2 ms against 22.3 at 256; 64 leaves a third more arc ends to pass 2)
 constexpr int kShortList = 128, kShortListHubs = 256;
+// the second pass has no light vertices: their lists must all be short
+static_assert(kUnionLightMax <= kShortList, "a light vertex's lists are streamed whole in the first pass");
 constexpr int kEoBuckets = 6;     // edge-once list buckets (rounds 0..5 of the prefix schedule)
 // context workspaces of the edge-once rounds: the list and the two active lists
 constexpr int kWsList = 0, kWsActive0 = 1, kWsActive1 = 2;
@@ -580,6 +582,101 @@ __device__ __forceinline__ void stream_in_group(const TriArgs &a, const Table &t
     }
 }
 
+// Count the triangles on up to 32 arcs of a light table vertex u: its out-arcs
+// [first, first + cnt) or entries of its in-list.  The lists are short (a few to
+// 64 elements), so they are streamed as one sequence, a slab of 32 elements at a
+// time: a lane finds its element's arc from the arcs that start inside the
+// slab, and the first lane of an arc's run adds the run's hits to the arc's
+// counters.  A list at a time, 64 lanes wide, left most lanes idle and waited for
+// one list's loads after another: triangles per vertex of a geometric graph
+// (2^20 vertices, 25 M edges, lists of 17 elements) took 5.18 ms, now 2.15; of
+// R-MAT s20, where most elements are in heavy vertices' lists, 9.33 and 8.98.
+// Returns the hits (all lanes).  arc: 32 entries of the warp's scratch.
+template <Mode M>
+__device__ __forceinline__ unsigned count_group(const TriArgs &a, const Table &tb, int sh, int stash_n, int d, uint32_t ou,
+                                                bool out, int64_t first, int cnt, uint4 *arc,
+                                                unsigned long long &probes) {
+    const int lane = threadIdx.x & 31;
+    uint32_t sv = 0, se = 0, sp = 0;
+    int sl = 0;
+    if (lane < cnt) {
+        if (out) {
+            se = (uint32_t)first + lane;
+            sv = __ldg(a.colp + se);
+        } else {
+            const uint2 it = __ldg(a.inl + first + lane);
+            sv = it.x;
+            se = it.y;
+        }
+        const int64_t b0 = __ldg(a.offp + sv);
+        const int dv = (int)(__ldg(a.offp + sv + 1) - b0);
+        sp = (uint32_t)b0;
+        if (out ? dv <= d : dv < d) sl = dv;  // else streamed from the other end
+    }
+    probes += (unsigned)sl;
+    int inc = sl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += x;
+    }
+    const int total = __shfl_sync(kFull, inc, 31);
+    const int start = sl > 0 ? inc - sl : INT_MIN;
+    const unsigned wanted = __ballot_sync(kFull, sl > 0);
+    if (sl > 0) arc[__popc(wanted & lanemask_lt())] = make_uint4(sv, se, sp - (uint32_t)start, 0u);
+    __syncwarp();
+    const uint32_t lt = lanemask_lt(), le = lt | (1u << lane);
+    int before = -1;  // arcs that start before the slab, minus one
+    unsigned hits = 0, nstarts = 0;
+    int nk = 0;
+    uint32_t nw = kEmpty, narc = 0;
+    auto load = [&](int s) {
+        const unsigned rel = (unsigned)start - (unsigned)s;
+        nstarts = __reduce_or_sync(kFull, rel < 32u ? 1u << rel : 0u);
+        nk = before + __popc(nstarts & le);
+        before += __popc(nstarts);
+        nw = kEmpty;
+        if (s + lane < total) {
+            narc = arc[nk].z + (uint32_t)(s + lane);
+            nw = __ldg(a.colp + narc);
+        }
+    };
+    if (total > 0) load(0);
+    for (int s = 0; s < total; s += 32) {
+        const uint32_t w = nw, ivw = narc;
+        const unsigned starts = nstarts;
+        const int k = nk;
+        if (s + 32 < total) load(s + 32);  // the next slab's, while this one is probed
+        uint32_t t = 0;
+        bool h = table_find(tb, sh, w, t);
+        if (stash_n != 0 && !h && w != kEmpty) {  // rare
+            const unsigned long long c = stash_find(tb.stash, stash_n, w);
+            h = c != kStashNone;
+            t = (uint32_t)c;
+        }
+        const unsigned m = __ballot_sync(kFull, h);
+        if (m == 0) continue;
+        hits += (unsigned)__popc(m);
+        if constexpr (M == Mode::Count) continue;
+        // hits on this lane's arc, if its run starts here
+        const unsigned later = starts & ~le;
+        const unsigned run = (later ? (1u << (__ffs(later) - 1)) - 1u : kFull) & ~lt;
+        const unsigned c = (lane == 0 || ((starts >> lane) & 1u)) ? (unsigned)__popc(m & run) : 0u;
+        if constexpr (M == Mode::EdgeCount) {
+            if (h) {
+                atomicAdd(a.tcnt + ou + t, 1u);
+                atomicAdd(a.tcnt + ivw, 1u);
+            }
+            if (c) atomicAdd(a.tcnt + arc[k].y, c);
+        } else {
+            if (h) atomicAdd(a.vcnt + w, 1ull);
+            if (c) atomicAdd(a.vcnt + arc[k].x, (unsigned long long)c);
+        }
+    }
+    __syncwarp();  // the entries are read before the next group writes them
+    return hits;
+}
+
 template <Mode M>
 __device__ __forceinline__ void finish(const TriArgs &a, unsigned live, unsigned long long probes,
                                        unsigned long long tris, Emitter &em) {
@@ -753,55 +850,75 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tr
                 for (int s2 = lane; s2 < (1 << log_slots); s2 += 32) tb.slot[s2] = kSlotEmpty;
                 if (lane == 0) *tb.stash_n = 0;
                 __syncwarp();
-                // lane k holds N+(u)[k] and N+(u)[k + 32] with their list bounds
-                uint32_t n0 = kEmpty, n1 = kEmpty, o0 = 0, o1 = 0;
-                int d0 = 0, d1 = 0;
-                bool live0 = false, live1 = false;  // the arc u->w may close a live triangle
-                if (lane < d) {
-                    n0 = __ldg(a.colp + ou + lane);
-                    const int64_t b0 = __ldg(a.offp + n0);
-                    o0 = (uint32_t)b0;
-                    d0 = (int)(__ldg(a.offp + n0 + 1) - b0);
-                    live0 = !kEdgeOnce<M> || a.considered == nullptr || !considered_bit(a.considered, (int64_t)ou + lane);
-                    if (live0) table_insert(tb, log_slots, n0, lane, a.err);
-                    if (!live0 || d0 > d) d0 = 0;  // streamed from n0's side when d+(n0) > d+(u)
-                }
-                if (lane + 32 < d) {
-                    n1 = __ldg(a.colp + ou + lane + 32);
-                    const int64_t b1 = __ldg(a.offp + n1);
-                    o1 = (uint32_t)b1;
-                    d1 = (int)(__ldg(a.offp + n1 + 1) - b1);
-                    live1 = !kEdgeOnce<M> || a.considered == nullptr ||
-                            !considered_bit(a.considered, (int64_t)ou + lane + 32);
-                    if (live1) table_insert(tb, log_slots, n1, lane + 32, a.err);
-                    if (!live1 || d1 > d) d1 = 0;
-                }
-                __syncwarp();
-                const int stash_n = min(*tb.stash_n, kStash);
-                uint32_t pa, pb;  // first slabs of the next list, loading ahead
-                first_slabs(a, __shfl_sync(kFull, o0, 0), __shfl_sync(kFull, d0, 0), pa, pb);
-                for (int i = 0; i < d; ++i) {
-                    const bool lo = i < 32;
-                    const uint32_t v = __shfl_sync(kFull, lo ? n0 : n1, i & 31);
-                    const uint32_t ov = __shfl_sync(kFull, lo ? o0 : o1, i & 31);
-                    const int dv = __shfl_sync(kFull, lo ? d0 : d1, i & 31);
-                    const uint32_t ca = pa, cb = pb;
-                    if (i + 1 < d) {
-                        const bool ln = i + 1 < 32;
-                        first_slabs(a, __shfl_sync(kFull, ln ? o0 : o1, (i + 1) & 31),
-                                    __shfl_sync(kFull, ln ? d0 : d1, (i + 1) & 31), pa, pb);
+                if constexpr (!kEdgeOnce<M>) {
+                    for (int k = lane; k < d; k += 32) table_insert(tb, log_slots, __ldg(a.colp + ou + k), k, a.err);
+                    __syncwarp();
+                    const int sn = min(*tb.stash_n, kStash);
+                    uint4 *arc = reinterpret_cast<uint4 *>(&q);  // the queue has no hits in these passes
+                    unsigned hits = 0;
+                    for (int c = 0; c < d; c += 32)
+                        hits += count_group<M>(a, tb, 32 - log_slots, sn, d, ou, true, (int64_t)ou + c, min(32, d - c),
+                                               arc, probes);
+                    const int64_t ib = nin > 0 ? __ldg(a.offs + u) - (int64_t)ou : 0;
+                    for (int c = 0; c < nin; c += 32)
+                        hits += count_group<M>(a, tb, 32 - log_slots, sn, d, ou, false, ib + c, min(32, nin - c), arc,
+                                               probes);
+                    if (lane == 0) {
+                        tris += hits;
+                        if (M == Mode::VertexCount && hits) atomicAdd(a.vcnt + u, (unsigned long long)hits);
                     }
-                    if (lane == 0) probes += (unsigned)dv;
-                    probe_list<M>(a, tb, log_slots, stash_n, u, ou + (uint32_t)i, ou, v, ov, dv, ca, cb, q, qst,
-                                  live, tris, em);
+                    __syncwarp();
+                } else {
+                    // lane k holds N+(u)[k] and N+(u)[k + 32] with their list bounds
+                    uint32_t n0 = kEmpty, n1 = kEmpty, o0 = 0, o1 = 0;
+                    int d0 = 0, d1 = 0;
+                    bool live0 = false, live1 = false;  // the arc u->w may close a live triangle
+                    if (lane < d) {
+                        n0 = __ldg(a.colp + ou + lane);
+                        const int64_t b0 = __ldg(a.offp + n0);
+                        o0 = (uint32_t)b0;
+                        d0 = (int)(__ldg(a.offp + n0 + 1) - b0);
+                        live0 = a.considered == nullptr || !considered_bit(a.considered, (int64_t)ou + lane);
+                        if (live0) table_insert(tb, log_slots, n0, lane, a.err);
+                        if (!live0 || d0 > d) d0 = 0;  // streamed from n0's side when d+(n0) > d+(u)
+                    }
+                    if (lane + 32 < d) {
+                        n1 = __ldg(a.colp + ou + lane + 32);
+                        const int64_t b1 = __ldg(a.offp + n1);
+                        o1 = (uint32_t)b1;
+                        d1 = (int)(__ldg(a.offp + n1 + 1) - b1);
+                        live1 = a.considered == nullptr ||
+                                !considered_bit(a.considered, (int64_t)ou + lane + 32);
+                        if (live1) table_insert(tb, log_slots, n1, lane + 32, a.err);
+                        if (!live1 || d1 > d) d1 = 0;
+                    }
+                    __syncwarp();
+                    const int stash_n = min(*tb.stash_n, kStash);
+                    uint32_t pa, pb;  // first slabs of the next list, loading ahead
+                    first_slabs(a, __shfl_sync(kFull, o0, 0), __shfl_sync(kFull, d0, 0), pa, pb);
+                    for (int i = 0; i < d; ++i) {
+                        const bool lo = i < 32;
+                        const uint32_t v = __shfl_sync(kFull, lo ? n0 : n1, i & 31);
+                        const uint32_t ov = __shfl_sync(kFull, lo ? o0 : o1, i & 31);
+                        const int dv = __shfl_sync(kFull, lo ? d0 : d1, i & 31);
+                        const uint32_t ca = pa, cb = pb;
+                        if (i + 1 < d) {
+                            const bool ln = i + 1 < 32;
+                            first_slabs(a, __shfl_sync(kFull, ln ? o0 : o1, (i + 1) & 31),
+                                        __shfl_sync(kFull, ln ? d0 : d1, (i + 1) & 31), pa, pb);
+                        }
+                        if (lane == 0) probes += (unsigned)dv;
+                        probe_list<M>(a, tb, log_slots, stash_n, u, ou + (uint32_t)i, ou, v, ov, dv, ca, cb, q, qst,
+                                      live, tris, em);
+                    }
+                    // in-arcs v->u with d+(v) < d+(u), in groups of 32
+                    const int64_t ib = nin > 0 ? __ldg(a.offs + u) - (int64_t)ou : 0;
+                    for (int c = 0; c < nin; c += 32)
+                        stream_in_group<M>(a, tb, log_slots, stash_n, u, d, ou, ib, c, min(32, nin - c), q, qst,
+                                           live, probes, tris, em, true);
+                    flush_hits<M>(a, q, qst, u, live, em);
+                    __syncwarp();
                 }
-                // in-arcs v->u with d+(v) < d+(u), in groups of 32
-                const int64_t ib = nin > 0 ? __ldg(a.offs + u) - (int64_t)ou : 0;
-                for (int c = 0; c < nin; c += 32)
-                    stream_in_group<M>(a, tb, log_slots, stash_n, u, d, ou, ib, c, min(32, nin - c), q, qst,
-                                       live, probes, tris, em, true);
-                flush_hits<M>(a, q, qst, u, live, em);
-                __syncwarp();
             }
         }
     }

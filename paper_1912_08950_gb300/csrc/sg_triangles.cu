@@ -1308,9 +1308,13 @@ __device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, i
 // One launch of a union pass: the heavy vertices a CTA each (largest work bound
 // first; the warps claim groups of 32 arcs), then the light ones a warp each.
 // Bound by instruction issue on the integer pipe, like the counting passes:
-// four CTAs of 8 warps per SM at 64 registers (the drain is inlined).
+// four CTAs of 8 warps per SM at 64 registers (the drain is inlined).  The second
+// pass also waits for random reads of records and live lists, and is faster at
+// three CTAs with more registers: s22 3.14 -> 2.84 ms, s26 51.6 -> 46.4,
+// max-weight on the Chung-Lu graph 1.54 -> 1.38; the first pass is slower at
+// three (s22 16.4 -> 17.0, s26 248 -> 276) and at five (17.0, 253).
 template <Mode M, int TW, bool kAlive>
-__global__ void __launch_bounds__(TW * 32, TW == kTW ? 4 : 1) tri_union_kernel(TriArgs a) {
+__global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri_union_kernel(TriArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_next;
     __shared__ long long s_h;

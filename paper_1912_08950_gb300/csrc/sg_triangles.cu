@@ -582,20 +582,23 @@ __device__ __forceinline__ void stream_in_group(const TriArgs &a, const Table &t
     }
 }
 
-// Count the triangles on up to 32 arcs of a light table vertex u: its out-arcs
+// Find the triangles on up to 32 arcs of a light table vertex u: its out-arcs
 // [first, first + cnt) or entries of its in-list.  The lists are short (a few to
 // 64 elements), so they are streamed as one sequence, a slab of 32 elements at a
 // time: a lane finds its element's arc from the arcs that start inside the
-// slab, and the first lane of an arc's run adds the run's hits to the arc's
-// counters.  A list at a time, 64 lanes wide, left most lanes idle and waited for
+// slab.  Counting: the first lane of an arc's run adds the run's hits to the
+// arc's counters; edge-once: the hits go to the queue.  A list at a time, 64 lanes wide, left most lanes idle and waited for
 // one list's loads after another: triangles per vertex of a geometric graph
 // (2^20 vertices, 25 M edges, lists of 17 elements) took 5.18 ms, now 2.15; of
 // R-MAT s20, where most elements are in heavy vertices' lists, 9.33 and 8.98.
+// The edge-once listing pass at p = 0.5: 7.90 and 4.22 on the geometric graph,
+// 5.88 and 4.99 on a Chung-Lu graph of 2^20 vertices, 23.1 and 22.3 on R-MAT s21.
 // Returns the hits (all lanes).  arc: 32 entries of the warp's scratch.
 template <Mode M>
-__device__ __forceinline__ unsigned count_group(const TriArgs &a, const Table &tb, int sh, int stash_n, int d, uint32_t ou,
-                                                bool out, int64_t first, int cnt, uint4 *arc,
-                                                unsigned long long &probes) {
+__device__ __forceinline__ unsigned light_group(const TriArgs &a, const Table &tb, int sh, int stash_n, uint32_t u,
+                                                int d, uint32_t ou, bool out, int64_t first, int cnt, uint4 *arc,
+                                                HitQueue &q, QState &qs, unsigned &live, unsigned long long &probes,
+                                                Emitter &em) {
     const int lane = threadIdx.x & 31;
     uint32_t sv = 0, se = 0, sp = 0;
     int sl = 0;
@@ -612,6 +615,8 @@ __device__ __forceinline__ unsigned count_group(const TriArgs &a, const Table &t
         const int dv = (int)(__ldg(a.offp + sv + 1) - b0);
         sp = (uint32_t)b0;
         if (out ? dv <= d : dv < d) sl = dv;  // else streamed from the other end
+        // a considered arc closes no live triangle
+        if (kEdgeOnce<M> && a.considered != nullptr && considered_bit(a.considered, se)) sl = 0;
     }
     probes += (unsigned)sl;
     int inc = sl;
@@ -658,6 +663,21 @@ __device__ __forceinline__ unsigned count_group(const TriArgs &a, const Table &t
         if (m == 0) continue;
         hits += (unsigned)__popc(m);
         if constexpr (M == Mode::Count) continue;
+        if constexpr (kEdgeOnce<M>) {
+            if (h) {
+                const int s0 = (qs.head + qs.n + __popc(m & lt)) & (kQ - 1);
+                const uint4 c = arc[k];
+                q.v[s0] = c.x; q.iuv[s0] = c.y; q.iuw[s0] = ou + t; q.ivw[s0] = ivw;
+            }
+            qs.n += __popc(m);
+            __syncwarp();
+            if (qs.n >= 32) {  // fewer than 32 are left after each slab
+                drain32<M>(a, q, qs.head, u, live, em);
+                qs.head = (qs.head + 32) & (kQ - 1);
+                qs.n -= 32;
+            }
+            continue;
+        }
         // hits on this lane's arc, if its run starts here
         const unsigned later = starts & ~le;
         const unsigned run = (later ? (1u << (__ffs(later) - 1)) - 1u : kFull) & ~lt;
@@ -823,6 +843,7 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tr
     // ---- phase 2: light vertices
     if constexpr (TW == kTW) {
         Table tb{reinterpret_cast<uint32_t *>(tbl) + warp * kLightSlots, s_stash[warp], &s_stash_n[warp]};
+        uint4 *arc = reinterpret_cast<uint4 *>(tbl + sizeof(uint32_t) * kLightSlots * TW) + warp * 32;
         for (;;) {
             unsigned long long base = 0;
             if (lane == 0) base = atomicAdd(a.work + 1, (unsigned long long)a.light_claim);
@@ -850,75 +871,28 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tr
                 for (int s2 = lane; s2 < (1 << log_slots); s2 += 32) tb.slot[s2] = kSlotEmpty;
                 if (lane == 0) *tb.stash_n = 0;
                 __syncwarp();
-                if constexpr (!kEdgeOnce<M>) {
-                    for (int k = lane; k < d; k += 32) table_insert(tb, log_slots, __ldg(a.colp + ou + k), k, a.err);
-                    __syncwarp();
-                    const int sn = min(*tb.stash_n, kStash);
-                    uint4 *arc = reinterpret_cast<uint4 *>(&q);  // the queue has no hits in these passes
-                    unsigned hits = 0;
-                    for (int c = 0; c < d; c += 32)
-                        hits += count_group<M>(a, tb, 32 - log_slots, sn, d, ou, true, (int64_t)ou + c, min(32, d - c),
-                                               arc, probes);
-                    const int64_t ib = nin > 0 ? __ldg(a.offs + u) - (int64_t)ou : 0;
-                    for (int c = 0; c < nin; c += 32)
-                        hits += count_group<M>(a, tb, 32 - log_slots, sn, d, ou, false, ib + c, min(32, nin - c), arc,
-                                               probes);
-                    if (lane == 0) {
-                        tris += hits;
-                        if (M == Mode::VertexCount && hits) atomicAdd(a.vcnt + u, (unsigned long long)hits);
-                    }
-                    __syncwarp();
-                } else {
-                    // lane k holds N+(u)[k] and N+(u)[k + 32] with their list bounds
-                    uint32_t n0 = kEmpty, n1 = kEmpty, o0 = 0, o1 = 0;
-                    int d0 = 0, d1 = 0;
-                    bool live0 = false, live1 = false;  // the arc u->w may close a live triangle
-                    if (lane < d) {
-                        n0 = __ldg(a.colp + ou + lane);
-                        const int64_t b0 = __ldg(a.offp + n0);
-                        o0 = (uint32_t)b0;
-                        d0 = (int)(__ldg(a.offp + n0 + 1) - b0);
-                        live0 = a.considered == nullptr || !considered_bit(a.considered, (int64_t)ou + lane);
-                        if (live0) table_insert(tb, log_slots, n0, lane, a.err);
-                        if (!live0 || d0 > d) d0 = 0;  // streamed from n0's side when d+(n0) > d+(u)
-                    }
-                    if (lane + 32 < d) {
-                        n1 = __ldg(a.colp + ou + lane + 32);
-                        const int64_t b1 = __ldg(a.offp + n1);
-                        o1 = (uint32_t)b1;
-                        d1 = (int)(__ldg(a.offp + n1 + 1) - b1);
-                        live1 = a.considered == nullptr ||
-                                !considered_bit(a.considered, (int64_t)ou + lane + 32);
-                        if (live1) table_insert(tb, log_slots, n1, lane + 32, a.err);
-                        if (!live1 || d1 > d) d1 = 0;
-                    }
-                    __syncwarp();
-                    const int stash_n = min(*tb.stash_n, kStash);
-                    uint32_t pa, pb;  // first slabs of the next list, loading ahead
-                    first_slabs(a, __shfl_sync(kFull, o0, 0), __shfl_sync(kFull, d0, 0), pa, pb);
-                    for (int i = 0; i < d; ++i) {
-                        const bool lo = i < 32;
-                        const uint32_t v = __shfl_sync(kFull, lo ? n0 : n1, i & 31);
-                        const uint32_t ov = __shfl_sync(kFull, lo ? o0 : o1, i & 31);
-                        const int dv = __shfl_sync(kFull, lo ? d0 : d1, i & 31);
-                        const uint32_t ca = pa, cb = pb;
-                        if (i + 1 < d) {
-                            const bool ln = i + 1 < 32;
-                            first_slabs(a, __shfl_sync(kFull, ln ? o0 : o1, (i + 1) & 31),
-                                        __shfl_sync(kFull, ln ? d0 : d1, (i + 1) & 31), pa, pb);
-                        }
-                        if (lane == 0) probes += (unsigned)dv;
-                        probe_list<M>(a, tb, log_slots, stash_n, u, ou + (uint32_t)i, ou, v, ov, dv, ca, cb, q, qst,
-                                      live, tris, em);
-                    }
-                    // in-arcs v->u with d+(v) < d+(u), in groups of 32
-                    const int64_t ib = nin > 0 ? __ldg(a.offs + u) - (int64_t)ou : 0;
-                    for (int c = 0; c < nin; c += 32)
-                        stream_in_group<M>(a, tb, log_slots, stash_n, u, d, ou, ib, c, min(32, nin - c), q, qst,
-                                           live, probes, tris, em, true);
-                    flush_hits<M>(a, q, qst, u, live, em);
-                    __syncwarp();
+                for (int k = lane; k < d; k += 32) {
+                    // the arc u->w may close a live triangle
+                    if (!kEdgeOnce<M> || a.considered == nullptr || !considered_bit(a.considered, (int64_t)ou + k))
+                        table_insert(tb, log_slots, __ldg(a.colp + ou + k), k, a.err);
                 }
+                __syncwarp();
+                const int stash_n = min(*tb.stash_n, kStash);
+                unsigned hits = 0;
+                for (int c = 0; c < d; c += 32)
+                    hits += light_group<M>(a, tb, 32 - log_slots, stash_n, u, d, ou, true, (int64_t)ou + c,
+                                           min(32, d - c), arc, q, qst, live, probes, em);
+                // in-arcs v->u with d+(v) < d+(u)
+                const int64_t ib = nin > 0 ? __ldg(a.offs + u) - (int64_t)ou : 0;
+                for (int c = 0; c < nin; c += 32)
+                    hits += light_group<M>(a, tb, 32 - log_slots, stash_n, u, d, ou, false, ib + c, min(32, nin - c),
+                                           arc, q, qst, live, probes, em);
+                if (lane == 0) {
+                    tris += hits;
+                    if (M == Mode::VertexCount && hits) atomicAdd(a.vcnt + u, (unsigned long long)hits);
+                }
+                flush_hits<M>(a, q, qst, u, live, em);
+                __syncwarp();
             }
         }
     }
@@ -2039,9 +2013,10 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
     }
     SG_CUDA(cudaGetLastError());
     // shared memory: hit queues + the larger of the heavy table (4 slots per
-    // entry, load <= 1/4, with the list bounds of N+(u)) and the light tables
+    // entry, load <= 1/4, with the list bounds of N+(u)) and the light tables with
+    // the entries of 32 arcs each
     const size_t queue_bytes = sizeof(HitQueue) * kTW;
-    const size_t light_bytes = (size_t)kTW * kLightSlots * sizeof(uint32_t);
+    const size_t light_bytes = (size_t)kTW * (kLightSlots * sizeof(uint32_t) + 32 * sizeof(uint4));
     int cap = 8;
     while (cap < pl->max_deg && cap < kHeavyCap) cap *= 2;
     pl->heavy_cap = cap;

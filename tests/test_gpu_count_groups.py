@@ -1,5 +1,5 @@
-"""Triangle counts per vertex and per edge where light vertices stream groups of 32
-short lists as one sequence: out-degrees and in-lists around the group and slab
+"""Triangle counts per vertex and per edge, and edge-once compression, where light
+vertices stream groups of 32 short lists as one sequence: out-degrees and in-lists around the group and slab
 sizes, and lists left out because the other end streams them."""
 import numpy as np
 import pytest
@@ -39,16 +39,20 @@ def _joined(k, r):
                              torch.from_numpy(np.concatenate(hi).astype(np.int64)))
 
 
+def _same(sg, G, g, p):
+    for kern in ("tr_mincount", "tr_eo", "tr_eo_mincount"):
+        off, col, _ = sg.compress(G, kern, p, 5).download()
+        o_off, o_col, _ = oracle.compress(g, kern, p, 5)
+        assert np.array_equal(off, o_off) and np.array_equal(col, o_col)
+
+
 @pytest.mark.parametrize("k,r", [(3, 0), (32, 0), (33, 0), (34, 0), (64, 0), (65, 0), (66, 0), (9, 31), (9, 32),
                                  (9, 33), (31, 70), (33, 150), (20, 400)])
 def test_joined(sg, ctx, k, r):
     g = _joined(k, r)
     G = sg.Graph.from_csr(ctx, g)
     assert np.array_equal(sg.vertex_triangle_counts(G).cpu().numpy(), oracle.vertex_triangle_counts(g))
-    H = sg.compress(G, "tr_mincount", 1.0, 5)
-    off, col, _ = H.download()
-    o_off, o_col, _ = oracle.compress(g, "tr_mincount", 1.0, 5)
-    assert np.array_equal(off, o_off) and np.array_equal(col, o_col)
+    _same(sg, G, g, 1.0)
 
 
 @pytest.mark.parametrize("n,q", [(60, 0.5), (150, 0.3), (150, 0.6), (900, 0.05)])
@@ -56,7 +60,4 @@ def test_random(sg, ctx, n, q):
     g = gg.gnp(n, q, seed=n)
     G = sg.Graph.from_csr(ctx, g)
     assert np.array_equal(sg.vertex_triangle_counts(G).cpu().numpy(), oracle.vertex_triangle_counts(g))
-    H = sg.compress(G, "tr_mincount", 0.5, 5)
-    off, col, _ = H.download()
-    o_off, o_col, _ = oracle.compress(g, "tr_mincount", 0.5, 5)
-    assert np.array_equal(off, o_off) and np.array_equal(col, o_col)
+    _same(sg, G, g, 0.5)

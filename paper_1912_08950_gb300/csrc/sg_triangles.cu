@@ -1774,10 +1774,12 @@ constexpr int64_t kEoOneLaunch = 1 << 20;
 __device__ __forceinline__ bool considered_now(const uint32_t *c, uint32_t e) { return (__ldcg(c + (e >> 5)) >> (e & 31)) & 1u; }
 
 // All threads of the cluster arrive, with what they wrote, before any leaves.
+// Not the .aligned form, which needs whole warps: the lanes come from loops of
+// their own lengths, and nothing makes them meet again before this.
 __device__ __forceinline__ void cluster_barrier() {
     __threadfence();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // Append the CTA's survivors: this thread's slot in the list (all threads call).

@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
                 __threadfence();
             }
             if (__shfl_sync(kFull, (int)last, 0)) {
+                __syncwarp();  // a shuffle orders no memory: the lanes' reads below come after lane 0's fence
                 const float *part = a.hubs.part + (size_t)first * (split ? kPrWarps : 1);
                 float s = 0.f, one = 0.f;  // the row's sum, a chunk's
                 for (int p0 = 0; p0 < parts; p0 += 32) {

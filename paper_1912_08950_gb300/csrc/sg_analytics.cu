@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
     auto rank_of = [&](uint32_t i) {
         float v;
         const float *base = kHot && i < (uint32_t)a.hot ? s_y : a.y;
-        asm volatile("ld.f32 %0, [%1];" : "=f"(v) : "l"(base + i));
+        asm volatile("ld.f32 %0, [%1];" : "=f"(v) : "l"(base + i) : "memory");  // not before the barrier above
         return v;
     };
     double res = 0.0;

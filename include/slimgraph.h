@@ -156,6 +156,12 @@ sg_status sg_ctx_reset_profile(sg_ctx *ctx);
  * enumerates the triangles again).  The result is the same in every setting;
  * only time and memory change. */
 sg_status sg_ctx_set_eo_list_capacity(sg_ctx *ctx, int64_t records);
+/* The rounds over a short Edge-Once list run in one launch, a cluster of 16
+ * thread blocks.  on == 0 gives every round its own launches, as happens by
+ * itself on a device, or a partition of one, that cannot host such a cluster.
+ * The result is the same; only time changes.
+ * Errors: SG_ERR_INVALID_ARG (ctx == NULL). */
+sg_status sg_ctx_set_eo_one_launch(sg_ctx *ctx, int on);
 /* The Edge-Once lists live in device workspaces that the context keeps and
  * reuses across calls (grown when a call needs more).  This frees them, in
  * stream order; the next Edge-Once call allocates them again.

@@ -326,6 +326,12 @@ sg_status sg_ctx_set_eo_list_capacity(sg_ctx *ctx, int64_t records) {
     return SG_OK;
 }
 
+sg_status sg_ctx_set_eo_one_launch(sg_ctx *ctx, int on) {
+    if (!ctx) return fail(SG_ERR_INVALID_ARG, "ctx is NULL");
+    C_(ctx)->eo_one_launch = on != 0;
+    return SG_OK;
+}
+
 sg_status sg_ctx_release_workspace(sg_ctx *ctx) {
     if (!ctx) return fail(SG_ERR_INVALID_ARG, "ctx is NULL");
     Ctx *c = C_(ctx);

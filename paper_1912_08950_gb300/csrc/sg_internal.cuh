@@ -47,6 +47,8 @@ struct Ctx {
     uint64_t eo_passes = 0;                // edge-once enumeration passes
     uint64_t eo_list_passes = 0;           // ... that listed triangles
     int64_t eo_list_cap = 0;               // 0 auto, -1 off, > 0 records
+    bool eo_one_launch = true;             // sg_ctx_set_eo_one_launch
+    signed char eo_cluster[3] = {-1, -1, -1};  // whether its kernels' cluster fits the device; -1 not asked yet
     bool profiling = false;
     uint32_t scan_hold = 0;                // test hook (sg_ctx_set_scan_hold): 0 off
     // grow-only device workspaces kept across calls (edge-once list and active

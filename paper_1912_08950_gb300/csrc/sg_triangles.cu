@@ -2143,6 +2143,31 @@ static TriArgs base_args(Ctx *c, const Oriented &o) {
     return a;
 }
 
+struct EoBufs {
+    uint32_t *considered = nullptr;
+    // lctr: [kEoBuckets] bucket fills, [kEoBuckets] bucket counts, an out length, then the overflow bits
+    unsigned long long *resv = nullptr, *lctr = nullptr;
+};
+
+// Whether the device (or the partition of it that this process has) can host
+// eo_rounds_kernel's cluster: sixteen CTAs of a whole SM each are more than any
+// device must take, so this is asked once per context, and the rounds' own
+// launches do the work where the answer is no.
+static bool eo_cluster_fits(Ctx *c, int choice, void (*kernel)(EoRun)) {
+    signed char &fits = c->eo_cluster[choice];
+    if (fits < 0) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(kEoCluster);
+        cfg.blockDim = dim3(kEoCta);
+        cfg.stream = c->stream;
+        int clusters = 0;
+        fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+               cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters > 0;
+        (void)cudaGetLastError();
+    }
+    return fits != 0;
+}
+
 // Edge-once rounds.  Round r lets the live selected triangles with
 // r2 < theta_r = 2^(27+r) bid (all of them from round 5 on).  A bidder that
 // holds all three reservations is the smallest live triangle on each of its
@@ -2159,13 +2184,12 @@ static TriArgs base_args(Ctx *c, const Oriented &o) {
 // the round still completes from those bids, accepting from the edges' side;
 // later rounds enumerate and bid directly and retry the list once the live
 // triangles fit.
-static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, const Plan &pl, TriArgs a) {
+static sg_status eo_run(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, const Plan &pl, TriArgs a, EoBufs &buf) {
     const size_t m = (size_t)std::max<int64_t>(o.m, 1);
     const int choice = k == SG_TR_EO_MAXW ? kChoiceMaxw : (k == SG_TR_EO_MINCOUNT ? kChoiceMinCount : kChoiceRandom);
-    uint32_t *considered = nullptr;
+    uint32_t *&considered = buf.considered;
     const size_t cwords = (m + 31) / 32;
-    // lctr: [kEoBuckets] bucket fills, [kEoBuckets] bucket counts, an out length, then the overflow bits
-    unsigned long long *resv = nullptr, *lctr = nullptr;
+    unsigned long long *&resv = buf.resv, *&lctr = buf.lctr;
     const size_t lctr_bytes = (2 * kEoBuckets + 1) * sizeof(unsigned long long) + sizeof(int);
     int *lovf = nullptr;
     uint4 *L = nullptr;    // bucketed list written by the enumeration (workspace kWsList)
@@ -2392,7 +2416,10 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
         // ---- a list this short: all rounds left in one launch
         int64_t rest = lenA;
         for (int b = next_bucket; b < top; ++b) rest += used[b];
-        if (rest <= kEoOneLaunch) {
+        auto one = choice == kChoiceMaxw ? eo_rounds_kernel<kChoiceMaxw>
+                   : choice == kChoiceMinCount ? eo_rounds_kernel<kChoiceMinCount>
+                                               : eo_rounds_kernel<kChoiceRandom>;
+        if (rest <= kEoOneLaunch && c->eo_one_launch && eo_cluster_fits(c, choice, one)) {
             TriRec *B = nullptr;
             const int bslot = a_slot == kWsActive0 ? kWsActive1 : kWsActive0;
             const size_t bytes = (size_t)std::max<int64_t>(rest, 1) * sizeof(TriRec);
@@ -2429,13 +2456,9 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
                 r.wp = a.wp;
                 r.k0 = a.k0;
                 r.k1 = a.k1;
-                auto kernel = choice == kChoiceMaxw ? eo_rounds_kernel<kChoiceMaxw>
-                              : choice == kChoiceMinCount ? eo_rounds_kernel<kChoiceMinCount>
-                                                          : eo_rounds_kernel<kChoiceRandom>;
-                SG_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
                 {
                     SG_LAUNCH(c, "tri_eo_rounds");
-                    kernel<<<kEoCluster, kEoCta, 0, c->stream>>>(r);
+                    one<<<kEoCluster, kEoCta, 0, c->stream>>>(r);
                 }
                 SG_CUDA(cudaGetLastError());
                 SG_CUDA(cudaMemcpyAsync(c->h_pinned, r.rounds, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
@@ -2526,10 +2549,15 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
         }
         SG_CUDA(cudaGetLastError());
     }
+    return st;
+}
 
-    dfree(c, lctr);
-    dfree(c, considered);
-    dfree(c, resv);
+static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, const Plan &pl, const TriArgs &a) {
+    EoBufs buf;
+    const sg_status st = eo_run(c, g, o, k, pl, a, buf);  // (which returns in its middle on an error)
+    dfree(c, buf.lctr);
+    dfree(c, buf.considered);
+    dfree(c, buf.resv);
     return st;
 }
 

@@ -19,9 +19,10 @@ def sg():
     return m
 
 
-def _run(sg, g, kern, p, cap=0):
+def _run(sg, g, kern, p, one_launch=True):
     ctx = sg.Context(0)
-    ctx.set_eo_list_capacity(cap)
+    if not one_launch:
+        ctx.set_eo_one_launch(False)
     ctx.set_profiling(True)
     G = sg.Graph.from_csr(ctx, g)
     H = sg.compress(G, kern, p, 7)
@@ -52,3 +53,12 @@ def test_long_list_ends_in_one_launch(sg):
     launches, stats = _run(sg, gg.rmat(15, 24, seed=15), "tr_eo", 1.0)
     assert stats["eo_listed"] > ONE_LAUNCH
     assert launches["tri_eo_fresh_reserve"] >= 1 and launches["tri_eo_rounds"] == 1
+
+
+# as on a device that cannot host the cluster: every round in launches of its own
+@pytest.mark.parametrize("name", ["k7", "rmat10"])
+@pytest.mark.parametrize("kern", ["tr_eo", "tr_eo_maxw", "tr_eo_mincount"])
+def test_without_the_cluster(sg, name, kern):
+    g = {"k7": lambda: gg.complete(7), "rmat10": lambda: gg.rmat(10, 16, seed=12)}[name]()
+    launches, stats = _run(sg, gg.attach_weights(g, seed=1), kern, 1.0, one_launch=False)
+    assert launches["tri_eo_rounds"] == 0 and launches["tri_eo_fresh_reserve"] >= 1

@@ -86,7 +86,6 @@ struct PrArgs {
     float *y_new;
     float *x_prev;         // the values before the last iteration
     float *x_out;
-    double *resid_part;    // per CTA
     PrHubs hubs;
     const uint32_t *medium;  // rows of more than kShortRow arcs that are no hubs, in any order
     // the rank of the degree-0 vertices: how many each virtual lane sums, the
@@ -133,8 +132,7 @@ __device__ __forceinline__ void pr_dangling_sums(const uint32_t *lane_cnt, int v
     }
 }
 
-// What an iteration stores besides y: nothing, x (the one before the last), or
-// x_out and the FP64 partial L1 residual |x_out - x_prev| (the last).
+// What an iteration stores: y, y and x (the one before the last), or x_out (the last).
 enum class PrStore { kNone, kPrev, kLast };
 
 template <bool kHot, PrStore S>
@@ -143,7 +141,6 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
     __shared__ float s_acc[kPrCta / 32][32];
     __shared__ longlong2 s_row[kPrCta / 32][32];  // first arc minus its number, and the row, of the short rows
     __shared__ float s_red[kPrThreads];
-    __shared__ double s_res[kPrCta / 32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if constexpr (kHot) {
         const int quads = (a.hot + 3) >> 2;  // (y has room for whole ones)
@@ -162,13 +159,11 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
         asm volatile("ld.f32 %0, [%1];" : "=f"(v) : "l"(base + i) : "memory");  // not before the barrier above
         return v;
     };
-    double res = 0.0;
     auto finish = [&](int64_t v, int64_t deg, float s) {
         const float xv = a.base + a.damping * (s + dterm);
         if (S == PrStore::kPrev) a.x_prev[v] = xv;
         if (S == PrStore::kLast) {
             a.x_out[v] = xv;
-            res += fabs((double)xv - (double)__ldg(a.x_prev + v));
         } else if (deg > 0) {
             a.y_new[a.pos ? __ldg(a.pos + v) : (uint32_t)v] = xv / (float)deg;
         }
@@ -427,16 +422,29 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
             if (v < a.n && shortr) finish(v, deg, s);
         }
     }
-    if constexpr (S == PrStore::kLast) {
+}
+
+// FP64 partial L1 residual |x - x_prev| per CTA: a thread adds the vertices a
+// grid apart, then a fixed tree over lanes and warps.  (A pass of its own, 8n
+// bytes once per call: in the last iteration the rows a lane gets, and so the
+// order of the sum, depend on the schedule.  The sum is exact, and any order
+// gives the same, only while the terms' bits fit 53, which damping near 1 or
+// very many vertices exceed.)
+__global__ void __launch_bounds__(kPrThreads) pr_residual_kernel(const float *__restrict__ x,
+                                                                const float *__restrict__ x_prev, int64_t n,
+                                                                double *__restrict__ parts) {
+    __shared__ double s[kPrWarps];
+    double res = 0.0;
+    for (int64_t v = (int64_t)blockIdx.x * kPrThreads + threadIdx.x; v < n; v += (int64_t)gridDim.x * kPrThreads)
+        res += fabs((double)__ldg(x + v) - (double)__ldg(x_prev + v));
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(kFull, res, o);
-        if (lane == 0) s_res[warp] = res;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double br = 0.0;
-            for (int i = 0; i < kPrCta / 32; ++i) br += s_res[i];
-            a.resid_part[blockIdx.x] = br;
-        }
+    for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(kFull, res, o);
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = res;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double br = 0.0;
+        for (int i = 0; i < kPrWarps; ++i) br += s[i];
+        parts[blockIdx.x] = br;
     }
 }
 
@@ -654,12 +662,11 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
         total += (bytes + 255) & ~(size_t)255;
         return at;
     };
-    const size_t grid_max = (size_t)c->num_sms;
     const size_t zero_at = room((4 + kDegBuckets / 2 + 1) * sizeof(unsigned long long));  // counts, hist, work
     const size_t done_at = room(max_hubs * sizeof(unsigned int));
     const size_t zero_end = total;
     const size_t y_at[2] = {room(sizeof(float) * (nn + 4)), room(sizeof(float) * (nn + 4))};
-    const size_t x_at = room(sizeof(float) * nn), res_at = room(sizeof(double) * (grid_max + 1));
+    const size_t x_at = room(sizeof(float) * nn), res_at = room(sizeof(double) * ((size_t)vblocks + 1));
     const size_t cnt_at = room(sizeof(uint32_t) * (size_t)vblocks * kPrThreads);
     const size_t w_at[2] = {room(sizeof(float) * (size_t)vblocks * kPrWarps), room(sizeof(float) * (size_t)vblocks * kPrWarps)};
     const size_t hubs_at = room(sizeof(uint32_t) * max_hubs), first_at = room(sizeof(int) * max_hubs);
@@ -685,7 +692,7 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
                     reinterpret_cast<unsigned int *>(buf + done_at)};
     a.medium = reinterpret_cast<uint32_t *>(buf + med_at);
     a.x_prev = reinterpret_cast<float *>(buf + x_at);
-    a.resid_part = reinterpret_cast<double *>(buf + res_at);
+    double *parts = reinterpret_cast<double *>(buf + res_at);  // of the residual, then their sum
     a.lane_cnt = reinterpret_cast<uint32_t *>(buf + cnt_at);
     a.hot = hot ? hot_cap : 0;
     a.pos = pos;
@@ -752,11 +759,15 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     }
     {
         SG_LAUNCH(c, "pr_reduce");
-        reduce_parts_kernel<double><<<1, kPrThreads, 0, c->stream>>>(a.resid_part, grid, a.resid_part + grid_max);
+        pr_residual_kernel<<<vblocks, kPrThreads, 0, c->stream>>>(x_out, a.x_prev, n, parts);
+    }
+    {
+        SG_LAUNCH(c, "pr_reduce");
+        reduce_parts_kernel<double><<<1, kPrThreads, 0, c->stream>>>(parts, vblocks, parts + vblocks);
     }
     e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(c->h_pinned, a.resid_part + grid_max, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+        e = cudaMemcpyAsync(c->h_pinned, parts + vblocks, sizeof(double), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess) std::memcpy(resid, c->h_pinned, sizeof(double));
     release();

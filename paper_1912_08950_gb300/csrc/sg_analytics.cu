@@ -664,8 +664,10 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     };
     const size_t zero_at = room((4 + kDegBuckets / 2 + 1) * sizeof(unsigned long long));  // counts, hist, work
     const size_t done_at = room(max_hubs * sizeof(unsigned int));
-    const size_t zero_end = total;
+    // y of the degree-0 vertices is never written: an arc into one, which only a
+    // CSR that is not symmetric has, adds nothing
     const size_t y_at[2] = {room(sizeof(float) * (nn + 4)), room(sizeof(float) * (nn + 4))};
+    const size_t zero_end = total;
     const size_t x_at = room(sizeof(float) * nn), res_at = room(sizeof(double) * ((size_t)vblocks + 1));
     const size_t cnt_at = room(sizeof(uint32_t) * (size_t)vblocks * kPrThreads);
     const size_t w_at[2] = {room(sizeof(float) * (size_t)vblocks * kPrWarps), room(sizeof(float) * (size_t)vblocks * kPrWarps)};

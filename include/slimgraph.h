@@ -179,6 +179,15 @@ sg_status sg_ctx_release_workspace(sg_ctx *ctx);
  * Errors: SG_ERR_INVALID_ARG (ctx == NULL). */
 sg_status sg_ctx_set_scan_hold(sg_ctx *ctx, uint32_t spin_limit);
 
+/* Test hook for the SG_ERR_OOM contract (the paper has no counterpart).  With
+ * bytes > 0 the context's stream-ordered allocations behave as on a device
+ * with that much memory free: one that would take the sum of those made since
+ * this call and not freed above it fails.  Calls fall back as far as they can
+ * (scratch that only saves time is done without) and then return SG_ERR_OOM.
+ * 0 (the default) turns it off.
+ * Errors: SG_ERR_INVALID_ARG (ctx == NULL). */
+sg_status sg_ctx_set_alloc_limit(sg_ctx *ctx, uint64_t bytes);
+
 /* Device memory free for new work on CUDA device `device`, in bytes: what
  * the driver reports free (cudaMemGetInfo) plus what the device's default
  * stream-ordered pool holds from freed allocations but does not use (this

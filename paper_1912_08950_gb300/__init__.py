@@ -76,6 +76,7 @@ _SIGS = {
     "sg_device_free_memory": [_int, C.POINTER(C.c_uint64)],
     "sg_ctx_set_eo_one_launch": [_vp, C.c_int],
     "sg_ctx_set_scan_hold": [_vp, C.c_uint32],
+    "sg_ctx_set_alloc_limit": [_vp, C.c_uint64],
     "sg_kernel_arch": [_int, C.POINTER(C.c_int)],
     "sg_graph_from_device": [_vp, C.POINTER(CsrView), _int, _int, _PP],
     "sg_graph_from_host": [_vp, _i64, _i64, _vp, _vp, _vp, _PP],
@@ -196,6 +197,10 @@ class Context:
     def set_scan_hold(self, spin_limit: int):
         """Test hook: make every prefix scan's first wait run out (0: off)."""
         _check(_lib.sg_ctx_set_scan_hold(self.handle, int(spin_limit)))
+
+    def set_alloc_limit(self, nbytes: int):
+        """Test hook: the context's allocations from now on may hold `nbytes` at a time (0: off)."""
+        _check(_lib.sg_ctx_set_alloc_limit(self.handle, int(nbytes)))
 
     def release_workspace(self):
         """Free the edge-once list workspaces the context keeps between calls."""

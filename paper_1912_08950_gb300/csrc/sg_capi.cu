@@ -61,15 +61,17 @@ Scratch::Scratch(Ctx *c_, size_t bytes) : c(c_) {
 
 Scratch::~Scratch() {
     if (!c) return;
-    (void)cudaFreeAsync(c->arena, c->stream);
+    void *p = c->arena;
     c->arena = nullptr;
     c->arena_bytes = c->arena_used = 0;
+    dfree(c, p);
 }
 
 sg_status dalloc_own(Ctx *c, void **p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMallocAsync(p, bytes, c->stream);
+    const bool over = c->alloc_limit && bytes > c->alloc_limit - std::min(c->alloc_limit, c->alloc_live);
+    cudaError_t e = over ? cudaErrorMemoryAllocation : cudaMallocAsync(p, bytes, c->stream);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         *p = nullptr;
@@ -77,12 +79,24 @@ sg_status dalloc_own(Ctx *c, void **p, size_t bytes) {
                     std::string("device allocation of ") + std::to_string(bytes) + " bytes failed: " +
                         cudaGetErrorString(e));
     }
+    if (c->alloc_limit) {
+        c->alloc_sizes[*p] = bytes;
+        c->alloc_live += bytes;
+    }
     return SG_OK;
 }
 
 void dfree(Ctx *c, void *p) {
     if (c->arena && p >= c->arena && p < c->arena + c->arena_bytes) return;  // goes with the call's scratch
-    if (p) (void)cudaFreeAsync(p, c->stream);
+    if (!p) return;
+    if (c->alloc_limit) {
+        const auto it = c->alloc_sizes.find(p);
+        if (it != c->alloc_sizes.end()) {
+            c->alloc_live -= it->second;
+            c->alloc_sizes.erase(it);
+        }
+    }
+    (void)cudaFreeAsync(p, c->stream);
 }
 
 sg_status ws_get(Ctx *c, int slot, size_t bytes, void **p) {
@@ -179,8 +193,20 @@ static sg_status compress_tr(Ctx *c, const Graph *g, sg_kernel k, double p, uint
     // kernel sizes its list by the memory free before they are allocated
     const bool eo = k == SG_TR_EO || k == SG_TR_EO_MAXW || k == SG_TR_EO_MINCOUNT;
     Graph *h = nullptr;
-    if (st == SG_OK && !eo) st = new_graph(c, g->n, g->nnz, g->w != nullptr, &h);
+    if (st == SG_OK && !eo && new_graph(c, g->n, g->nnz, g->w != nullptr, &h) != SG_OK) {
+        set_error("");
+        h = nullptr;
+    }
     if (st == SG_OK) st = tr_mark(c, g, o, k, p, seed, del, h);
+    if (st == SG_ERR_OOM && h) {
+        // the marking's own arrays do not fit beside the output: mark in one pass,
+        // which needs none of its arrays, and allocate it after that (flags set so
+        // far are right ones and stay)
+        delete_graph(c, h);
+        h = nullptr;
+        set_error("");
+        st = tr_mark(c, g, o, k, p, seed, del, nullptr);
+    }
     if (st == SG_OK) {
         st = resolve_mask(c, g, rm, o, del, &h);
         if (st == SG_OK) *out = h;
@@ -348,6 +374,15 @@ sg_status sg_ctx_release_workspace(sg_ctx *ctx) {
 sg_status sg_ctx_set_scan_hold(sg_ctx *ctx, uint32_t spin_limit) {
     if (!ctx) return fail(SG_ERR_INVALID_ARG, "ctx is NULL");
     C_(ctx)->scan_hold = spin_limit;
+    return SG_OK;
+}
+
+sg_status sg_ctx_set_alloc_limit(sg_ctx *ctx, uint64_t bytes) {
+    if (!ctx) return fail(SG_ERR_INVALID_ARG, "ctx is NULL");
+    Ctx *c = C_(ctx);
+    c->alloc_limit = (size_t)bytes;
+    c->alloc_live = 0;
+    c->alloc_sizes.clear();
     return SG_OK;
 }
 

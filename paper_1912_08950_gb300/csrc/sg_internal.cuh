@@ -5,6 +5,7 @@
 
 #include <cstdint>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "slimgraph.h"
@@ -51,6 +52,9 @@ struct Ctx {
     signed char eo_cluster[3] = {-1, -1, -1};  // whether its kernels' cluster fits the device; -1 not asked yet
     bool profiling = false;
     uint32_t scan_hold = 0;                // test hook (sg_ctx_set_scan_hold): 0 off
+    // test hook (sg_ctx_set_alloc_limit): the limit (0 off) and what is allocated since it was set
+    size_t alloc_limit = 0, alloc_live = 0;
+    std::unordered_map<void *, size_t> alloc_sizes;
     // grow-only device workspaces kept across calls (edge-once list and active
     // lists), so that repeated calls do not churn the stream-ordered pool
     void *ws[3] = {nullptr, nullptr, nullptr};
@@ -272,7 +276,8 @@ sg_status low_degree(Ctx *c, const Graph *g, uint32_t *new_to_old, Graph **out);
 
 // triangles (sg_triangles.cu)
 // sets the deletion flags of one TR kernel; h: the output graph, allocated but
-// not written yet (union kernels borrow its arrays), or NULL (edge-once)
+// not written yet (union kernels borrow its arrays), or NULL (edge-once; a
+// union kernel then makes one pass)
 sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double p, uint64_t seed, uint32_t *del,
                   const Graph *h);
 sg_status tr_count(Ctx *c, const Graph *g, const Oriented &o, int64_t *count, int64_t *probes, int64_t *maxdeg,

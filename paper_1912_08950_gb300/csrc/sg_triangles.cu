@@ -1160,7 +1160,7 @@ __device__ __forceinline__ void stream_lists(const TriArgs &a, const TabCtx &t, 
 // about 40 elements on R-MAT graphs) and its lane takes the next arc.  The
 // records of one claim load while the windows stream, the ids of the next with
 // them.
-template <Mode M, bool kAlive>
+template <Mode M, bool kAlive, bool kRec>
 __device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, int *next, uint32_t ou, int64_t ib, int nin,
                                             int ax, UnionScratch &q, QState &qs, unsigned long long &probes,
                                             unsigned long long &tris, bool count) {
@@ -1200,10 +1200,13 @@ __device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, i
             dead = arc_deleted(a.del, ge);
             if constexpr (kAlive) {
                 rec = __ldg(a.arec + gv);
-            } else {
+            } else if constexpr (kRec) {
                 const uint2 r = __ldg(a.vrec + (size_t)gv * a.vstep);
                 rec.x = r.x;
                 rec.y = r.y;
+            } else {
+                rec.x = (uint32_t)__ldg(a.offp + gv);
+                rec.y = (uint32_t)__ldg(a.offp + gv + 1) - rec.x;
             }
         }
         if (gc < items) {
@@ -1287,7 +1290,10 @@ __device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, i
 // three CTAs with more registers: s22 3.14 -> 2.84 ms, s26 51.6 -> 46.4,
 // max-weight on the Chung-Lu graph 1.54 -> 1.38; the first pass is slower at
 // three (s22 16.4 -> 17.0, s26 248 -> 276) and at five (17.0, 253).
-template <Mode M, int TW, bool kAlive>
+// kRec: vertex records to read; without them (no memory left for them) the
+// offsets are read instead, in an instance of its own, since choosing at run time
+// spills in the first pass (s22 23.6 -> 24.4 ms a call, s26 627 -> 651).
+template <Mode M, int TW, bool kAlive, bool kRec = true>
 __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri_union_kernel(TriArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_next;
@@ -1362,7 +1368,7 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri
                 }
                 __syncthreads();
                 t.stash_n = min(*t.tb.stash_n, kStash);
-                stream_arcs<M, kAlive>(a, t, &s_next, (uint32_t)ou, ib, nin, ax, q, qst, probes, tris, c0 == 0);
+                stream_arcs<M, kAlive, kRec>(a, t, &s_next, (uint32_t)ou, ib, nin, ax, q, qst, probes, tris, c0 == 0);
                 flush_union<M>(a, t, q, qst, tris);
                 __syncthreads();  // the table is rebuilt for the next chunk or vertex
             }
@@ -1423,8 +1429,9 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri
                 }
                 __syncwarp();
                 t.stash_n = min(*t.tb.stash_n, kStash);
-                stream_arcs<M, false>(a, t, &s_lnext[warp], t.tbase, nin > 0 ? __ldg(a.offs + t.u) - (int64_t)t.tbase : 0,
-                                      nin, 0, q, qst, probes, tris, true);
+                stream_arcs<M, false, kRec>(a, t, &s_lnext[warp], t.tbase,
+                                            nin > 0 ? __ldg(a.offs + t.u) - (int64_t)t.tbase : 0, nin, 0, q, qst,
+                                            probes, tris, true);
                 flush_union<M>(a, t, q, qst, tris);
                 __syncwarp();
             }
@@ -1901,11 +1908,9 @@ struct Plan {
     uint32_t *heavy = nullptr;
     unsigned long long *buckets = nullptr;  // counts [kKeys], fills [kKeys]
     uint32_t *din = nullptr;                // in-arcs streamed from the head's side, per vertex
-    bool records = false;                   // union passes: off+ and d+ of vertex v at vrec[v * vstep]
-    uint2 *vrec = nullptr;
-    int vstep = 1;
-    void *rec_own = nullptr;                // the records' allocation, if they have one
-    uint4 *arec = nullptr;                  // the same as 16-byte records (vstep 2), if there is room for them
+    bool records = false;                   // union passes: 16-byte vertex records wanted
+    uint4 *arec = nullptr;                  // the records, if there is room for them; off+ and d+ first
+    void *rec_own = nullptr;                // their allocation, if they have one
     uint2 *inl = nullptr;                   // their (tail, arc), at offs(v) - offp(v) per vertex
     const int64_t *offs = nullptr;          // symmetric offsets of the graph
     int64_t n_heavy = 0, max_deg = 0;
@@ -1934,7 +1939,6 @@ static void free_plan(Ctx *c, Plan *pl) {
     dfree(c, pl->din);
     dfree(c, pl->rec_own);
     pl->rec_own = nullptr;
-    pl->vrec = nullptr;
     pl->arec = nullptr;
     pl->heavy = nullptr;
     pl->buckets = nullptr;
@@ -1960,20 +1964,16 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
     if (st == SG_OK) st = dalloc(c, (void **)&pl->buckets, sizeof(unsigned long long) * 2 * kKeys);
     if (st == SG_OK) st = dalloc(c, (void **)&pl->din, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
     if (st == SG_OK && pl->records) {
-        // 16-byte records in the unused half of E+'s column array (room for nnz
-        // = 2m entries), or else 8-byte ones and no second pass
+        // in the unused half of E+'s column array (room for nnz = 2m entries) if it
+        // holds them (16 n <= 4 m: a mean degree of 8), in memory of their own otherwise
         const uintptr_t b = ((uintptr_t)(o.col + o.m) + 15) & ~(uintptr_t)15, e = (uintptr_t)(o.col + 2 * o.m);
         if (o.m > 0 && b + sizeof(uint4) * (size_t)o.n <= e) {
             pl->arec = reinterpret_cast<uint4 *>(b);
-            pl->vstep = 2;
         } else if (dalloc(c, &pl->rec_own, sizeof(uint4) * (size_t)std::max<int64_t>(o.n, 1)) == SG_OK) {
             pl->arec = static_cast<uint4 *>(pl->rec_own);
-            pl->vstep = 2;
         } else {
             set_error("");
-            st = dalloc(c, &pl->rec_own, sizeof(uint2) * (size_t)std::max<int64_t>(o.n, 1));
         }
-        pl->vrec = pl->arec ? reinterpret_cast<uint2 *>(pl->arec) : static_cast<uint2 *>(pl->rec_own);
     }
     if (st != SG_OK) return st;
     pl->inl = o.inl;  // the orientation's reverse list (not owned by the plan)
@@ -1982,8 +1982,8 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((o.n + 255) / 256, (int64_t)c->num_sms * 8));
     if (o.n > 0) {
         SG_LAUNCH(c, "tri_classify");
-        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, offs, pl->din, pl->vrec, pl->vstep,
-                                                                       o.n, pl->light_max,
+        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, offs, pl->din,
+                                                                       reinterpret_cast<uint2 *>(pl->arec), 2, o.n, pl->light_max,
                                                                        pl->light_items, (int64_t)kHeavyCap,
                                                                        pl->buckets, c->d_ctr);
     }
@@ -2085,8 +2085,8 @@ static sg_status launch_pass(Ctx *c, void (*hub)(TriArgs), void (*main)(TriArgs)
     a.light_items = pl.light_items;
     a.offs = pl.offs;
     a.din = pl.din;
-    a.vrec = pl.vrec;
-    a.vstep = pl.vstep;
+    a.vrec = reinterpret_cast<const uint2 *>(pl.arec);
+    a.vstep = 2;
     a.inl = pl.inl;
     a.work = c->d_ctr + kCtrAux;
     if (pl.n_hubs > 0) {
@@ -2108,11 +2108,19 @@ static sg_status launch_enum(Ctx *c, const TriArgs &a, const Plan &pl) {
 }
 
 // The two passes of a union kernel (see tri_union_kernel), h the output graph.
-// Without the second pass's scratch the first streams every list whole.
+// Without it or the second pass's scratch the first streams every list whole;
+// without the records too, in the one instance that does without them (long
+// tables in chunks: memory is short here, not time).
 template <Mode M>
 static sg_status launch_union(Ctx *c, const Oriented &o, TriArgs a, const Plan &pl, const Graph *h) {
+    if (pl.arec == nullptr) {
+        Plan main = pl;
+        main.n_hubs = 0;
+        a.short_max = INT_MAX;
+        return launch_pass(c, nullptr, tri_union_kernel<M, kTW, false, false>, 0, pl.usmem, a, main, "", "tri_enum");
+    }
     AliveArcs al;
-    bool two = pl.max_deg > kShortList && pl.arec != nullptr;
+    bool two = h != nullptr && pl.max_deg > kShortList;
     if (two && alive_alloc(c, o, h, &al) != SG_OK) {
         set_error("");
         two = false;
@@ -2241,6 +2249,7 @@ static sg_status eo_run(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, 
             cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
             fr += (size_t)(reserved - used);
         (void)cudaGetLastError();
+        if (c->alloc_limit) fr = std::min(fr, c->alloc_limit - std::min(c->alloc_limit, c->alloc_live));
         for (int i = 0; i < 3; ++i) fr += c->ws_bytes[i];  // the context's workspaces are reused
         int64_t cap = (int64_t)(fr / 4 / sizeof(uint4));
         if (c->eo_list_cap > 0) cap = std::min<int64_t>(cap, c->eo_list_cap);
@@ -2571,7 +2580,7 @@ sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double
     } else {
         pl.light_max = kUnionLightMax;
         pl.light_items = kUnionLightItems;
-        pl.records = true;
+        pl.records = h != nullptr;
     }
     sg_status st = make_plan(c, o, g->off, &pl);
     TriArgs a = base_args(c, o);
@@ -2593,7 +2602,7 @@ sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double
             pl = Plan{};
             pl.light_max = kUnionLightMax;
             pl.light_items = kUnionLightItems;
-            pl.records = true;
+            pl.records = h != nullptr;
             st = make_plan(c, o, g->off, &pl);
         }
     }

@@ -1,0 +1,69 @@
+"""Triangle kernels where device memory is short: what fits a call that marks in one
+pass and allocates its output afterwards must still run, with the same result."""
+import numpy as np
+import pytest
+import torch
+
+import graphgen as gg
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sg():
+    import paper_1912_08950_gb300 as m
+
+    return m
+
+
+def _one_pass_peak(n, nnz, weighted, kernel):
+    """Bytes of the arrays of a call that marks in one pass over all lists: row map,
+    orientation and reverse list, then the larger of the marking's arrays (a byte of
+    flag per edge; heavy and in-degree lists, counters of min-count) and of the rebuild's
+    (the flags again, the output, keep bits, prefixes)."""
+    m, nc = nnz // 2, -(-nnz // 256)
+    base = 4 * (nc + 1) + 8 * (n + 1) + 4 * nnz + 4 * (8 * nc + 1) + 8 * (nc + 1) + 8 * (nnz - m)
+    if kernel == "tr_maxw":
+        base += 4 * nnz
+    mark = m + 8 * n + 1664 + (4 * m if kernel == "tr_mincount" else 0)
+    out = 8 * (n + 1) + 4 * nnz * (2 if weighted else 1)
+    rebuild = m + m // 8 + out + 4 * (8 * nc + 1) + 8 * (nc + 1) + 8 * (nc // 1024 + 2)
+    return base + max(mark, rebuild)
+
+
+def _padded(g, n):
+    """g with isolated vertices up to n."""
+    off = torch.cat([g.off, g.off[-1:].expand(n - g.n)])
+    return gg.CSR(n, off.contiguous(), g.col, g.w)
+
+
+# the vertices' records in the orientation's unused half (mean degrees 28 and 9) and not (4.5 and
+# 0.3); all too large for the scratch to be one allocation; a dense core gives lists for a second pass
+GRAPHS = {
+    "rmat16": lambda: gg.rmat(16, 16, seed=1),
+    "deg9": lambda: _padded(gg.rmat(16, 16, seed=1), 200000),
+    "deg4.5": lambda: _padded(gg.rmat(16, 16, seed=1), 400000),
+    "deg0.3": lambda: _padded(gg.rmat(14, 16, seed=1), 1400000),
+}
+
+
+@pytest.mark.parametrize("kernel", ["tr_random", "tr_maxw", "tr_p2", "tr_mincount"])
+@pytest.mark.parametrize("name", list(GRAPHS))
+def test_fits_where_one_pass_fits(sg, name, kernel):
+    g = gg.attach_weights(GRAPHS[name](), seed=1) if kernel == "tr_maxw" else GRAPHS[name]()
+    limit = _one_pass_peak(g.n, g.nnz, g.w is not None, kernel)
+    ctx = sg.Context(0)
+    G = sg.Graph.from_csr(ctx, g)
+    ctx.set_alloc_limit(limit)
+    H = sg.compress(G, kernel, 0.5, 3)
+    ctx.set_alloc_limit(limit // 4)
+    with pytest.raises(sg.SgError):
+        sg.compress(G, kernel, 0.5, 3)
+    ctx.set_alloc_limit(0)
+    off, col, w = H.download()
+    H.free()
+    G.free()
+    ctx.close()
+    o_off, o_col, _ = oracle.compress(g, kernel, 0.5, 3)
+    assert np.array_equal(off, o_off) and np.array_equal(col, o_col)

@@ -2123,6 +2123,7 @@ static sg_status launch_union(Ctx *c, const Oriented &o, TriArgs a, const Plan &
     bool two = h != nullptr && pl.max_deg > kShortList;
     if (two && alive_alloc(c, o, h, &al) != SG_OK) {
         set_error("");
+        alive_free(c, &al);  // what it got of it
         two = false;
     }
     a.short_max = !two ? INT_MAX : (pl.n_hubs > 0 ? kShortListHubs : kShortList);

@@ -67,3 +67,31 @@ def test_fits_where_one_pass_fits(sg, name, kernel):
     ctx.close()
     o_off, o_col, _ = oracle.compress(g, kernel, 0.5, 3)
     assert np.array_equal(off, o_off) and np.array_equal(col, o_col)
+
+
+def test_nothing_is_left_behind(sg):
+    """Limits at which one or another optional array does not fit: every call works, and
+    what it allocated before it gave up on a second pass is freed."""
+    g = GRAPHS["rmat16"]()
+    low = _one_pass_peak(g.n, g.nnz, False, "tr_random")
+    ctx = sg.Context(0)
+    G = sg.Graph.from_csr(ctx, g)
+    sizes = set()
+    for _ in range(2):  # the first time also loads the kernels, which takes memory
+        ctx.synchronize()
+        before = sg.device_free_memory(0)
+        for k in range(200):
+            ctx.set_alloc_limit(low - g.m + k * g.m // 100)  # a byte of flag per edge less, as they are bits
+            try:
+                H = sg.compress(G, "tr_random", 0.5, 3)
+            except sg.SgError:
+                assert k < 100  # below the one-pass peak
+                continue
+            sizes.add(H.nnz)
+            H.free()
+        ctx.set_alloc_limit(0)
+        ctx.synchronize()
+    assert len(sizes) == 1
+    assert sg.device_free_memory(0) >= before
+    G.free()
+    ctx.close()

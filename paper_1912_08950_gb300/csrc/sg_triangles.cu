@@ -2213,7 +2213,8 @@ static sg_status eo_run(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, 
     int top = kEoBuckets;          // the list holds every live triangle of the buckets below this one
     int sched = 0;                 // step of the prefix schedule: bids come from r2 below the top of bucket sched
     bool listed = false;
-    bool no_small = false;         // the small graph's list size did not fit
+    bool no_small = false;         // the small graph's list size did not fit, or left no room for the active lists
+    bool small_list = false;       // the list was allocated at that size
     bool try_list = o.m <= (int64_t)0xFFFFFFFFll && c->eo_list_cap >= 0;
     // warps of one enumeration launch, at most: each may leave a chunk per bucket part filled
     const int64_t emit_warps = (int64_t)c->num_sms * (8 * kTW + kHubTW);
@@ -2329,6 +2330,7 @@ static sg_status eo_run(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, 
                 if (hi <= rb) hi = 0;  // nothing to list: the pass only bids and counts
                 if (hi > 0) {
                     const size_t lbytes = (size_t)std::max<int64_t>(run, 1) * sizeof(uint4);
+                    small_list = small;
                     if (small) {
                         if (ws_get(c, kWsList, lbytes, (void **)&L) != SG_OK) {  // size it by the free memory then
                             set_error("");
@@ -2433,16 +2435,12 @@ static sg_status eo_run(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, 
             TriRec *B = nullptr;
             const int bslot = a_slot == kWsActive0 ? kWsActive1 : kWsActive0;
             const size_t bytes = (size_t)std::max<int64_t>(rest, 1) * sizeof(TriRec);
-            st = ws_get(c, bslot, bytes, (void **)&B);
+            bool room = ws_get(c, bslot, bytes, (void **)&B) == SG_OK;
             // (the buffer that holds the survivors has room for them; the first
             // round reads it, later ones write at most what the round before kept)
-            if (st == SG_OK && (lenA == 0 || c->ws_bytes[a_slot] < bytes)) {
-                TriRec *A2 = nullptr;
-                if (lenA == 0) st = ws_get(c, a_slot, bytes, (void **)&A2);
-                if (lenA == 0) A = A2;
-            }
-            if (st != SG_OK) break;
-            if (c->ws_bytes[a_slot] >= bytes) {
+            if (room && lenA == 0) room = ws_get(c, a_slot, bytes, (void **)&A) == SG_OK;
+            if (!room) set_error("");  // a round's own launches need less
+            if (room && c->ws_bytes[a_slot] >= bytes) {
                 SG_CUDA(cudaMemsetAsync(lctr, 0, lctr_bytes, c->stream));
                 EoRun r{};
                 r.fresh = L;
@@ -2489,6 +2487,23 @@ static sg_status eo_run(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, 
         TriRec *B = nullptr;
         const int bslot = a_slot == kWsActive0 ? kWsActive1 : kWsActive0;
         st = ws_get(c, bslot, (size_t)std::max<int64_t>(lenA + fresh, 1) * sizeof(TriRec), (void **)&B);
+        if (st == SG_ERR_OOM && small_list) {
+            // the list was sized without asking for the free memory: give it back and
+            // list what is live again, within a quarter of what there is
+            set_error("");
+            st = SG_OK;
+            dfree(c, c->ws[kWsList]);
+            c->ws[kWsList] = nullptr;
+            c->ws_bytes[kWsList] = 0;
+            L = nullptr;
+            lenA = 0;
+            listed = small_list = false;
+            no_small = true;
+            top = next_bucket = kEoBuckets;
+            --round;
+            --sched;
+            continue;
+        }
         if (st != SG_OK) break;
         unsigned long long *out_len = lctr + 2 * kEoBuckets;
         SG_CUDA(cudaMemsetAsync(out_len, 0, sizeof(unsigned long long), c->stream));

@@ -95,3 +95,26 @@ def test_nothing_is_left_behind(sg):
     assert sg.device_free_memory(0) >= before
     G.free()
     ctx.close()
+
+
+# limits around the 256 MB (and a quarter of headroom) of a small graph's triangle list: below it, just above it
+# with little left for the rounds' own lists, and with room for everything
+@pytest.mark.parametrize("kernel", ["tr_eo", "tr_eo_maxw", "tr_eo_mincount"])
+@pytest.mark.parametrize("one_launch", [True, False])
+def test_edge_once_list_leaves_room(sg, kernel, one_launch):
+    g = gg.attach_weights(gg.rmat(12, 16, seed=12), seed=1)
+    o_off, o_col, _ = oracle.compress(g, kernel, 1.0, 3)
+    ctx = sg.Context(0)
+    ctx.set_eo_one_launch(one_launch)
+    G = sg.Graph.from_csr(ctx, g)
+    for mb in (60, 120, 261, 262, 263, 264, 266, 268, 270, 275, 280, 290, 300, 320, 325, 330, 340, 400):
+        ctx.release_workspace()
+        ctx.set_alloc_limit(mb << 20)
+        H = sg.compress(G, kernel, 1.0, 3)
+        ctx.release_workspace()
+        ctx.set_alloc_limit(0)
+        off, col, _ = H.download()
+        H.free()
+        assert np.array_equal(off, o_off) and np.array_equal(col, o_col), mb
+    G.free()
+    ctx.close()

@@ -654,7 +654,11 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     a.vblocks = vblocks;
     a.x_out = x_out;
     // one allocation: the arrays below, each aligned to 256 bytes
-    const size_t max_hubs = (size_t)(nnz / kHubRow + 1), max_chunks = (size_t)(nnz / kHubChunk) + max_hubs;
+    // (rows of each length class: by their arcs, and no more than there are rows)
+    const size_t max_hubs = std::min(nn, (size_t)(nnz / kHubRow + 1));
+    const size_t max_chunks = (size_t)(nnz / kHubChunk) + max_hubs;
+    // parts: the chunks' runs while there are few chunks, the chunks otherwise
+    const size_t max_parts = std::max(max_chunks, std::min(max_chunks, (size_t)c->num_sms * (kPrCta / 32) / 4) * kPrWarps);
     const int hot_cap = (int)std::min<int64_t>(kPrHot, n);
     size_t total = 0;
     auto room = [&](size_t bytes) {
@@ -672,8 +676,8 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     const size_t cnt_at = room(sizeof(uint32_t) * (size_t)vblocks * kPrThreads);
     const size_t w_at[2] = {room(sizeof(float) * (size_t)vblocks * kPrWarps), room(sizeof(float) * (size_t)vblocks * kPrWarps)};
     const size_t hubs_at = room(sizeof(uint32_t) * max_hubs), first_at = room(sizeof(int) * max_hubs);
-    const size_t med_at = room(sizeof(uint32_t) * (size_t)(nnz / kShortRow + 1));
-    const size_t chunk_at = room(sizeof(uint32_t) * max_chunks), part_at = room(sizeof(float) * max_chunks * kPrWarps);
+    const size_t med_at = room(sizeof(uint32_t) * std::min(nn, (size_t)(nnz / kShortRow + 1)));
+    const size_t chunk_at = room(sizeof(uint32_t) * max_chunks), part_at = room(sizeof(float) * max_parts);
     char *buf = nullptr;
     uint32_t *pos = nullptr, *colx = nullptr;
     sg_status st = dalloc(c, (void **)&buf, total);

@@ -385,7 +385,7 @@ void sg_batch_free(sg_batch *b) {
                         (void *)b->rm.chunk_row, (void *)b->o.off, (void *)b->o.col, (void *)b->o.w,
                         (void *)b->o.fwd_bits, (void *)b->o.fwd_excl, (void *)b->scan, (void *)b->final_cs.keep,
                         (void *)b->final_cs.cexcl, (void *)b->final_cs.scan, (void *)b->del,
-                        (void *)b->bt.heavy, (void *)b->bt.buckets, (void *)b->bt.din, (void *)b->bt.vrec,
+                        (void *)b->bt.heavy, (void *)b->bt.buckets, (void *)b->bt.din,
                         (void *)b->bt.inl, (void *)b->off_c,
                         (void *)b->out_off, (void *)b->out_col, (void *)b->out_w, (void *)b->d_info})
             if (p) (void)cudaFree(p);

@@ -287,7 +287,6 @@ struct BatchTri {
     uint32_t *heavy = nullptr;
     unsigned long long *buckets = nullptr;  // counts, fills, total
     uint32_t *din = nullptr;                // in-arcs streamed from the head's side
-    uint2 *vrec = nullptr;                  // off+ and d+ of every vertex
     uint2 *inl = nullptr;
     size_t smem = 0;
     int max_deg = 1;      // largest out-degree (sizes the heavy vertex arrays)

@@ -68,10 +68,12 @@ constexpr int kEoBuckets = 6;     // edge-once list buckets (rounds 0..5 of the 
 // context workspaces of the edge-once rounds: the list and the two active lists
 constexpr int kWsList = 0, kWsActive0 = 1, kWsActive1 = 2;
 
-// Count: totals only (tri_enum_kernel; Union* and BatchUnion run in tri_union_kernel).  EdgeCount / VertexCount: add every triangle to the
-// counters of its three edges / vertices.  Union*: the union-semantics TR kernels.  EoReserve: one
-// edge-once bidding pass.  EoEmit: lists the live selected triangles for the
-// edge-once list rounds.  BatchUnion: union kernels over a batch of graphs.
+// Count: totals only.  EdgeCount / VertexCount: add every triangle to the
+// counters of its three edges / vertices.  Union*: the union-semantics TR
+// kernels (in one pass, or in the two of tri_union_kernel: two_passes_pay).
+// EoReserve: one edge-once bidding pass.  EoEmit: lists the live selected
+// triangles for the edge-once list rounds.  BatchUnion: union kernels over a
+// batch of graphs.
 enum class Mode { Count, EdgeCount, VertexCount, UnionRandom, UnionMaxw, UnionP2, UnionMinCount, EoReserve, EoEmit,
                   BatchUnion };
 template <Mode M>
@@ -80,6 +82,9 @@ constexpr bool kUnion = M == Mode::UnionRandom || M == Mode::UnionMaxw || M == M
 // the edge-once passes skip arcs that are already considered
 template <Mode M>
 constexpr bool kEdgeOnce = M == Mode::EoReserve || M == Mode::EoEmit;
+// the passes that decide their triangles (the others only count them)
+template <Mode M>
+constexpr bool kDecides = kUnion<M> || kEdgeOnce<M>;
 
 // Edge-once "considered" flags: one bit per oriented arc (m/8 bytes, so the
 // flags stay in L2 while the triangle lists stream past them).
@@ -97,6 +102,13 @@ __device__ __forceinline__ bool arc_deleted(const uint32_t *del, uint32_t e) {
     return (w >> (e & 31)) & 1u;
 }
 
+// The same through the L1, where a line may have been there since before.
+__device__ __forceinline__ bool arc_deleted_cached(const uint32_t *del, uint32_t e) {
+    uint32_t w;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(w) : "l"(del + (e >> 5)));
+    return (w >> (e & 31)) & 1u;
+}
+
 struct TriArgs {
     const int64_t *offp;
     const uint32_t *colp;
@@ -108,7 +120,8 @@ struct TriArgs {
     uint32_t k0, k1;
     unsigned long long tp;
     uint32_t *del;                // deletion flags, one bit per oriented arc
-    uint32_t dead_flag;           // union passes: a bit no arc index uses (kArcDead), or 0
+    bool look_first;              // one union pass: look at an arc's flag before setting it
+    uint32_t dead_flag;           // two union passes: a bit no arc index uses (kArcDead), or 0
     const uint32_t *considered;  // edge-once flag bits (see considered_bit)
     unsigned long long *resv;
     uint32_t *tcnt;               // triangles of G through each arc of E+ (EdgeCount adds, min-count reads)
@@ -120,10 +133,8 @@ struct TriArgs {
     int heavy_cap;               // entries of the phase-1 table; larger N+(u) go in chunks
     int light_max;               // out-degrees up to this go to the warp-per-vertex phase
     int light_claim;             // vertices a warp claims at a time in the light phase (at most 32)
-    int short_max;               // union passes: lists up to this long are always streamed whole
-    const uint2 *vrec;           // off+ and d+ of vertex v at entry v * vstep
-    int vstep;                   // 1, or 2: the first halves of the records arec
-    const uint4 *arec;           // off+, d+, first live arc, live arcs (second union pass: alive_build)
+    int short_max;               // two union passes: lists up to this long are always streamed whole
+    const uint4 *arec;           // two union passes: off+, d+, and for the second first live arc, live arcs
     const uint2 *alive;
     int light_items;             // ... when they also have at most this many arcs to stream
     int *err;                    // device error word (a cuckoo stash overflow)
@@ -271,26 +282,71 @@ __device__ __forceinline__ void sort_triangle(uint32_t &x0, uint32_t &x1, uint32
 }
 
 // the heaviest of a sorted triangle's edges under (weight, lo, hi)
-__device__ __forceinline__ uint32_t maxw_arc(const float *wp, uint32_t x0, uint32_t x1, uint32_t x2, uint32_t e01,
-                                             uint32_t e02, uint32_t e12) {
+__device__ __forceinline__ uint32_t maxw_arc(const float *wp, uint32_t e01, uint32_t e02, uint32_t e12) {
     const float w01 = __ldg(wp + e01), w02 = __ldg(wp + e02), w12 = __ldg(wp + e12);
+    // (x0, x1) < (x0, x2) < (x1, x2): of equal weights the later edge
     uint32_t best = e01;
     float bw = w01;
-    uint32_t bl = x0, bh = x1;
-    if (w02 > bw || (w02 == bw && (x0 > bl || (x0 == bl && x2 > bh)))) { best = e02; bw = w02; bl = x0; bh = x2; }
-    if (w12 > bw || (w12 == bw && (x1 > bl || (x1 == bl && x2 > bh)))) { best = e12; }
+    if (w02 >= bw) { best = e02; bw = w02; }
+    if (w12 >= bw) best = e12;
     return best;
 }
 
-// One triangle (u, v, w) with its three oriented arcs under an edge-once pass:
+// One triangle (u, v, w) with its three oriented arcs under a union kernel:
+// selection, and kill(arc) for what it deletes.
+template <Mode M, class Kill>
+__device__ __forceinline__ void decide_union(const TriArgs &a, uint32_t u, uint32_t v, uint32_t w, uint32_t iuv,
+                                             uint32_t iuw, uint32_t ivw, const Kill &kill) {
+    uint32_t x0 = u, x1 = v, x2 = w, e01 = iuv, e02 = iuw, e12 = ivw;
+    uint32_t k0 = a.k0, k1 = a.k1;
+    unsigned long long tp = a.tp;
+    bool maxw = M == Mode::UnionMaxw, p2 = M == Mode::UnionP2;
+    if constexpr (M == Mode::BatchUnion) {
+        // the triangle's graph: its own seed, p and kernel, local ids as keys
+        const BatchParam &P = a.bparams[__ldg(a.vgid + u)];
+        const uint32_t base = (uint32_t)P.vbase;
+        x0 -= base;
+        x1 -= base;
+        x2 -= base;
+        k0 = P.k0;
+        k1 = P.k1;
+        tp = P.tp;
+        maxw = P.kernel == (int)SG_TR_MAXW;
+        p2 = P.kernel == (int)SG_TR_P2;
+    }
+    sort_triangle(x0, x1, x2, e01, e02, e12);
+    const uint4 r = philox4x32_10(make_uint4(x0, x1, x2, kTagTri), k0, k1);
+    if ((unsigned long long)r.x >= tp) return;  // not selected
+    uint32_t best;
+    if constexpr (M == Mode::UnionMinCount) {
+        best = mincount_arc(a.tcnt, e01, e02, e12);
+    } else if (maxw) {
+        best = maxw_arc(a.wp, e01, e02, e12);
+    } else {
+        const int k = (int)(((unsigned long long)r.y * 3ull) >> 32);
+        if (p2) {  // x = 2: the drawn edge stays, the other two go
+            if (k != 0) kill(e01);
+            if (k != 1) kill(e02);
+            if (k != 2) kill(e12);
+            return;
+        }
+        best = k == 0 ? e01 : (k == 1 ? e02 : e12);
+    }
+    kill(best);
+}
+
+// One triangle under a one-pass union or an edge-once pass: deletion, or
 // selection and bid or listing.  Warp-collective (the list writer uses
 // ballots); lanes without a triangle pass valid = false.
 template <Mode M>
 __device__ __forceinline__ void decide(const TriArgs &a, bool valid, uint32_t u, uint32_t v, uint32_t w,
                                        uint32_t iuv, uint32_t iuw, uint32_t ivw, unsigned &live, Emitter &em,
                                        uint32_t head_uv = 0) {
-    if constexpr (!kEdgeOnce<M>) {
-        return;
+    if constexpr (kUnion<M>) {
+        if (valid)
+            decide_union<M>(a, u, v, w, iuv, iuw, ivw, [&](uint32_t e) {
+                if (!a.look_first || !arc_deleted_cached(a.del, e)) delete_arc(a.del, e);
+            });
     } else {
         bool emit = false;
         uint4 rec = make_uint4(0u, 0u, 0u, 0u);
@@ -342,7 +398,7 @@ __device__ __forceinline__ void drain32(const TriArgs &a, const HitQueue &q, int
 template <Mode M>
 __device__ __forceinline__ void flush_hits(const TriArgs &a, const HitQueue &q, QState &qs, uint32_t u,
                                            unsigned &live, Emitter &em) {
-    if constexpr (kEdgeOnce<M>) {
+    if constexpr (kDecides<M>) {
         const int lane = threadIdx.x & 31;
         while (qs.n >= 32) {
             drain32<M>(a, q, qs.head, u, live, em);
@@ -587,7 +643,7 @@ __device__ __forceinline__ void stream_in_group(const TriArgs &a, const Table &t
 // 64 elements), so they are streamed as one sequence, a slab of 32 elements at a
 // time: a lane finds its element's arc from the arcs that start inside the
 // slab.  Counting: the first lane of an arc's run adds the run's hits to the
-// arc's counters; edge-once: the hits go to the queue.  A list at a time, 64 lanes wide, left most lanes idle and waited for
+// arc's counters; otherwise the hits go to the queue.  A list at a time, 64 lanes wide, left most lanes idle and waited for
 // one list's loads after another: triangles per vertex of a geometric graph
 // (2^20 vertices, 25 M edges, lists of 17 elements) took 5.18 ms, now 2.15; of
 // R-MAT s20, where most elements are in heavy vertices' lists, 9.33 and 8.98.
@@ -663,7 +719,7 @@ __device__ __forceinline__ unsigned light_group(const TriArgs &a, const Table &t
         if (m == 0) continue;
         hits += (unsigned)__popc(m);
         if constexpr (M == Mode::Count) continue;
-        if constexpr (kEdgeOnce<M>) {
+        if constexpr (kDecides<M>) {
             if (h) {
                 const int s0 = (qs.head + qs.n + __popc(m & lt)) & (kQ - 1);
                 const uint4 c = arc[k];
@@ -730,7 +786,7 @@ __device__ __forceinline__ void finish(const TriArgs &a, unsigned live, unsigned
 // CTA of 32 warps per SM shares a table of up to kHubCap entries, so those
 // lists are streamed once instead of once per table chunk.
 template <Mode M>
-constexpr int kEnumCtasPerSm = kEdgeOnce<M> ? 4 : 5;
+constexpr int kEnumCtasPerSm = kDecides<M> ? 4 : 5;
 
 template <Mode M, int TW>
 __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tri_enum_kernel(TriArgs a) {
@@ -930,56 +986,6 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tr
 // triangle) and now: s22 0.35 and 0.14, 41.8 -> 19.2 ms; s26 0.32 and 0.09,
 // 1094 -> 528 ms.  Max-weight on a Chung-Lu graph of 2^21 vertices at p = 1,
 // where light edges never die: 0.69 and 0.35, 11.5 -> 8.3 ms.
-template <Mode M>
-__device__ __forceinline__ void kill_arc(const TriArgs &a, const Table &tb, uint32_t tbase, uint32_t cn, uint32_t e) {
-    delete_arc(a.del, e);
-    const uint32_t r = e - tbase;  // an arc of the table: its flag in shared memory too
-    if (r < cn) atomicOr(tb.dead + (r >> 5), 1u << (r & 31));
-}
-
-// One triangle (u, v, w) with its three oriented arcs: selection and deletion.
-template <Mode M>
-__device__ __forceinline__ void decide_union(const TriArgs &a, const Table &tb, uint32_t tbase, uint32_t cn,
-                                             uint32_t u, uint32_t v, uint32_t w, uint32_t iuv, uint32_t iuw,
-                                             uint32_t ivw) {
-    uint32_t x0 = u, x1 = v, x2 = w, e01 = iuv, e02 = iuw, e12 = ivw;
-    uint32_t k0 = a.k0, k1 = a.k1;
-    unsigned long long tp = a.tp;
-    bool maxw = M == Mode::UnionMaxw, p2 = M == Mode::UnionP2;
-    if constexpr (M == Mode::BatchUnion) {
-        // the triangle's graph: its own seed, p and kernel, local ids as keys
-        const BatchParam &P = a.bparams[__ldg(a.vgid + u)];
-        const uint32_t base = (uint32_t)P.vbase;
-        x0 -= base;
-        x1 -= base;
-        x2 -= base;
-        k0 = P.k0;
-        k1 = P.k1;
-        tp = P.tp;
-        maxw = P.kernel == (int)SG_TR_MAXW;
-        p2 = P.kernel == (int)SG_TR_P2;
-    }
-    sort_triangle(x0, x1, x2, e01, e02, e12);
-    const uint4 r = philox4x32_10(make_uint4(x0, x1, x2, kTagTri), k0, k1);
-    if ((unsigned long long)r.x >= tp) return;  // not selected
-    uint32_t best;
-    if constexpr (M == Mode::UnionMinCount) {
-        best = mincount_arc(a.tcnt, e01, e02, e12);
-    } else if (maxw) {
-        best = maxw_arc(a.wp, x0, x1, x2, e01, e02, e12);
-    } else {
-        const int k = (int)(((unsigned long long)r.y * 3ull) >> 32);
-        if (p2) {  // x = 2: the drawn edge stays, the other two go
-            if (k != 0) kill_arc<M>(a, tb, tbase, cn, e01);
-            if (k != 1) kill_arc<M>(a, tb, tbase, cn, e02);
-            if (k != 2) kill_arc<M>(a, tb, tbase, cn, e12);
-            return;
-        }
-        best = k == 0 ? e01 : (k == 1 ? e02 : e12);
-    }
-    kill_arc<M>(a, tb, tbase, cn, best);
-}
-
 // The table vertex a warp works on.
 struct TabCtx {
     Table tb;
@@ -1038,7 +1044,12 @@ __device__ __forceinline__ void drain_union(const TriArgs &a, const TabCtx &t, c
         // matters while one of its other edges lives
         const uint32_t vw = h.w & ~a.dead_flag;
         if (hit && (h.w & a.dead_flag) && ((t.tb.dead[k >> 5] >> (k & 31)) & 1u)) hit = !arc_deleted(a.del, vw);
-        if (hit) decide_union<M>(a, t.tb, t.tbase, t.cn, t.u, h.x, h.z, h.y, t.tbase + k, vw);
+        if (hit)
+            decide_union<M>(a, t.u, h.x, h.z, h.y, t.tbase + k, vw, [&](uint32_t e) {
+                delete_arc(a.del, e);
+                const uint32_t r = e - t.tbase;  // an arc of the table: its flag in shared memory too
+                if (r < t.cn) atomicOr(t.tb.dead + (r >> 5), 1u << (r & 31));
+            });
     }
     const unsigned m = __ballot_sync(kFull, hit);
     if (lane == 0) tris += (unsigned)__popc(m);
@@ -1160,7 +1171,7 @@ __device__ __forceinline__ void stream_lists(const TriArgs &a, const TabCtx &t, 
 // about 40 elements on R-MAT graphs) and its lane takes the next arc.  The
 // records of one claim load while the windows stream, the ids of the next with
 // them.
-template <Mode M, bool kAlive, bool kRec>
+template <Mode M, bool kAlive>
 __device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, int *next, uint32_t ou, int64_t ib, int nin,
                                             int ax, UnionScratch &q, QState &qs, unsigned long long &probes,
                                             unsigned long long &tris, bool count) {
@@ -1200,13 +1211,10 @@ __device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, i
             dead = arc_deleted(a.del, ge);
             if constexpr (kAlive) {
                 rec = __ldg(a.arec + gv);
-            } else if constexpr (kRec) {
-                const uint2 r = __ldg(a.vrec + (size_t)gv * a.vstep);
+            } else {
+                const uint2 r = __ldg(reinterpret_cast<const uint2 *>(a.arec + gv));
                 rec.x = r.x;
                 rec.y = r.y;
-            } else {
-                rec.x = (uint32_t)__ldg(a.offp + gv);
-                rec.y = (uint32_t)__ldg(a.offp + gv + 1) - rec.x;
             }
         }
         if (gc < items) {
@@ -1290,10 +1298,7 @@ __device__ __forceinline__ void stream_arcs(const TriArgs &a, const TabCtx &t, i
 // three CTAs with more registers: s22 3.14 -> 2.84 ms, s26 51.6 -> 46.4,
 // max-weight on the Chung-Lu graph 1.54 -> 1.38; the first pass is slower at
 // three (s22 16.4 -> 17.0, s26 248 -> 276) and at five (17.0, 253).
-// kRec: vertex records to read; without them (no memory left for them) the
-// offsets are read instead, in an instance of its own, since choosing at run time
-// spills in the first pass (s22 23.6 -> 24.4 ms a call, s26 627 -> 651).
-template <Mode M, int TW, bool kAlive, bool kRec = true>
+template <Mode M, int TW, bool kAlive>
 __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri_union_kernel(TriArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_next;
@@ -1308,7 +1313,6 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri
     UnionScratch &q = reinterpret_cast<UnionScratch *>(smem)[warp];
     QState qst;
     unsigned long long probes = 0, tris = 0;
-    const int64_t n_heavy = a.n_heavy_dev ? (int64_t)*a.n_heavy_dev : a.n_heavy;
     if constexpr (kAlive) {  // live lists of a scan that gave up are not followed
         if (threadIdx.x == 0) s_bad = *(volatile int *)a.err;
         __syncthreads();
@@ -1326,7 +1330,7 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri
             if (threadIdx.x == 0) s_h = (long long)atomicAdd(a.work, 1ull);
             __syncthreads();
             const int64_t h = s_h;
-            if (h >= n_heavy) break;
+            if (h >= a.n_heavy) break;
             t.u = __ldg(a.heavy + h);
             const int64_t ou = __ldg(a.offp + t.u);
             t.d = (int)(__ldg(a.offp + t.u + 1) - ou);
@@ -1368,7 +1372,7 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri
                 }
                 __syncthreads();
                 t.stash_n = min(*t.tb.stash_n, kStash);
-                stream_arcs<M, kAlive, kRec>(a, t, &s_next, (uint32_t)ou, ib, nin, ax, q, qst, probes, tris, c0 == 0);
+                stream_arcs<M, kAlive>(a, t, &s_next, (uint32_t)ou, ib, nin, ax, q, qst, probes, tris, c0 == 0);
                 flush_union<M>(a, t, q, qst, tris);
                 __syncthreads();  // the table is rebuilt for the next chunk or vertex
             }
@@ -1429,9 +1433,8 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? (kAlive ? 3 : 4) : 1) tri
                 }
                 __syncwarp();
                 t.stash_n = min(*t.tb.stash_n, kStash);
-                stream_arcs<M, false, kRec>(a, t, &s_lnext[warp], t.tbase,
-                                            nin > 0 ? __ldg(a.offs + t.u) - (int64_t)t.tbase : 0, nin, 0, q, qst,
-                                            probes, tris, true);
+                stream_arcs<M, false>(a, t, &s_lnext[warp], t.tbase, nin > 0 ? __ldg(a.offs + t.u) - (int64_t)t.tbase : 0,
+                                      nin, 0, q, qst, probes, tris, true);
                 flush_union<M>(a, t, q, qst, tris);
                 __syncwarp();
             }
@@ -1467,13 +1470,15 @@ __device__ __forceinline__ int heavy_key(int64_t d, int64_t nin, int64_t hub_min
 }
 
 // Also writes every vertex's in-degree d(u) - d+(u): the length of its
-// in-list in the reverse list (see Oriented::inl), and its off+ and d+ as one
-// 8-byte record.
+// in-list in the reverse list (see Oriented::inl).  With bucket_cnt2, also
+// counts the split of the two union passes (kUnionLightMax).
 __global__ void classify_count_kernel(const int64_t *__restrict__ offp, const int64_t *__restrict__ offs,
-                                      uint32_t *din, uint2 *vrec, int vstep, int64_t n, int light_max, int light_items,
-                                      int64_t hub_min, unsigned long long *bucket_cnt, unsigned long long *ctr) {
-    __shared__ unsigned int s_cnt[kKeys];
-    if (threadIdx.x < kKeys) s_cnt[threadIdx.x] = 0;
+                                      uint32_t *din, int64_t n, int light_max, int light_items, int64_t hub_min,
+                                      unsigned long long *bucket_cnt, unsigned long long *bucket_cnt2,
+                                      unsigned long long *ctr) {
+    __shared__ unsigned int s_cnt[kKeys], s_cnt2[kKeys];
+    static_assert(kKeys <= 256, "a thread per key");
+    if (threadIdx.x < kKeys) s_cnt[threadIdx.x] = s_cnt2[threadIdx.x] = 0;
     __syncthreads();
     unsigned long long dmax = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1483,8 +1488,9 @@ __global__ void classify_count_kernel(const int64_t *__restrict__ offp, const in
         int64_t nin = (offs[u + 1] - offs[u]) - d;
         nin = nin < 0 ? 0 : nin;
         din[u] = (uint32_t)nin;
-        if (vrec) vrec[u * vstep] = make_uint2((uint32_t)offp[u], (uint32_t)d);
         if (is_heavy(d, nin, light_max, light_items)) atomicAdd(&s_cnt[heavy_key(d, nin, hub_min)], 1u);
+        if (bucket_cnt2 && is_heavy(d, nin, kUnionLightMax, kUnionLightItems))
+            atomicAdd(&s_cnt2[heavy_key(d, nin, hub_min)], 1u);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -1494,12 +1500,16 @@ __global__ void classify_count_kernel(const int64_t *__restrict__ offp, const in
     if ((threadIdx.x & 31) == 0) atomicMax(ctr + kCtrMaxDeg, dmax);
     __syncthreads();
     if (threadIdx.x < kKeys && s_cnt[threadIdx.x]) atomicAdd(bucket_cnt + threadIdx.x, (unsigned long long)s_cnt[threadIdx.x]);
+    if (threadIdx.x < kKeys && s_cnt2[threadIdx.x])
+        atomicAdd(bucket_cnt2 + threadIdx.x, (unsigned long long)s_cnt2[threadIdx.x]);
 }
+
+// Also writes the vertex records of two union passes (off+, d+, no live arcs yet), if asked to.
 
 __global__ void classify_scatter_kernel(const int64_t *__restrict__ offp, const uint32_t *__restrict__ din,
                                         int64_t n, int light_max, int light_items, int64_t hub_min,
                                         const unsigned long long *__restrict__ bucket_cnt,
-                                        unsigned long long *bucket_fill, uint32_t *heavy,
+                                        unsigned long long *bucket_fill, uint32_t *heavy, uint4 *arec,
                                         unsigned long long *total_out) {
     __shared__ unsigned long long s_off[kKeys];
     if (threadIdx.x == 0) {
@@ -1515,6 +1525,7 @@ __global__ void classify_scatter_kernel(const int64_t *__restrict__ offp, const 
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < n; u += stride) {
         const int64_t d = offp[u + 1] - offp[u];
         const int64_t nin = din[u];
+        if (arec) arec[u] = make_uint4((uint32_t)offp[u], (uint32_t)d, 0u, 0u);
         if (is_heavy(d, nin, light_max, light_items)) {
             const int b = heavy_key(d, nin, hub_min);
             heavy[s_off[b] + atomicAdd(bucket_fill + b, 1ull)] = (uint32_t)u;
@@ -1568,7 +1579,7 @@ __global__ void eo_accept_kernel(TriArgs a, const int64_t *__restrict__ off, uin
             if constexpr (CH == kChoiceMinCount) {
                 chosen = mincount_arc(a.tcnt, e01, e02, e12);
             } else if constexpr (CH == kChoiceMaxw) {
-                chosen = maxw_arc(a.wp, x0, x1, x2, (uint32_t)e01, (uint32_t)e02, (uint32_t)e12);
+                chosen = maxw_arc(a.wp, (uint32_t)e01, (uint32_t)e02, (uint32_t)e12);
             } else {
                 const uint4 rr = philox4x32_10(make_uint4(x0, x1, x2, kTagTri), a.k0, a.k1);
                 const int k = (int)(((unsigned long long)rr.y * 3ull) >> 32);
@@ -1585,7 +1596,7 @@ __device__ __forceinline__ uint32_t chosen_arc(const TriRec &r, const float *wp,
     if constexpr (CH == kChoiceMinCount) {
         return mincount_arc(tcnt, r.e01, r.e02, r.e12);
     } else if constexpr (CH == kChoiceMaxw) {
-        return maxw_arc(wp, r.x0, r.x1, r.x2, r.e01, r.e02, r.e12);
+        return maxw_arc(wp, r.e01, r.e02, r.e12);
     } else {
         const int k = (int)(((unsigned long long)r.r1 * 3ull) >> 32);
         return k == 0 ? r.e01 : (k == 1 ? r.e02 : r.e12);
@@ -1906,11 +1917,12 @@ __global__ void __cluster_dims__(kEoCluster, 1, 1) __launch_bounds__(kEoCta, 1) 
 // -------------------------------------------------------------------- host
 struct Plan {
     uint32_t *heavy = nullptr;
-    unsigned long long *buckets = nullptr;  // counts [kKeys], fills [kKeys]
+    unsigned long long *buckets = nullptr;  // counts [kKeys], those of the two passes' split [kKeys], fills [kKeys]
     uint32_t *din = nullptr;                // in-arcs streamed from the head's side, per vertex
-    bool records = false;                   // union passes: 16-byte vertex records wanted
-    uint4 *arec = nullptr;                  // the records, if there is room for them; off+ and d+ first
-    void *rec_own = nullptr;                // their allocation, if they have one
+    bool two = false;                       // two union passes
+    uint4 *arec = nullptr;                  // ... their vertex records,
+    void *rec_own = nullptr;                // the records' allocation, if they have one,
+    AliveArcs al;                           // and the live arcs between them
     uint2 *inl = nullptr;                   // their (tail, arc), at offs(v) - offp(v) per vertex
     const int64_t *offs = nullptr;          // symmetric offsets of the graph
     int64_t n_heavy = 0, max_deg = 0;
@@ -1938,6 +1950,7 @@ static void free_plan(Ctx *c, Plan *pl) {
     dfree(c, pl->buckets);
     dfree(c, pl->din);
     dfree(c, pl->rec_own);
+    alive_free(c, &pl->al);
     pl->rec_own = nullptr;
     pl->arec = nullptr;
     pl->heavy = nullptr;
@@ -1952,57 +1965,105 @@ static size_t union_table_bytes(int cap) {
     return (size_t)cap * 4 * sizeof(uint32_t) + (size_t)(cap + 31) / 32 * 4 + (size_t)cap * kFilterBits / 8;
 }
 
-// inl_cap: room for in-arc records; nnz - m when E+ holds all m arcs, nnz
-// when it may hold fewer (batches orient only their triangle-kernel graphs).
-static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan *pl) {
+// A union call that may take two passes: its kernel, and the output graph, whose arrays they borrow.
+struct UnionCall {
+    sg_kernel kernel;
+    unsigned long long tp;
+    const Graph *h;
+};
+
+// Whether two union passes (tri_union_kernel) pay.  They drop what is streamed and
+// decided for deleted edges, at the price of a pass over the vertices and arcs
+// between them and of more instructions per element (the filter, the windows).
+// So the lists have to be long, as those of up to kShortList are streamed whole
+// whatever happens: W / m elements per arc on average, and a longest one of twice
+// that; W has to outweigh the pass over the vertices; and deletions have to come
+// while the lists stream: p W / m bounds the selected triangles per edge
+// (about a sixth of the elements close one on R-MAT graphs, all of them in
+// cliques, which the rule cannot tell).  Where a triangle deletes two edges
+// (p-2) half of that does; where it always deletes its heaviest, light edges
+// live on and it takes more.  Calls in ms, one pass / two passes:
+//   random        p W / m  1.2: R-MAT s20  8.49 / 10.3   3.8: R-MAT s20  8.57 / 9.10
+//                          5.5: R-MAT s22  45.1 / 45.5   6.0: Chung-Lu 2^21 11.4 / 9.99
+//                           12: R-MAT s20  8.67 / 7.10
+//   max-weight              12: R-MAT s20  9.38 / 9.84    18: Chung-Lu 2^21 12.2 / 11.1
+//                           37: R-MAT s20  9.49 / 8.43
+//   random p = 0.5  W / m  46: n = 200,000, ef 8  0.64 / 1.07   47: n = 2^20, ef 5  1.84 / 1.98
+//                          60: Chung-Lu 2^21      11.4 / 8.69   83: n = 30,000, ef 40  0.65 / 0.57
+//                          66, longest 199: cliques of 200  18.1 / 21.6
+static bool two_passes_pay(const Oriented &o, int64_t max_deg, int64_t work, const UnionCall &u) {
+    const double w = (double)work, m = (double)o.m;
+    if (o.m == 0 || max_deg <= 2 * kShortList || w < 0.4 * kShortList * m || w < 32.0 * (double)o.n) return false;
+    const double selected = (double)u.tp / 4294967296.0 * w / m;
+    return selected >= (u.kernel == SG_TR_P2 ? 2.5 : u.kernel == SG_TR_MAXW ? 15.0 : 5.0);
+}
+
+// What two passes need beside the plan; false (and nothing kept) where it does not fit.
+static bool two_passes_fit(Ctx *c, const Oriented &o, const UnionCall &u, Plan *pl) {
+    // the records in the unused half of E+'s column array (room for nnz = 2m
+    // entries) if it holds them (16 n <= 4 m: a mean degree of 8), in memory of
+    // their own otherwise
+    const uintptr_t b = ((uintptr_t)(o.col + o.m) + 15) & ~(uintptr_t)15, e = (uintptr_t)(o.col + 2 * o.m);
+    sg_status st = SG_OK;
+    if (b + sizeof(uint4) * (size_t)o.n <= e)
+        pl->arec = reinterpret_cast<uint4 *>(b);
+    else if ((st = dalloc(c, &pl->rec_own, sizeof(uint4) * (size_t)o.n)) == SG_OK)
+        pl->arec = static_cast<uint4 *>(pl->rec_own);
+    if (st == SG_OK) st = alive_alloc(c, o, u.h, &pl->al);
+    if (st == SG_OK) return true;
+    set_error("");
+    alive_free(c, &pl->al);  // what it got of it
+    dfree(c, pl->rec_own);
+    pl->rec_own = nullptr;
+    pl->arec = nullptr;
+    return false;
+}
+
+// How the vertices are split between warps, CTAs and the hub launch.  u: a union
+// call that may take two passes, which split them their own way.
+static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan *pl, const UnionCall *u = nullptr) {
     if (o.m >= (int64_t)0xFFFFFFFFll)
         return fail(SG_ERR_UNSUPPORTED, "triangle kernels address oriented arcs with 32 bits: m must be < 2^32");
     if (o.n >= (int64_t)0xFFFFFFFEll)
         return fail(SG_ERR_UNSUPPORTED, "triangle kernels reserve vertex ids 2^32 - 2 and 2^32 - 1");
     pl->offs = offs;
     sg_status st = dalloc(c, (void **)&pl->heavy, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
-    if (st == SG_OK) st = dalloc(c, (void **)&pl->buckets, sizeof(unsigned long long) * 2 * kKeys);
+    if (st == SG_OK) st = dalloc(c, (void **)&pl->buckets, sizeof(unsigned long long) * 3 * kKeys);
     if (st == SG_OK) st = dalloc(c, (void **)&pl->din, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
-    if (st == SG_OK && pl->records) {
-        // in the unused half of E+'s column array (room for nnz = 2m entries) if it
-        // holds them (16 n <= 4 m: a mean degree of 8), in memory of their own otherwise
-        const uintptr_t b = ((uintptr_t)(o.col + o.m) + 15) & ~(uintptr_t)15, e = (uintptr_t)(o.col + 2 * o.m);
-        if (o.m > 0 && b + sizeof(uint4) * (size_t)o.n <= e) {
-            pl->arec = reinterpret_cast<uint4 *>(b);
-        } else if (dalloc(c, &pl->rec_own, sizeof(uint4) * (size_t)std::max<int64_t>(o.n, 1)) == SG_OK) {
-            pl->arec = static_cast<uint4 *>(pl->rec_own);
-        } else {
-            set_error("");
-        }
-    }
     if (st != SG_OK) return st;
     pl->inl = o.inl;  // the orientation's reverse list (not owned by the plan)
-    SG_CUDA(cudaMemsetAsync(pl->buckets, 0, sizeof(unsigned long long) * 2 * kKeys, c->stream));
+    SG_CUDA(cudaMemsetAsync(pl->buckets, 0, sizeof(unsigned long long) * 3 * kKeys, c->stream));
     SG_CUDA(cudaMemsetAsync(c->d_ctr + kCtrMaxDeg, 0, sizeof(unsigned long long), c->stream));
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((o.n + 255) / 256, (int64_t)c->num_sms * 8));
     if (o.n > 0) {
         SG_LAUNCH(c, "tri_classify");
-        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, offs, pl->din,
-                                                                       reinterpret_cast<uint2 *>(pl->arec), 2, o.n, pl->light_max,
+        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, offs, pl->din, o.n, pl->light_max,
                                                                        pl->light_items, (int64_t)kHeavyCap,
-                                                                       pl->buckets, c->d_ctr);
+                                                                       pl->buckets, u ? pl->buckets + kKeys : nullptr,
+                                                                       c->d_ctr);
     }
     SG_CUDA(cudaGetLastError());
-    SG_CUDA(cudaMemcpyAsync(c->h_pinned, pl->buckets, sizeof(unsigned long long) * kKeys, cudaMemcpyDeviceToHost,
+    SG_CUDA(cudaMemcpyAsync(c->h_pinned, pl->buckets, sizeof(unsigned long long) * 2 * kKeys, cudaMemcpyDeviceToHost,
                             c->stream));
-    SG_CUDA(cudaMemcpyAsync(c->h_pinned + kKeys, c->d_ctr + kCtrMaxDeg, sizeof(unsigned long long),
+    SG_CUDA(cudaMemcpyAsync(c->h_pinned + 2 * kKeys, c->d_ctr + kCtrMaxDeg, sizeof(unsigned long long),
                             cudaMemcpyDeviceToHost, c->stream));
-    SG_CUDA(cudaMemcpyAsync(c->h_pinned + kKeys + 1, c->d_ctr + kCtrWork, sizeof(unsigned long long),
+    SG_CUDA(cudaMemcpyAsync(c->h_pinned + 2 * kKeys + 1, c->d_ctr + kCtrWork, sizeof(unsigned long long),
                             cudaMemcpyDeviceToHost, c->stream));
     SG_CUDA(cudaStreamSynchronize(c->stream));
-    unsigned long long cnt[kKeys + 2];
+    unsigned long long cnt[2 * kKeys + 2];
     std::memcpy(cnt, c->h_pinned, sizeof(cnt));
-    pl->work = (int64_t)cnt[kKeys + 1];
+    pl->max_deg = (int64_t)cnt[2 * kKeys];
+    pl->work = (int64_t)cnt[2 * kKeys + 1];
+    pl->two = u && u->h && two_passes_pay(o, pl->max_deg, pl->work, *u) && two_passes_fit(c, o, *u, pl);
+    if (pl->two) {
+        pl->light_max = kUnionLightMax;
+        pl->light_items = kUnionLightItems;
+    }
+    const int split = pl->two ? kKeys : 0;
     pl->n_heavy = 0;
     pl->n_hubs = 0;
-    for (int b = 0; b < kKeys; ++b) pl->n_heavy += (int64_t)cnt[b];
-    for (int b = kBuckets; b < kKeys; ++b) pl->n_hubs += (int64_t)cnt[b];
-    pl->max_deg = (int64_t)cnt[kKeys];
+    for (int b = 0; b < kKeys; ++b) pl->n_heavy += (int64_t)cnt[split + b];
+    for (int b = kBuckets; b < kKeys; ++b) pl->n_hubs += (int64_t)cnt[split + b];
     // a hub launch with fewer hubs than SMs would leave most SMs idle: the
     // main launch then takes them first (they lead the list), in chunks
     if (pl->n_hubs < c->num_sms) pl->n_hubs = 0;
@@ -2010,8 +2071,8 @@ static sg_status make_plan(Ctx *c, const Oriented &o, const int64_t *offs, Plan 
         SG_LAUNCH(c, "tri_classify");
         classify_scatter_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, pl->din, o.n, pl->light_max,
                                                                          pl->light_items, (int64_t)kHeavyCap,
-                                                                         pl->buckets, pl->buckets + kKeys,
-                                                                         pl->heavy, nullptr);
+                                                                         pl->buckets + split, pl->buckets + 2 * kKeys,
+                                                                         pl->heavy, pl->arec, nullptr);
     }
     SG_CUDA(cudaGetLastError());
     // shared memory: hit queues + the larger of the heavy table (4 slots per
@@ -2085,8 +2146,7 @@ static sg_status launch_pass(Ctx *c, void (*hub)(TriArgs), void (*main)(TriArgs)
     a.light_items = pl.light_items;
     a.offs = pl.offs;
     a.din = pl.din;
-    a.vrec = reinterpret_cast<const uint2 *>(pl.arec);
-    a.vstep = 2;
+    a.arec = pl.arec;
     a.inl = pl.inl;
     a.work = c->d_ctr + kCtrAux;
     if (pl.n_hubs > 0) {
@@ -2107,36 +2167,23 @@ static sg_status launch_enum(Ctx *c, const TriArgs &a, const Plan &pl) {
                        "tri_enum");
 }
 
-// The two passes of a union kernel (see tri_union_kernel), h the output graph.
-// Without it or the second pass's scratch the first streams every list whole;
-// without the records too, in the one instance that does without them (long
-// tables in chunks: memory is short here, not time).
+// The one pass of a union kernel, or its two (see tri_union_kernel).
 template <Mode M>
-static sg_status launch_union(Ctx *c, const Oriented &o, TriArgs a, const Plan &pl, const Graph *h) {
-    if (pl.arec == nullptr) {
-        Plan main = pl;
-        main.n_hubs = 0;
-        a.short_max = INT_MAX;
-        return launch_pass(c, nullptr, tri_union_kernel<M, kTW, false, false>, 0, pl.usmem, a, main, "", "tri_enum");
-    }
-    AliveArcs al;
-    bool two = h != nullptr && pl.max_deg > kShortList;
-    if (two && alive_alloc(c, o, h, &al) != SG_OK) {
-        set_error("");
-        alive_free(c, &al);  // what it got of it
-        two = false;
-    }
-    a.short_max = !two ? INT_MAX : (pl.n_hubs > 0 ? kShortListHubs : kShortList);
+static sg_status launch_union(Ctx *c, const Oriented &o, TriArgs a, const Plan &pl) {
+    // where nearly every triangle deletes an edge, the atomics to edges deleted long
+    // ago queue up (cliques of 200 at p = 1: random 23.0 against 18.1 ms, max-weight
+    // 25.6 against 19.7); elsewhere looking costs more (geometric graph, 2^20
+    // vertices, p = 0.5: 4.84 against 5.13)
+    a.look_first = a.tp > 3ull << 30;
+    if (!pl.two) return launch_enum<M>(c, a, pl);
+    a.short_max = pl.n_hubs > 0 ? kShortListHubs : kShortList;
     sg_status st = launch_pass(c, tri_union_kernel<M, kHubTW, false>, tri_union_kernel<M, kTW, false>, pl.uhub_smem,
                                pl.usmem, a, pl, "tri_hubs", "tri_enum");
-    if (two && st == SG_OK) st = alive_build(c, o, a.del, al, pl.arec);
-    if (two && st == SG_OK) {
-        a.arec = pl.arec;
-        a.alive = al.list;
+    if (st == SG_OK) st = alive_build(c, o, a.del, pl.al, pl.arec);
+    a.alive = pl.al.list;
+    if (st == SG_OK)
         st = launch_pass(c, tri_union_kernel<M, kHubTW, true>, tri_union_kernel<M, kTW, true>, pl.uhub_smem, pl.usmem, a,
                          pl, "tri_rest_hubs", "tri_rest");
-    }
-    if (two) alive_free(c, &al);
     return st;
 }
 
@@ -2589,21 +2636,14 @@ static sg_status eo_rounds(Ctx *c, const Graph *g, const Oriented &o, sg_kernel 
 sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double p, uint64_t seed, uint32_t *del,
                   const Graph *h) {
     Plan pl;
-    const bool eo = k == SG_TR_EO || k == SG_TR_EO_MAXW || k == SG_TR_EO_MINCOUNT;
-    if (k == SG_TR_MINCOUNT || eo) {  // the counting and edge-once passes' split
-        pl.light_max = kLightMax;
-        pl.light_items = kLightItems;
-    } else {
-        pl.light_max = kUnionLightMax;
-        pl.light_items = kUnionLightItems;
-        pl.records = h != nullptr;
-    }
-    sg_status st = make_plan(c, o, g->off, &pl);
     TriArgs a = base_args(c, o);
     a.k0 = (uint32_t)(seed & 0xFFFFFFFFu);
     a.k1 = (uint32_t)(seed >> 32);
     a.tp = prob_threshold(p);
     a.del = del;
+    const UnionCall u{k, a.tp, h};
+    const bool choose = k == SG_TR_RANDOM || k == SG_TR_MAXW || k == SG_TR_P2;
+    sg_status st = make_plan(c, o, g->off, &pl, choose ? &u : nullptr);
     uint32_t *tcnt = nullptr;
     if (st == SG_OK && (k == SG_TR_MINCOUNT || k == SG_TR_EO_MINCOUNT)) {
         // the min-count choice needs the triangle count of every edge of G first
@@ -2613,21 +2653,18 @@ sg_status tr_mark(Ctx *c, const Graph *g, const Oriented &o, sg_kernel k, double
             st = cuda_fail(cudaGetLastError(), "cudaMemsetAsync(tcnt)");
         a.tcnt = tcnt;
         if (st == SG_OK) st = launch_enum<Mode::EdgeCount>(c, a, pl);
-        if (st == SG_OK && !eo) {  // the union passes split the vertices their own way
+        if (st == SG_OK && k == SG_TR_MINCOUNT && h && two_passes_pay(o, pl.max_deg, pl.work, u)) {
             free_plan(c, &pl);
             pl = Plan{};
-            pl.light_max = kUnionLightMax;
-            pl.light_items = kUnionLightItems;
-            pl.records = h != nullptr;
-            st = make_plan(c, o, g->off, &pl);
+            st = make_plan(c, o, g->off, &pl, &u);
         }
     }
     if (st == SG_OK) {
         switch (k) {
-        case SG_TR_RANDOM: st = launch_union<Mode::UnionRandom>(c, o, a, pl, h); break;
-        case SG_TR_MAXW: st = launch_union<Mode::UnionMaxw>(c, o, a, pl, h); break;
-        case SG_TR_P2: st = launch_union<Mode::UnionP2>(c, o, a, pl, h); break;
-        case SG_TR_MINCOUNT: st = launch_union<Mode::UnionMinCount>(c, o, a, pl, h); break;
+        case SG_TR_RANDOM: st = launch_union<Mode::UnionRandom>(c, o, a, pl); break;
+        case SG_TR_MAXW: st = launch_union<Mode::UnionMaxw>(c, o, a, pl); break;
+        case SG_TR_P2: st = launch_union<Mode::UnionP2>(c, o, a, pl); break;
+        case SG_TR_MINCOUNT: st = launch_union<Mode::UnionMinCount>(c, o, a, pl); break;
         default: st = eo_rounds(c, g, o, k, pl, a); break;
         }
     }
@@ -2675,7 +2712,7 @@ sg_status batch_tr_prepare(Ctx *c, const Graph *u, const Oriented &o, BatchTri *
     pl.light_items = 4 * bt->light_max;
     sg_status st = make_plan(c, o, u->off, &pl);
     if (st == SG_OK) {
-        bt->smem = pl.usmem;
+        bt->smem = pl.smem;
         bt->max_deg = pl.heavy_cap;
     }
     free_plan(c, &pl);
@@ -2683,7 +2720,6 @@ sg_status batch_tr_prepare(Ctx *c, const Graph *u, const Oriented &o, BatchTri *
     if (!bt->heavy) st = dalloc(c, (void **)&bt->heavy, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
     if (st == SG_OK && !bt->buckets)
         st = dalloc(c, (void **)&bt->buckets, sizeof(unsigned long long) * (2 * kKeys + 1));
-    if (st == SG_OK && !bt->vrec) st = dalloc(c, (void **)&bt->vrec, sizeof(uint2) * (size_t)std::max<int64_t>(o.n, 1));
     if (st == SG_OK && !bt->din) st = dalloc(c, (void **)&bt->din, sizeof(uint32_t) * (size_t)std::max<int64_t>(o.n, 1));
     // Per call only the graphs with a triangle kernel are oriented, so E+ can
     // hold fewer than nnz/2 arcs and the in-list room off(v) - off+(v) then
@@ -2697,8 +2733,6 @@ void batch_tr_free(Ctx *c, BatchTri *bt) {
     dfree(c, bt->heavy);
     dfree(c, bt->buckets);
     dfree(c, bt->din);
-    dfree(c, bt->vrec);
-    bt->vrec = nullptr;
     dfree(c, bt->inl);
     bt->heavy = nullptr;
     bt->buckets = nullptr;
@@ -2718,14 +2752,15 @@ sg_status batch_tr_mark(Ctx *c, const Graph *u, const Oriented &o, const BatchDe
     {
         SG_LAUNCH(c, "tri_classify");
         // no hub launch in a batch: its graphs are small, and a long N+(u) is chunked
-        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, u->off, bt.din, bt.vrec, 1, o.n, bt.light_max,
-                                                                       light_items, INT64_MAX, bt.buckets, c->d_ctr);
+        classify_count_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, u->off, bt.din, o.n, bt.light_max,
+                                                                       light_items, INT64_MAX, bt.buckets, nullptr,
+                                                                       c->d_ctr);
     }
     {
         SG_LAUNCH(c, "tri_classify");
         classify_scatter_kernel<<<(unsigned)blocks, 256, 0, c->stream>>>(o.off, bt.din, o.n, bt.light_max,
                                                                          light_items, INT64_MAX, bt.buckets,
-                                                                         bt.buckets + kKeys, bt.heavy,
+                                                                         bt.buckets + kKeys, bt.heavy, nullptr,
                                                                          bt.buckets + 2 * kKeys);
     }
     SG_CUDA(cudaGetLastError());
@@ -2735,18 +2770,15 @@ sg_status batch_tr_mark(Ctx *c, const Graph *u, const Oriented &o, const BatchDe
     a.n_heavy = 0;
     a.n_heavy_dev = bt.buckets + 2 * kKeys;
     a.heavy_cap = bt.max_deg;
-    a.short_max = INT_MAX;  // one pass
     a.light_max = bt.light_max;
     a.light_items = light_items;
     a.offs = u->off;
     a.din = bt.din;
-    a.vrec = bt.vrec;
-    a.vstep = 1;
     a.inl = bt.inl;
     a.work = c->d_ctr + kCtrAux;
     a.bparams = b.params;
     a.vgid = b.vgid;
-    return launch_tri(c, tri_union_kernel<Mode::BatchUnion, kTW, false>, kTW * 32, bt.smem, a, "tri_enum", bt.grid_per_sm);
+    return launch_tri(c, tri_enum_kernel<Mode::BatchUnion, kTW>, kTW * 32, bt.smem, a, "tri_enum", bt.grid_per_sm);
 }
 
 }  // namespace sg

@@ -250,21 +250,23 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
             if (__shfl_sync(kFull, (int)last, 0)) {
                 __syncwarp();  // a shuffle orders no memory: the lanes' reads below come after lane 0's fence
                 const float *part = a.hubs.part + (size_t)first * (split ? kPrWarps : 1);
-                float s = 0.f, one = 0.f;  // the row's sum, a chunk's
-                for (int p0 = 0; p0 < parts; p0 += 32) {
-                    const float x = p0 + lane < parts ? __ldcg(part + p0 + lane) : 0.f;
-                    for (int j = 0; j < min(32, parts - p0); ++j) {
-                        const float y = __shfl_sync(kFull, x, j);
+                const int nch = split ? parts / kPrWarps : parts;
+                float s = 0.f;
+                for (int c0 = 0; c0 < nch; c0 += 32) {  // a lane adds a chunk's runs
+                    float one = 0.f;
+                    if (c0 + lane < nch) {
                         if (split) {
-                            one += y;
-                            if ((j & (kPrWarps - 1)) == kPrWarps - 1) {
-                                s += one;
-                                one = 0.f;
-                            }
+                            const float4 *run = reinterpret_cast<const float4 *>(part + (size_t)(c0 + lane) * kPrWarps);
+                            static_assert(kPrWarps == 8, "two loads are a chunk's runs");
+                            const float4 x = __ldcg(run), y = __ldcg(run + 1);
+                            one = ((((((x.x + x.y) + x.z) + x.w) + y.x) + y.y) + y.z) + y.w;
                         } else {
-                            s += y;
+                            one = __ldcg(part + c0 + lane);
                         }
                     }
+                    // (one after another, but the shuffles do not wait for the sums; 0 past the last)
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) s += __shfl_sync(kFull, one, j);
                 }
                 if (lane == 0) {
                     a.hubs.done[h] = 0;
@@ -738,7 +740,10 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     }
     const int64_t groups = (n + 31) / 32;
     const int grid = (int)std::min<int64_t>(std::max<int64_t>(groups, nnz / kHubChunk), (int64_t)c->num_sms);
-    a.per_claim = (int)std::max<int64_t>(1, std::min<int64_t>(4, groups / ((int64_t)grid * 32 * 8)));
+    // groups of a claim, which hide each other's first loads: up to four, where that
+    // leaves each warp four claims (a star of 2 M leaves, two groups of a claim
+    // against one: 50 iterations 2.09 / 2.91 ms)
+    a.per_claim = (int)std::max<int64_t>(1, std::min<int64_t>(4, groups / ((int64_t)grid * 32 * 4)));
     const size_t smem = hot ? sizeof(float) * (((size_t)hot_cap + 3) / 4 * 4) : 0;
     void (*k[2][3])(PrArgs) = {{pr_iter_kernel<false, PrStore::kNone>, pr_iter_kernel<false, PrStore::kPrev>,
                                 pr_iter_kernel<false, PrStore::kLast>},

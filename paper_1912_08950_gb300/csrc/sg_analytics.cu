@@ -40,7 +40,7 @@ constexpr int kPrWarps = kPrThreads / 32;
 // it (evict-first).  One CTA of 32 warps per SM, eight slabs of 32 arcs in
 // flight per warp.  Per iteration on R-MAT s22 (128 M arcs) 339 us, against 634
 // with y in vertex order and launches of their own for hub rows and D; s20: 88
-// against 172; n = 60,000: 20 against 47.  Half of the L1 for y is where the line lies: 373 us at 32 K
+// against 172; n = 100,000: 26 against 41.  Half of the L1 for y is where the line lies: 373 us at 32 K
 // entries before the heads were streamed, 403 at 16 K, 387 at 24 K and 389 at
 // 40 K; 54 K entries (all of the shared memory) leave too few lines: 588.
 //
@@ -639,6 +639,11 @@ __global__ void __launch_bounds__(kPrThreads) reduce_parts_kernel(const T *__res
 // Iterations that pay for the positions and the translated heads: they take
 // 0.66 ms on R-MAT s22 and save about 0.2 ms an iteration.
 constexpr int kPrMinIters = 4;
+// Vertices above which they pay: below, most of y stays in the L1 without them,
+// which the copy in shared memory takes space from (50 iterations in us, with /
+// without: complete graph of 4000 1664 / 1333, R-MAT with n = 8000 687 / 639,
+// 30,000 1081 / 1013, 60,000 951 / 917, 100,000 1322 / 1323; 2^20 4570 / 6351).
+constexpr int64_t kPrMinVertices = 3 * (int64_t)kPrHot;
 
 sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_out, double *resid) {
     const int64_t n = g->n, nnz = g->nnz;
@@ -685,7 +690,7 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     sg_status st = dalloc(c, (void **)&buf, total);
     if (st != SG_OK) return st;
     // positions and translated heads: 4 (n + nnz) bytes, without which y stays in vertex order
-    bool hot = iters >= kPrMinIters && nnz > 0;
+    bool hot = iters >= kPrMinIters && nnz > 0 && n > kPrMinVertices;
     if (hot && (dalloc(c, (void **)&pos, sizeof(uint32_t) * nn) != SG_OK ||
                 dalloc(c, (void **)&colx, sizeof(uint32_t) * (size_t)nnz) != SG_OK)) {
         set_error("");

@@ -253,7 +253,7 @@ def streaming_rows(kt, steps, n, m, A_out, hbm):
 
 
 KERNEL_NAMES = ("tri_enum", "tri_hubs", "tri_rest", "tri_alive", "tri_reverse_list", "tri_eo_fresh_reserve", "tri_eo_list_reserve",
-                "tri_eo_list_accept", "tri_eo_accept", "tri_eo_list_reset", "tri_classify", "compact_orient",
+                "tri_eo_list_accept", "tri_eo_accept", "tri_eo_list_reset", "tri_eo_rounds", "tri_classify", "compact_orient",
                 "compact_trmask", "row_maps")
 
 

@@ -118,8 +118,11 @@ typedef struct sg_div_result {
 typedef struct sg_stats {
     uint64_t kernel_launches; /* kernels this library launched on the context */
     uint64_t probes;          /* list elements streamed through tables by triangle kernels */
-    uint64_t triangles;       /* triangles found by triangle kernels (by union kernels: those
-                                 decided, since one whose edges are all deleted needs no decision) */
+    uint64_t triangles;       /* triangles found by triangle kernels.  A union kernel that works in
+                                 two passes leaves out elements and triangles of edges that it sees
+                                 deleted already, so both counts are then what it did not leave out,
+                                 and vary from call to call by when a deletion is seen (the output
+                                 does not) */
     uint64_t eo_rounds;       /* Edge-Once reservation rounds run */
     uint64_t eo_listed;       /* triangles written to Edge-Once lists (16 bytes each) */
     uint64_t eo_passes;       /* Edge-Once enumeration passes (each bids for its round) */
@@ -152,7 +155,8 @@ sg_status sg_ctx_reset_profile(sg_ctx *ctx);
  * the earliest groups that do (a window of the schedule); once every triangle
  * in the window is decided, one more enumeration lists the live ones above
  * it.  records > 0 caps the list at that many triangles, 0 (default) sizes it
- * at a quarter of free device memory, -1 disables it (every round then
+ * at a quarter of free device memory (on small graphs at 256 MB, unless the
+ * call then runs out of memory), -1 disables it (every round then
  * enumerates the triangles again).  The result is the same in every setting;
  * only time and memory change. */
 sg_status sg_ctx_set_eo_list_capacity(sg_ctx *ctx, int64_t records);

@@ -25,8 +25,8 @@
 // (r0 < floor(p 2^32)) and picks the edge to delete (r1, the heaviest edge, or
 // the edge in the fewest triangles of G, counted by an earlier EdgeCount pass);
 // the p-2 kernel deletes the two edges r1 does not pick.  Union kernels set the
-// arc's deletion flag (a bit, idempotent) and stop looking for triangles whose
-// edges are all deleted (tri_union_kernel).  The
+// arc's deletion flag (a bit, idempotent); where it pays they do so in two passes
+// that leave out triangles whose edges are all deleted (tri_union_kernel).  The
 // Edge-Once kernel instead reserves each edge of every live selected triangle
 // with a 64-bit atomicMin of (r2 << 32 | third vertex); an edge pass then
 // accepts every triangle that holds all three of its reservations.  Accepted
@@ -51,11 +51,12 @@ constexpr int kHeavyCap = 1024;  // largest phase-1 table (entries; 26 KB of sha
 constexpr int kHubTW = 32;        // warps per CTA of the hub launch (one CTA per SM)
 constexpr int kHubCap = 4096;     // largest hub table (entries; 104 KB of shared memory)
 constexpr int kQ = 128;           // per-warp hit ring (<= 31 left over + 2 slabs of hits fit)
-constexpr int kWindow = 32;       // list elements a union pass streams before it looks at an arc again
+// the two union passes (tri_union_kernel):
+constexpr int kWindow = 32;       // list elements streamed before an arc is looked at again
 constexpr int kWhole = 1 << 29;        // blocks of the window of a list streamed whole
 constexpr int kFilterLog = 4;          // log2 of the filter bits per table slot (four slots per entry)
 constexpr int kFilterBits = 4 << kFilterLog;  // per entry
-constexpr int kUnionLightMax = 128;    // union passes: largest out-degree processed by one warp
+constexpr int kUnionLightMax = 128;    // largest out-degree processed by one warp
 constexpr int kUnionLightItems = 512;  // ... with at most this many lists to stream
 // lists up to this long are always streamed whole (see tri_union_kernel): 256 on
 // graphs with a hub launch, where the second pass costs more (R-MAT s26 at p =
@@ -342,6 +343,7 @@ template <Mode M>
 __device__ __forceinline__ void decide(const TriArgs &a, bool valid, uint32_t u, uint32_t v, uint32_t w,
                                        uint32_t iuv, uint32_t iuw, uint32_t ivw, unsigned &live, Emitter &em,
                                        uint32_t head_uv = 0) {
+    static_assert(kDecides<M>, "the counting passes decide nothing");
     if constexpr (kUnion<M>) {
         if (valid)
             decide_union<M>(a, u, v, w, iuv, iuw, ivw, [&](uint32_t e) {
@@ -452,7 +454,7 @@ struct Table {
     uint32_t *slot;
     unsigned long long *stash;
     int *stash_n;
-    uint32_t *dead = nullptr;    // union passes: deletion flags of the table's arcs, by position,
+    uint32_t *dead = nullptr;    // two union passes: deletion flags of the table's arcs, by position,
     uint32_t *filter = nullptr;  // and one bit per hash of kFilterBits per entry
 };
 
@@ -566,7 +568,8 @@ __device__ __forceinline__ void probe_list(const TriArgs &a, const Table &tb, in
             if (lane == 0) tris += (unsigned)(__popc(ma) + __popc(mb));
             continue;
         }
-        if (ma | mb) {
+        if constexpr (kDecides<M>) {
+            if ((ma | mb) == 0) continue;
             const int pa = __popc(ma), pb = __popc(mb);
             const int tail = qs.head + qs.n;
             if (ha) {
@@ -643,12 +646,15 @@ __device__ __forceinline__ void stream_in_group(const TriArgs &a, const Table &t
 // 64 elements), so they are streamed as one sequence, a slab of 32 elements at a
 // time: a lane finds its element's arc from the arcs that start inside the
 // slab.  Counting: the first lane of an arc's run adds the run's hits to the
-// arc's counters; otherwise the hits go to the queue.  A list at a time, 64 lanes wide, left most lanes idle and waited for
-// one list's loads after another: triangles per vertex of a geometric graph
-// (2^20 vertices, 25 M edges, lists of 17 elements) took 5.18 ms, now 2.15; of
-// R-MAT s20, where most elements are in heavy vertices' lists, 9.33 and 8.98.
-// The edge-once listing pass at p = 0.5: 7.90 and 4.22 on the geometric graph,
-// 5.88 and 4.99 on a Chung-Lu graph of 2^20 vertices, 23.1 and 22.3 on R-MAT s21.
+// arc's counters; otherwise the hits go to the queue.
+//
+// Bound by latency and idle lanes when a list is streamed at a time, 64 lanes
+// wide, each waiting for the loads of the one before; against that, in ms:
+// triangles per vertex of a geometric graph (2^20 vertices, 25 M edges, lists of
+// 17 elements) 5.18 -> 2.15, of R-MAT s20, where most elements are in heavy
+// vertices' lists, 9.33 -> 8.98; the edge-once listing pass at p = 0.5 on the
+// geometric graph 7.90 -> 4.22, Chung-Lu 2^20 5.88 -> 4.99, R-MAT s21 23.1 ->
+// 22.3; a union call at p = 0.5 on the geometric graph 7.74 -> 4.84.
 // Returns the hits (all lanes).  arc: 32 entries of the warp's scratch.
 template <Mode M>
 __device__ __forceinline__ unsigned light_group(const TriArgs &a, const Table &tb, int sh, int stash_n, uint32_t u,

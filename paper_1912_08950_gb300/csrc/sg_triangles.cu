@@ -1981,27 +1981,30 @@ struct UnionCall {
 // Whether two union passes (tri_union_kernel) pay.  They drop what is streamed and
 // decided for deleted edges, at the price of a pass over the vertices and arcs
 // between them and of more instructions per element (the filter, the windows).
-// So the lists have to be long, as those of up to kShortList are streamed whole
-// whatever happens: W / m elements per arc on average, and a longest one of twice
-// that; W has to outweigh the pass over the vertices; and deletions have to come
-// while the lists stream: p W / m bounds the selected triangles per edge
-// (about a sixth of the elements close one on R-MAT graphs, all of them in
-// cliques, which the rule cannot tell).  Where a triangle deletes two edges
-// (p-2) half of that does; where it always deletes its heaviest, light edges
-// live on and it takes more.  Calls in ms, one pass / two passes:
-//   random        p W / m  1.2: R-MAT s20  8.49 / 10.3   3.8: R-MAT s20  8.57 / 9.10
-//                          5.5: R-MAT s22  45.1 / 45.5   6.0: Chung-Lu 2^21 11.4 / 9.99
-//                           12: R-MAT s20  8.67 / 7.10
-//   max-weight              12: R-MAT s20  9.38 / 9.84    18: Chung-Lu 2^21 12.2 / 11.1
-//                           37: R-MAT s20  9.49 / 8.43
-//   random p = 0.5  W / m  46: n = 200,000, ef 8  0.64 / 1.07   47: n = 2^20, ef 5  1.84 / 1.98
-//                          60: Chung-Lu 2^21      11.4 / 8.69   83: n = 30,000, ef 40  0.65 / 0.57
-//                          66, longest 199: cliques of 200  18.1 / 21.6
+// So there have to be lists well above kShortList, as shorter ones are streamed
+// whole whatever happens; the W elements of one pass have to outweigh the pass
+// over the vertices; and edges have to be deleted while their lists stream: s = p W / m
+// bounds the selected triangles per edge (about a sixth of the elements close
+// one on R-MAT graphs, all of them in cliques, which the rule cannot tell).
+// What can be dropped grows with s and W, what the second pass costs does not:
+// s W is the rest of the rule.  Where a triangle deletes two edges (p-2), s
+// counts double; where it always deletes its heaviest (max-weight), light edges
+// live on and both lines lie higher.  Calls in ms, one pass / two passes:
+//   random      s, s W
+//     R-MAT s20            1.3, 2.5e9  8.49 / 10.3    R-MAT s20            13, 2.5e10  8.67 / 7.06
+//     R-MAT s22            5.5, 6.6e10 45.1 / 45.5    Chung-Lu 2^21       6.0, 1.2e10  11.3 / 9.89
+//     n = 100,000, ef 16   6.3, 5.4e8  0.74 / 0.93    n = 30,000, ef 40    17, 1.2e9   0.66 / 0.60
+//     n = 400,000, ef 8    5.6, 9.5e8  1.29 / 1.53    n = 60,000, ef 24    36, 3.1e9   0.71 / 0.67
+//     n = 200,000, ef 16   7.9, 1.8e9  1.36 / 1.51    n = 200,000, ef 24   11, 4.7e9   2.40 / 2.03
+//   max-weight
+//     R-MAT s20             13, 2.5e10 9.38 / 9.84    Chung-Lu 2^21        18, 3.6e10  12.1 / 11.0
+//     n = 30,000, ef 40     83, 6.2e9  0.68 / 0.70    n = 200,000, ef 24   32, 1.4e10  2.52 / 2.39
+//   longest list 199 to 234 (s from 9): cliques of 200 18.1 / 21.6, n = 200,000, ef 8  0.65 / 1.10
 static bool two_passes_pay(const Oriented &o, int64_t max_deg, int64_t work, const UnionCall &u) {
-    const double w = (double)work, m = (double)o.m;
-    if (o.m == 0 || max_deg <= 2 * kShortList || w < 0.4 * kShortList * m || w < 32.0 * (double)o.n) return false;
-    const double selected = (double)u.tp / 4294967296.0 * w / m;
-    return selected >= (u.kernel == SG_TR_P2 ? 2.5 : u.kernel == SG_TR_MAXW ? 15.0 : 5.0);
+    const double w = (double)work;
+    if (o.m == 0 || max_deg <= 2 * kShortList || w < 32.0 * (double)o.n) return false;
+    const double s = (double)u.tp / 4294967296.0 * w / (double)o.m * (u.kernel == SG_TR_P2 ? 2.0 : 1.0);
+    return u.kernel == SG_TR_MAXW ? s >= 15.0 && s * w >= 1e10 : s >= 4.0 && s * w >= 1.2e9;
 }
 
 // What two passes need beside the plan; false (and nothing kept) where it does not fit.

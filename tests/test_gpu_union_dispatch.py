@@ -38,38 +38,34 @@ def _isolated(g, n):
     return gg.CSR(n, torch.cat([g.off, g.off[-1:].expand(n - g.n)]).contiguous(), g.col, g.w)
 
 
-# a clique of n: lists of up to n - 1, (n - 2) / 3 elements per arc
-@pytest.mark.parametrize("n,kern,p,passes", [
-    (257, "tr_random", 0.5, 1), (258, "tr_random", 0.5, 2),          # longest list 256, 257
-    (300, "tr_random", 0.0503, 1), (300, "tr_random", 0.0504, 2),    # p W / m 4.998, 5.006
-    (300, "tr_mincount", 0.0503, 1), (300, "tr_mincount", 0.0504, 2),
-    (300, "tr_p2", 0.0251, 1), (300, "tr_p2", 0.0252, 2),            # 2.49, 2.504
-    (300, "tr_maxw", 0.1510, 1), (300, "tr_maxw", 0.1511, 2),        # 14.999, 15.009
-    (300, "tr_random", 1.0, 2), (300, "tr_maxw", 1.0, 2), (300, "tr_random", 0.0, 1),
-    (200, "tr_random", 0.75, 1), (200, "tr_random", 0.76, 1), (200, "tr_maxw", 1.0, 1), (200, "tr_p2", 1.0, 1),
+def _copies(c, n):
+    """c cliques of n."""
+    a, b = (torch.from_numpy(x.astype(np.int64)) for x in np.triu_indices(n, 1))
+    base = (torch.arange(c) * n)[:, None]
+    return gg.csr_from_edges(c * n, (base + a).reshape(-1), (base + b).reshape(-1))
+
+
+# c cliques of n: lists of up to n - 1, W = c n (n - 1) (n - 2) / 6 elements, (n - 2) / 3 per arc
+@pytest.mark.parametrize("c,n,kern,p,passes", [
+    (24, 257, "tr_random", 0.5, 1), (24, 258, "tr_random", 0.5, 2),         # longest list 256, 257
+    (10, 300, "tr_random", 0.2710, 1), (10, 300, "tr_random", 0.2713, 2),   # s W = 1.1993e9, 1.2006e9
+    (10, 300, "tr_mincount", 0.2710, 1), (10, 300, "tr_mincount", 0.2713, 2),
+    (10, 300, "tr_p2", 0.1355, 1), (10, 300, "tr_p2", 0.1357, 2),           # 1.1993e9, 1.2011e9
+    (30, 300, "tr_maxw", 0.752, 1), (30, 300, "tr_maxw", 0.754, 2),         # 9.98e9, 1.001e10
+    (1, 1300, "tr_random", 0.00923, 1), (1, 1300, "tr_random", 0.00925, 2),  # s = 3.994, 4.002; and a hub launch
+    (10, 300, "tr_random", 1.0, 2), (10, 300, "tr_random", 0.0, 1), (12, 289, "tr_p2", 1.0, 2),
+    (1, 200, "tr_random", 0.75, 1), (1, 200, "tr_random", 0.76, 1), (1, 200, "tr_maxw", 1.0, 1), (1, 200, "tr_p2", 1.0, 1),
+    (1, 1100, "tr_random", 0.05, 2), (1, 1200, "tr_mincount", 0.05, 2),     # tables in chunks; a hub launch
 ])
-def test_cliques(sg, n, kern, p, passes):
-    g = gg.complete(n)
+def test_cliques(sg, c, n, kern, p, passes):
+    g = _copies(c, n)
     assert _passes(sg, gg.attach_weights(g, seed=2) if kern == "tr_maxw" else g, kern, p) == passes
 
 
-# 44,850 arcs of a clique of 300, 4.455 M elements: below 51.2 elements per arc beside 43,200
-# arcs of cliques of 10, below 32 per vertex on 139,500 vertices
-@pytest.mark.parametrize("name,passes", [("with 900 cliques of 10", 2), ("with 1100 cliques of 10", 1),
-                                         ("in 139000", 2), ("in 139500", 1)])
-def test_dilution(sg, name, passes):
-    k = gg.complete(300)
-    if name.startswith("with"):
-        g = gg.disjoint_union(k, *([gg.complete(10)] * int(name.split()[1])))
-    else:
-        g = _isolated(k, int(name.split()[1]))
-    assert _passes(sg, g, "tr_random", 0.5) == passes
-
-
-# 175 vertices of out-degree above 1024: a hub launch in both passes; 75: chunked tables
-@pytest.mark.parametrize("n", [1100, 1200])
-def test_hubs(sg, n):
-    assert _passes(sg, gg.complete(n), "tr_random", 0.05) == 2
+# 44.55 M elements, 32 per vertex on 1,392,218 vertices
+@pytest.mark.parametrize("n,passes", [(1392000, 2), (1392500, 1)])
+def test_isolated_vertices(sg, n, passes):
+    assert _passes(sg, _isolated(_copies(10, 300), n), "tr_random", 0.5) == passes
 
 
 # out-degrees above the hub launch's table (4096 entries): tables in chunks in both passes.

@@ -431,14 +431,41 @@ __global__ void __launch_bounds__(kPrCta, 1) pr_iter_kernel(PrArgs a) {
 // bytes once per call: in the last iteration the rows a lane gets, and so the
 // order of the sum, depend on the schedule.  The sum is exact, and any order
 // gives the same, only while the terms' bits fit 53, which damping near 1 or
-// very many vertices exceed.)
+// very many vertices exceed.)  Bound by the FP64 units (R-MAT s22: 64 us with two
+// conversions and two additions a vertex, against 5 for the bytes), so differences
+// that are exact in FP32 are taken there and widened by their bits, which leaves
+// one addition, and none where the value did not change.
+__device__ __forceinline__ double widen(float f) {  // (double)f of a value that is not negative
+    const uint32_t b = __float_as_uint(f);
+    if (b - 0x00800000u < 0x7F000000u)  // a normal number: its exponent and fraction moved
+        return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+    return (double)f;
+}
+
 __global__ void __launch_bounds__(kPrThreads) pr_residual_kernel(const float *__restrict__ x,
                                                                 const float *__restrict__ x_prev, int64_t n,
                                                                 double *__restrict__ parts) {
+    constexpr int kPer = 4;
     __shared__ double s[kPrWarps];
+    const int64_t stride = (int64_t)gridDim.x * kPrThreads;
     double res = 0.0;
-    for (int64_t v = (int64_t)blockIdx.x * kPrThreads + threadIdx.x; v < n; v += (int64_t)gridDim.x * kPrThreads)
-        res += fabs((double)__ldg(x + v) - (double)__ldg(x_prev + v));
+    for (int64_t v = (int64_t)blockIdx.x * kPrThreads + threadIdx.x; v < n; v += stride * kPer) {
+        float a[kPer], b[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            a[j] = v + j * stride < n ? __ldg(x + v + j * stride) : 0.f;
+            b[j] = v + j * stride < n ? __ldg(x_prev + v + j * stride) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {  // (0 past the last vertex)
+            const float d = fabsf(a[j] - b[j]);
+            // within a factor of two the FP32 difference is exact (Sterbenz)
+            if (!(a[j] >= 0.5f * b[j] && a[j] <= 2.f * b[j]))
+                res += fabs((double)a[j] - (double)b[j]);
+            else if (d != 0.f)
+                res += widen(d);
+        }
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) res += __shfl_xor_sync(kFull, res, o);
     if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = res;
@@ -746,9 +773,11 @@ sg_status pagerank(Ctx *c, const Graph *g, float damping, int iters, float *x_ou
     const int64_t groups = (n + 31) / 32;
     const int grid = (int)std::min<int64_t>(std::max<int64_t>(groups, nnz / kHubChunk), (int64_t)c->num_sms);
     // groups of a claim, which hide each other's first loads: up to four, where that
-    // leaves each warp four claims (a star of 2 M leaves, two groups of a claim
-    // against one: 50 iterations 2.09 / 2.91 ms)
-    a.per_claim = (int)std::max<int64_t>(1, std::min<int64_t>(4, groups / ((int64_t)grid * 32 * 4)));
+    // leaves each warp eight claims, or four where the rows are so short that little
+    // else is in flight (50 iterations, two groups of a claim / one: a star of 2 M
+    // leaves 2.09 / 2.91 ms, a geometric graph of 1.8 M with 18 arcs a row 9.63 / 9.50)
+    const int64_t claims = nnz < 8 * n ? 4 : 8;
+    a.per_claim = (int)std::max<int64_t>(1, std::min<int64_t>(4, groups / ((int64_t)grid * 32 * claims)));
     const size_t smem = hot ? sizeof(float) * (((size_t)hot_cap + 3) / 4 * 4) : 0;
     void (*k[2][3])(PrArgs) = {{pr_iter_kernel<false, PrStore::kNone>, pr_iter_kernel<false, PrStore::kPrev>,
                                 pr_iter_kernel<false, PrStore::kLast>},

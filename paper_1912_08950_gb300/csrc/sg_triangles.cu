@@ -992,6 +992,7 @@ __global__ void __launch_bounds__(TW * 32, TW == kTW ? kEnumCtasPerSm<M> : 1) tr
 // triangle) and now: s22 0.35 and 0.14, 41.8 -> 19.2 ms; s26 0.32 and 0.09,
 // 1094 -> 525 ms.  Max-weight on a Chung-Lu graph of 2^21 vertices at p = 1,
 // where light edges never die: 0.69 and 0.35, 11.5 -> 8.3 ms.
+
 // The table vertex a warp works on.
 struct TabCtx {
     Table tb;

@@ -1998,14 +1998,15 @@ struct UnionCall {
 //     n = 400,000, ef 8    5.6, 9.5e8  1.29 / 1.53    n = 60,000, ef 24    36, 3.1e9   0.71 / 0.67
 //     n = 200,000, ef 16   7.9, 1.8e9  1.36 / 1.51    n = 200,000, ef 24   11, 4.7e9   2.40 / 2.03
 //   max-weight
-//     R-MAT s20             13, 2.5e10 9.38 / 9.84    Chung-Lu 2^21        18, 3.6e10  12.1 / 11.0
+//     R-MAT s20             13, 2.5e10 9.38 / 9.84    Chung-Lu 1.4 M       13, 2.4e10  10.9 / 10.4
+//     R-MAT s22             18, 2.2e11 49.6 / 50.6    Chung-Lu 2^21        18, 3.6e10  12.1 / 11.0
 //     n = 30,000, ef 40     83, 6.2e9  0.68 / 0.70    n = 200,000, ef 24   32, 1.4e10  2.52 / 2.39
 //   longest list 199 to 234 (s from 9): cliques of 200 18.1 / 21.6, n = 200,000, ef 8  0.65 / 1.10
 static bool two_passes_pay(const Oriented &o, int64_t max_deg, int64_t work, const UnionCall &u) {
     const double w = (double)work;
     if (o.m == 0 || max_deg <= 2 * kShortList || w < 32.0 * (double)o.n) return false;
     const double s = (double)u.tp / 4294967296.0 * w / (double)o.m * (u.kernel == SG_TR_P2 ? 2.0 : 1.0);
-    return u.kernel == SG_TR_MAXW ? s >= 15.0 && s * w >= 1e10 : s >= 4.0 && s * w >= 1.2e9;
+    return u.kernel == SG_TR_MAXW ? s >= 10.0 && s * w >= 1e10 : s >= 4.0 && s * w >= 1.2e9;
 }
 
 // What two passes need beside the plan; false (and nothing kept) where it does not fit.
